@@ -287,6 +287,7 @@ Params base_params(const Common& c, unsigned* status) {
   if (exp_w) p.recon = p.ste = 0;  // (neither a reconstruction nor a surrogate placement applies)
   p.x3 = c.prec == KINT_PREC_3XTF32;
   p.BH = c.B * c.H;
+  p.bh_magic = p.BH > 1 ? ~0ull / (unsigned)p.BH + 1ull : 0ull;
   p.nqb = (c.T + 127) / 128;
   p.tau = c.tau;
   p.scale = (float)(1.0 / std::sqrt((double)c.d));
@@ -345,42 +346,61 @@ int plan_probe(Params& p) {
   return total;
 }
 
-// mode: PV_MAIN / PV_MAIN_LERP / PV_LERP.  Picks the TMEM score double-buffering
-// and the deepest K/V ring that fit.
+// mode: PV_MAIN / PV_MAIN_LERP / PV_LERP.  Persistent CTAs loop over the items; picks the groups, the
+// TMEM layout, the depth of the K and V^T rings (64-key tiles) and where the outputs are
+// staged: beside the rings when two slots of each still fit, else over the V^T ring.
 int plan_main(Params& p, int mode) {
-  const int parts = p.x3 ? 2 : 1, tile = p.d * 512;
-  // (e_r, e_{r+1}) pairs: per row for MinMax ([K][128]), one shared [K] for FWMR; FWM's
-  // half-bin table of 16-byte entries, q in [-2, 2K]
-  const int table = p.calib == KINT_CALIB_MINMAX ? p.Kint * 1024
-                    : p.calib == KINT_CALIB_FWM  ? std::max(1024, round_up((2 * p.Kint + 3) * 16, 128))
+  const int parts = p.x3 ? 2 : 1, tile = p.d * 512, slot = parts * p.d * 64 * 4;
+  // per-row tables for MinMax ([K][128] pairs, or [2K + 1][128] endpoints), one shared [K] pair
+  // table for FWMR, FWM's half-bin table of 24-byte entries, q in [-2, 2K]
+  const int table = p.calib == KINT_CALIB_MINMAX ? p.Kint * 1024 + 512
+                    : p.calib == KINT_CALIB_FWM  ? round_up((2 * p.Kint + 3) * 24, 128)
                     : p.calib == KINT_CALIB_FWM_RESOLVED ? 1024 : 0;
-  const bool useA2 = mode == PV_MAIN_LERP || p.x3;
-  const int cols1 = 128 + (useA2 ? 128 : 0) + p.d + (mode == PV_MAIN_LERP ? p.d : 0);
-  const int ostage = (mode == PV_MAIN_LERP ? 2 : 1) * 128 * p.d * 4;  // O (and O_lerp) staging tiles
+  const bool both = mode == PV_MAIN_LERP, useA2 = both || p.x3;
   p.nitems = p.nqb * p.BH;
   p.sm_a = 0;
   p.sm_stage0 = parts * tile;
-  p.sm_stage_bytes = parts * 2 * tile;
-  // One CTA per SM looping over the items needs its own output staging area (the
-  // stage ring keeps loading the next item); at least two stages.  Otherwise one item
-  // per CTA, staging in the ring, which is idle by the epilogue.
-  for (int persist = 1; persist >= 0; --persist) {
-    for (p.nstage = 3; p.nstage >= (persist ? 2 : 1); --p.nstage) {
-      p.nbuf = (cols1 + 128 <= 512) ? 2 : 1;
-      p.sm_table = p.sm_stage0 + p.nstage * p.sm_stage_bytes;
-      p.sm_ostage = persist ? round_up(p.sm_table + table, 1024) : p.sm_stage0;
-      const int end = persist ? p.sm_ostage + ostage : p.sm_table + table;
-      const int total = std::max(finish_plan(p, end, 11 + 2 * p.nstage), kOneCtaPerSm);
-      if (total <= kSmemLimit) {
-        // Issuing S(kb+1) before P V(kb) needs tile kb+1 in a second stage while
-        // tile kb's V^T is still being read; with one stage the two would wait on
-        // each other, so a single stage means a single score buffer.
-        if (p.nstage == 1) p.nbuf = 1;
-        p.ngrid = persist ? std::min(p.nitems, num_sms()) : p.nitems;
-        return total;
-      }
+  p.sm_stage_bytes = slot;
+  auto layout = [&](int alias, int limit) -> int {
+    p.nstage_v = std::max(2, p.nstage);
+    p.ost_alias = alias;
+    p.ost_n = both && (!alias || p.nstage_v * slot >= 2 * tile) ? 2 : 1;
+    p.sm_v = p.sm_stage0 + p.nstage * slot;
+    p.sm_table = p.sm_v + p.nstage_v * slot;
+    p.sm_rows = p.sm_table + table;  // the row sums and the ring of chunk sums
+    const int rows_end = p.sm_rows + 2048 + 8192 * (both ? 2 : 1);
+    p.sm_ostage = alias ? p.sm_v : round_up(rows_end, 1024);
+    const int total = finish_plan(p, alias ? rows_end : p.sm_ostage + p.ost_n * tile, 29 + 2 * (p.nstage + p.nstage_v));
+    return total <= limit ? total : -1;
+  };
+  // Two CTAs per SM, 256 TMEM columns each (two score buffers, O, Q): TF32 at d = 64 without
+  // O_lerp, with more items than SMs (fewer leave each item an SM of its own, where one CTA's
+  // sixteen compute warps finish it sooner).  At B=8 H=12 T=1024 the softmax pass takes 35.6 us
+  // so, 40.9 with one CTA; FWM LERP at B=4 T=1000 31.6 against 34.8.  With O_lerp the columns
+  // leave one score buffer per CTA: 79 us against 66.8 with one CTA.
+  if (!p.x3 && p.d == 64 && !both && p.nitems > num_sms()) {
+    p.main_groups = 1;
+    p.q_tmem = 1;
+    p.nbuf = 2;
+    p.ngrid = std::min(p.nitems, 2 * num_sms());
+    for (p.nstage = 2; p.nstage >= 1; --p.nstage) {
+      const int total = layout(1, 113 * 1024);
+      if (total > 0) return total;
     }
   }
+  p.main_groups = 2;
+  // Q in TMEM beside the accumulators, the A2 buffers and at least two score buffers (all but
+  // d = 128 with O_lerp); then as many score buffers as fit, four at most.  S with Q in shared
+  // memory reads three times the operand bytes there: 144.7 us against 134.5 at B=4 H=16 T=2048 d=128.
+  const int cols = (useA2 ? 128 : 0) + p.d * (both ? 2 : 1);
+  p.q_tmem = cols + parts * p.d + 128 <= 512;
+  p.nbuf = std::min(4, (512 - cols - (p.q_tmem ? parts * p.d : 0)) / 64);
+  p.ngrid = std::min(p.nitems, num_sms());
+  for (int alias = 0; alias <= 1; ++alias)
+    for (p.nstage = 4; p.nstage >= (alias ? 1 : 2); --p.nstage) {
+      const int total = layout(alias, kSmemLimit);
+      if (total > 0) return std::max(total, kOneCtaPerSm);
+    }
   return -1;
 }
 
@@ -513,10 +533,10 @@ int forward_prologue(const float* Q, const float* K, const float* V, const Param
   bool ok = true;
   if (p.x3) {
     ok = ok && map_nat(&maps.q, w.qh, BH, T, d, 128) && map_nat(&maps.q_lo, w.ql, BH, T, d, 128);
-    ok = ok && map_nat(&maps.k, w.kh, BH, T, d, 128) && map_nat(&maps.k_lo, w.kl, BH, T, d, 128);
+    ok = ok && map_nat(&maps.k, w.kh, BH, T, d, 64) && map_nat(&maps.k_lo, w.kl, BH, T, d, 64);
     ok = ok && map_tr(&maps.vt, w.vth, BH, T, Tp, d) && map_tr(&maps.vt_lo, w.vtl, BH, T, Tp, d);
   } else {
-    ok = ok && map_nat(&maps.q, Q, BH, T, d, 128) && map_nat(&maps.k, K, BH, T, d, 128);
+    ok = ok && map_nat(&maps.q, Q, BH, T, d, 128) && map_nat(&maps.k, K, BH, T, d, 64);
     ok = ok && map_tr(&maps.vt, w.vth, BH, T, Tp, d);
   }
   if (!ok) return KINT_ERR_LAUNCH;
@@ -848,9 +868,9 @@ int kint_attn_probe(const float* Q, const float* K, const kint_rowstats* st, flo
     pl.add(K, w.kh, w.kl, nullptr, nullptr);
     if (prep(pl, p.BH, T, round_up(T, 32), d, true, s) != cudaSuccess) return KINT_ERR_LAUNCH;
     ok = map_nat(&maps.q, w.qh, p.BH, T, d, 128) && map_nat(&maps.q_lo, w.ql, p.BH, T, d, 128) &&
-         map_nat(&maps.k, w.kh, p.BH, T, d, 128) && map_nat(&maps.k_lo, w.kl, p.BH, T, d, 128);
+         map_nat(&maps.k, w.kh, p.BH, T, d, 64) && map_nat(&maps.k_lo, w.kl, p.BH, T, d, 64);
   } else {
-    ok = map_nat(&maps.q, Q, p.BH, T, d, 128) && map_nat(&maps.k, K, p.BH, T, d, 128);
+    ok = map_nat(&maps.q, Q, p.BH, T, d, 128) && map_nat(&maps.k, K, p.BH, T, d, 64);
   }
   if (!ok) return KINT_ERR_LAUNCH;
   // pass 1 (row extrema), then the probe's two sweeps

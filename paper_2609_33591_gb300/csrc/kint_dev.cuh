@@ -100,6 +100,12 @@ struct RingPos {
       ph ^= 1u;
     }
   }
+  __device__ __forceinline__ void prev(int n) {
+    if (--i < 0) {
+      i = n - 1;
+      ph ^= 1u;
+    }
+  }
 };
 
 // Clean-up before a kernel leaves (also after a wait ran out): the last n loads issued
@@ -159,6 +165,13 @@ __device__ __forceinline__ int sched_item(const Sched& s, int n) {
   if (s.n == 0) return snake_item(n);
   const int k = s.off[blockIdx.x] + n;
   return k < s.off[blockIdx.x + 1] ? (int)s.idx[k] : 0x7fffffff;
+}
+
+// item / BH (the block of a (block, head) item): the high half of item * ceil(2^64 / BH), which
+// is exact for item * BH < 2^64; a plain division costs a persistent kernel's warps several
+// hundred cycles per item.
+__device__ __forceinline__ int item_block(const Params& p, int item) {
+  return p.BH == 1 ? item : (int)__umul64hi((unsigned long long)(unsigned)item, p.bh_magic);
 }
 
 // ---------------------------------------------------------------------------
@@ -245,6 +258,7 @@ __device__ __forceinline__ uint32_t fwm_half_bits(float v, float twoK) {
   return __float_as_uint(__fadd_rd(fminf(fmaxf(v, -1.0f), twoK), kMagic));
 }
 constexpr int kHalfTail = 2;  // tail entries ahead of q = 0
+constexpr uint32_t kLineStride = 24;  // bytes per entry of pass 2's line table
 
 // Entry q in [-2, 2K] of the half-bin table: (w^N, Delta_r / h) with r = min(q >> 1, K - 1)
 // (zeros in the tail); Delta_r / h is rounded as the full decode path rounds it.
@@ -265,6 +279,41 @@ __device__ __forceinline__ float4 fwm_line_entry(const Params& p, int q) {
   const int r = min(q >> 1, p.Kint - 1);
   const float beta = 0.5f * __fsub_rn(p.fwm_e[r + 1], p.fwm_e[r]);
   return make_float4(__fmaf_rn(-2.0f * (float)r, beta, p.fwm_e[r]), beta, p.fwm_e[(q + 1) >> 1], 0.f);
+}
+
+// Two fp32 operations in one instruction (f32x2), each rounded like its scalar form.
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  float2 d;
+  asm("{\n\t.reg .b64 a, b, c, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 c, {%6, %7};\n\t"
+      "fma.rn.f32x2 d, a, b, c;\n\tmov.b64 {%0, %1}, d;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return d;
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 a, b, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
+      "mul.rn.f32x2 d, a, b;\n\tmov.b64 {%0, %1}, d;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 a, b, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
+      "add.rn.f32x2 d, a, b;\n\tmov.b64 {%0, %1}, d;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+// (rounded toward minus infinity)
+__device__ __forceinline__ float2 add2_rd(float2 a, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 a, b, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
+      "add.rm.f32x2 d, a, b;\n\tmov.b64 {%0, %1}, d;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
 }
 
 __device__ __forceinline__ float lds_f32(uint32_t addr) {

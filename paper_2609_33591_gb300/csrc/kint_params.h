@@ -52,6 +52,7 @@ struct Sched {
 struct Params {
   int B, H, T, d, Kint, calib, recon, ste, grad, x3;
   int BH, nqb;  // number of 128-row query blocks
+  unsigned long long bh_magic;  // floor(2^64 / BH) + 1, BH > 1 (item_block)
   float tau, scale;       // scale = 1/sqrt(d)
   float fwm_inv_h;        // K / tau (FWM), host-rounded
   float fwm_hl, fwm_b0l;  // (tau / K) log2 e and -tau log2 e (resolved grid below the window)
@@ -68,8 +69,13 @@ struct Params {
   int nitems;     // work items (128-row query or key block, head), longest first
   int ngrid;      // CTAs launched: nitems, or one per SM when the kernel loops over items
   int sm_ostage;  // smem tile(s) the epilogue stages outputs in for TMA stores
+  int ost_alias, ost_n;  // pass 2: the staging area lies over the V^T ring; staging tiles (1, or 2: O and O_lerp)
+  int nstage_v;          // pass 2: slots of the V^T ring
+  int main_groups;       // pass 2: groups of compute warps per CTA (1: two CTAs per SM, 2: one)
+  int q_tmem;            // pass 2: Q as a TMEM operand (copied in by the compute warps)
   int ops_smem;  // backward: the 128-row TMEM operands (Q, dO / K, V) are staged in smem by TMA first
-  int sm_v, sm_kt;  // single-pass backward: the V tile (A operand of g^T) and the K^T tile (B operand of dQ)
+  int sm_v, sm_kt;  // single-pass backward: the V tile (A operand of g^T) and the K^T tile (B operand of dQ);
+                    // pass 2: sm_v is the V^T ring
   // Launch gate of the backward kernels that run on one side of a device-side decision:
   // with gate set, the kernel does its work only if (*gate != 0) == (gate_on != 0)
   const int* gate;

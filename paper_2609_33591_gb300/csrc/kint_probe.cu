@@ -127,8 +127,8 @@ __global__ void __launch_bounds__(NTHR, 1) k_fwd_probe(const __grid_constant__ M
         }
         uint8_t* dst = sm + p.sm_stage0 + s * p.sm_stage_bytes;
         mbar_arrive_expect_tx(&bar_full[s], parts * tile);
-        load_rows_tile(dst, &maps.k, &bar_full[s], D, 128, 0, kb * 128, bh);
-        if (p.x3) load_rows_tile(dst + tile, &maps.k_lo, &bar_full[s], D, 128, 0, kb * 128, bh);
+        load_rows_tile_boxed(dst, &maps.k, &bar_full[s], D, 128, 64, 0, kb * 128, bh);
+        if (p.x3) load_rows_tile_boxed(dst + tile, &maps.k_lo, &bar_full[s], D, 128, 64, 0, kb * 128, bh);
       }
     }
     // clean-up: the last K tiles and Q tile issued have landed

@@ -375,11 +375,12 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16]) 
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-// Round-to-nearest(ties away) to the tf32 grid, low 13 mantissa bits zero.
+// Round-to-nearest (ties away) to the tf32 grid, low 13 mantissa bits zero: half a unit added to
+// the magnitude, the low bits cleared (the value cvt.rna.tf32.f32 gives for every number;
+// that instruction runs on the conversion unit at an eighth of the issue rate, and 3xTF32
+// splits every weight).  A NaN comes out as some other value, and the lo part x - hi is NaN then.
 __device__ __forceinline__ float tf32_rna(float x) {
-  uint32_t r;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-  return __uint_as_float(r);
+  return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xFFFFE000u);
 }
 
 }  // namespace kint

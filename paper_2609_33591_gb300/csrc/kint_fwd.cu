@@ -185,87 +185,91 @@ cudaError_t launch_prep(const PrepJobs& jobs, int BH, int T, int Tp, int d, bool
 // kb is reduced; the producer warp streams K tiles through a TMA ring.
 // ---------------------------------------------------------------------------
 
-// One 32-key chunk: chunk extrema by a max/min tree, then (warp-uniform branch,
-// taken while a lane's running extremum can still move) the lanes whose chunk
-// reaches their running extremum count the chunk's equal keys with a bit mask;
-// its lowest set bit is the lowest index.  Masked keys (j > i) take -inf / +inf.
-// MIN: also the minimum side, which only the MinMax grid spans (FWM and the softmax
-// comparator are anchored at M alone).  RAW: the scale is a power of two (d = 64: 2^-3), so
-// the chunk compares the unscaled dot products, whose order and equalities are those of
-// the scaled scores (exact scaling: only scores below 2^-123 in magnitude, subnormal after
-// scaling, could merge), and M, m are scaled once when the row is stored.
-template <bool DIAG, bool MIN, bool RAW>
-__device__ __forceinline__ void stats_chunk(float (&v)[32], int j0, int i, float scale, float& M, float& m,
-                                            int& amax, int& amin, int& nmax, int& nmin) {
-  float hi[16], lo[16];
+// One 16-key chunk against a row's running extremum.  The chunk's maximum comes from a tree; a
+// lane whose chunk beats its running maximum keeps a copy of the chunk (one select per key),
+// and only the row's end looks for the equal keys in the last copy: some lane of a warp
+// improves in most chunks, and finding the equal keys there took about five instructions per
+// key against the select's one (pass 1 at B=8 H=12 T=1024 d=64: 31.6 -> 27.4 us).  A chunk that
+// only ties with the running maximum (rare) counts its equal keys at once.  Masked keys
+// (j > i) are -inf.  SIGN = -1 takes the minimum side, on negated scores.  RAW: the scale is a
+// power of two (d = 64: 2^-3), so the dot products are compared unscaled (exact scaling: only
+// scores below 2^-123 in magnitude, subnormal after scaling, could merge), and the extremum is
+// scaled once when the row is stored.
+constexpr int SCW = 16;
+struct RunMax {
+  float M = -FLT_MAX;  // running maximum
+  int j = -1;          // first key of the kept chunk
+  int extra = 0;       // keys of later chunks equal to it
+  float best[SCW];     // the kept chunk
+  __device__ __forceinline__ void chunk(const float (&v)[SCW], int j0) {
+    float t[SCW / 2];
+#pragma unroll
+    for (int q = 0; q < SCW / 2; ++q) t[q] = fmaxf(v[q], v[q + SCW / 2]);
+#pragma unroll
+    for (int w = SCW / 4; w >= 1; w >>= 1)
+#pragma unroll
+      for (int q = 0; q < w; ++q) t[q] = fmaxf(t[q], t[q + w]);
+    const bool up = t[0] > M, tie = t[0] == M;
+    if (__any_sync(0xffffffffu, up)) {
+#pragma unroll
+      for (int q = 0; q < SCW; ++q) best[q] = up ? v[q] : best[q];
+      M = up ? t[0] : M;
+      j = up ? j0 : j;
+      extra = up ? 0 : extra;
+    }
+    if (__any_sync(0xffffffffu, tie)) {
+      int c = 0;
+#pragma unroll
+      for (int q = 0; q < SCW; ++q) c += v[q] == M ? 1 : 0;
+      if (tie) extra += c;
+    }
+  }
+  // lowest index (0 where no chunk exceeded -FLT_MAX) and number of the keys equal to M
+  __device__ __forceinline__ void finish(int& arg, int& n) const {
+    uint32_t mk = 0;
+#pragma unroll
+    for (int q = 0; q < SCW; ++q) mk |= best[q] == M ? (1u << q) : 0u;
+    arg = j < 0 ? 0 : j + __ffs(mk) - 1;
+    n = extra + (j < 0 ? 0 : __popc(mk));
+  }
+};
+
+// LW keys of a thread's row from key j0: masking, scaling, and the extrema.
+template <bool MASK, bool MIN, bool RAW, int LW>
+__device__ __forceinline__ void stats_chunk(float (&v)[LW], int j0, int i, float scale, RunMax& hi, RunMax& lo) {
   if constexpr (!RAW) {
 #pragma unroll
-    for (int jj = 0; jj < 32; ++jj) v[jj] = __fmul_rn(v[jj], scale);
+    for (int jj = 0; jj < LW; ++jj) v[jj] = __fmul_rn(v[jj], scale);
   }
 #pragma unroll
-  for (int jj = 0; jj < 16; ++jj) {
-    float a = v[jj], b = v[jj + 16], a2 = a, b2 = b;
-    if constexpr (DIAG) {
-      const bool oa = j0 + jj <= i, ob = j0 + jj + 16 <= i;
-      a = oa ? a : -INFINITY;
-      b = ob ? b : -INFINITY;
-      a2 = oa ? a2 : INFINITY;
-      b2 = ob ? b2 : INFINITY;
-    }
-    hi[jj] = fmaxf(a, b);
-    if constexpr (MIN) lo[jj] = fminf(a2, b2);
-  }
+  for (int h = 0; h < LW; h += SCW) {
+    float x[SCW];
 #pragma unroll
-  for (int w = 8; w >= 1; w >>= 1)
+    for (int q = 0; q < SCW; ++q) x[q] = MASK && j0 + h + q > i ? -INFINITY : v[h + q];
+    hi.chunk(x, j0 + h);
+    if constexpr (MIN) {
 #pragma unroll
-    for (int jj = 0; jj < w; ++jj) {
-      hi[jj] = fmaxf(hi[jj], hi[jj + w]);
-      if constexpr (MIN) lo[jj] = fminf(lo[jj], lo[jj + w]);
-    }
-  const float cmax = hi[0];
-  float cmin = 0.f;
-  if constexpr (MIN) cmin = lo[0];
-  const bool um = cmax >= M, un = MIN && cmin <= m;
-  if (__any_sync(0xffffffffu, um)) {
-    uint32_t mk = 0;
-#pragma unroll
-    for (int jj = 0; jj < 32; ++jj) {
-      const bool e = (v[jj] == cmax) && (!DIAG || j0 + jj <= i);
-      mk |= e ? (1u << jj) : 0u;
-    }
-    if (um) {
-      if (cmax > M) {
-        M = cmax;
-        amax = j0 + __ffs(mk) - 1;
-        nmax = __popc(mk);
-      } else {
-        nmax += __popc(mk);
-      }
+      for (int q = 0; q < SCW; ++q) x[q] = MASK && j0 + h + q > i ? -INFINITY : -v[h + q];
+      lo.chunk(x, j0 + h);
     }
   }
-  if (MIN && __any_sync(0xffffffffu, un)) {
-    uint32_t mk = 0;
-#pragma unroll
-    for (int jj = 0; jj < 32; ++jj) {
-      const bool e = (v[jj] == cmin) && (!DIAG || j0 + jj <= i);
-      mk |= e ? (1u << jj) : 0u;
-    }
-    if (un) {
-      if (cmin < m) {
-        m = cmin;
-        amin = j0 + __ffs(mk) - 1;
-        nmin = __popc(mk);
-      } else {
-        nmin += __popc(mk);
-      }
-    }
+}
+
+// The extrema of a row's two column halves: value, lowest index, count (the half at `o` second).
+__device__ __forceinline__ void merge_max(float& M, int& a, int& n, float Mo, int ao, int no) {
+  if (Mo > M || (Mo == M && no > 0 && ao < a)) a = (Mo > M || n == 0) ? ao : min(a, ao);
+  if (Mo > M) {
+    n = no;
+    M = Mo;
+  } else if (Mo == M) {
+    n += no;
   }
 }
 
 static dim3 launch_grid(const Params& p) { return dim3((unsigned)p.ngrid); }
 
 template <bool MIN, bool RAW>
-__global__ void __launch_bounds__(NTHR, 2) k_fwd_stats(const __grid_constant__ Maps maps, const Params p,
+__global__ void __launch_bounds__(NTHR, RAW ? 2 : 1) k_fwd_stats(const __grid_constant__ Maps maps, const Params p,
                                                          const __grid_constant__ Sched sch) {
   uint8_t* sm = smem_base();
   const int D = p.d, tile = D * 512, parts = p.x3 ? 2 : 1, NS = p.nstage;
@@ -380,8 +384,7 @@ __global__ void __launch_bounds__(NTHR, 2) k_fwd_stats(const __grid_constant__ M
     for (int item = sched_item(sch, n); item < p.nitems && !failed; item = sched_item(sch, ++n)) {
       const int qb = p.nqb - 1 - item / p.BH, bh = item % p.BH, nkb = qb + 1;
       const int i = qb * 128 + row;
-      float M = -FLT_MAX, m = FLT_MAX;
-      int amax = 0, amin = 0, nmax = 0, nmin = 0;
+      RunMax hi, lo;  // (lo: of the negated scores)
       for (int kb = 0; kb < nkb; ++kb) {
         const int gk = g + kb, b = gk & 1;
         if (!mbar_wait(&bar_s[b], (gk >> 1) & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_MMA)) {
@@ -390,17 +393,17 @@ __global__ void __launch_bounds__(NTHR, 2) k_fwd_stats(const __grid_constant__ M
         }
         tc_fence_after();
         const bool diag = kb == qb;
+        constexpr int LW = MIN && RAW ? 16 : 32;  // (two CTAs per SM: two kept chunks leave few registers)
 #pragma unroll 1
-        for (int cc = 0; cc < 2; ++cc) {
-          const int c = cg * 2 + cc;
-          float v[32];
-          tmem_ld32(lane_addr(tmem, b * 128 + c * 32), v);
+        for (int c = cg * 64; c < cg * 64 + 64; c += LW) {
+          float v[LW];
+          tmem_ldw<LW>(lane_addr(tmem, b * 128 + c), v);
           tmem_ld_wait();
-          const int j0 = kb * 128 + c * 32;
+          const int j0 = kb * 128 + c;
           if (diag)
-            stats_chunk<true, MIN, RAW>(v, j0, i, p.scale, M, m, amax, amin, nmax, nmin);
+            stats_chunk<true, MIN, RAW>(v, j0, i, p.scale, hi, lo);
           else
-            stats_chunk<false, MIN, RAW>(v, j0, i, p.scale, M, m, amax, amin, nmax, nmin);
+            stats_chunk<false, MIN, RAW>(v, j0, i, p.scale, hi, lo);
         }
         tc_fence_before();
         __syncwarp();
@@ -410,6 +413,13 @@ __global__ void __launch_bounds__(NTHR, 2) k_fwd_stats(const __grid_constant__ M
       failed = group_any(BAR_COMPUTE, NCOMP, failed);
       if (failed) break;
       // combine the two column halves of each row
+      float M = hi.M, m = -FLT_MAX;
+      int amax, nmax, amin = 0, nmin = 0;
+      hi.finish(amax, nmax);
+      if constexpr (MIN) {
+        m = lo.M;
+        lo.finish(amin, nmin);
+      }
       if (cg == 1) {
         xch[0 * 128 + row] = M;
         xch[1 * 128 + row] = m;
@@ -423,21 +433,10 @@ __global__ void __launch_bounds__(NTHR, 2) k_fwd_stats(const __grid_constant__ M
         const float M1 = xch[row], m1 = xch[128 + row];
         const int amax1 = __float_as_int(xch[256 + row]), amin1 = __float_as_int(xch[384 + row]);
         const int nmax1 = __float_as_int(xch[512 + row]), nmin1 = __float_as_int(xch[640 + row]);
-        if (M1 > M || (M1 == M && nmax1 > 0 && amax1 < amax)) amax = (M1 > M || nmax == 0) ? amax1 : min(amax, amax1);
-        if (M1 > M) {
-          nmax = nmax1;
-          M = M1;
-        } else if (M1 == M) {
-          nmax += nmax1;
-        }
+        merge_max(M, amax, nmax, M1, amax1, nmax1);
         if (MIN) {
-          if (m1 < m || (m1 == m && nmin1 > 0 && amin1 < amin)) amin = (m1 < m || nmin == 0) ? amin1 : min(amin, amin1);
-          if (m1 < m) {
-            nmin = nmin1;
-            m = m1;
-          } else if (m1 == m) {
-            nmin += nmin1;
-          }
+          merge_max(m, amin, nmin, m1, amin1, nmin1);
+          m = -m;
         } else {  // not computed: +inf, index -1, count 0
           m = INFINITY;
           amin = -1;

@@ -450,12 +450,14 @@ int plan_dkdv(Params& p, int sel) {
   p.nbuf = (base + 256 + acc <= 512) ? 2 : 1;
   p.sm_a = 0;
   p.sm_stage0 = p.ops_smem ? 2 * 128 * p.d * 4 : 0;
-  p.sm_stage_bytes = 4 * parts * qtile + 64 * 64 + (p.calib == KINT_CALIB_MINMAX ? 64 * p.Kp * 8 : 0);
+  // the tiles this launch reads: Q; dO, Q^T for dK; dO^T for dV
+  const int tiles = 1 + (doDK ? 2 : 0) + (doDV ? 1 : 0);
+  p.sm_stage_bytes = round_up(tiles * parts * qtile + 64 * 64 + (p.calib == KINT_CALIB_MINMAX ? 64 * p.Kp * 8 : 0), 1024);
   for (p.nstage = 4; p.nstage >= 1; --p.nstage) {
     p.sm_table = p.sm_stage0 + p.nstage * p.sm_stage_bytes;
     // FWM Nearest: the half-bin table, 2K + 3 entries of 8 bytes
     const int table = (p.calib == KINT_CALIB_FWM || p.calib == KINT_CALIB_FWM_RESOLVED) ? 2048 : 1024;
-    const int total = std::max(finish_plan(p, p.sm_table + table, 4 * p.nstage + 9), kOneCtaPerSm);
+    const int total = std::max(finish_plan(p, p.sm_table + table, 4 * p.nstage + 10), kOneCtaPerSm);
     if (total <= kSmemLimit) {
       if (p.nstage == 1) p.nbuf = 1;
       // one CTA per SM looping over the (key block, head) items

@@ -6,13 +6,26 @@
 
 namespace kint {
 
+// Thread roles: sixteen compute warps (thread t owns key kb*128 + t%128 and the 16 query columns
+// 16 (t/128) .. + 15 of each 64-query tile), the MMA warp, the producer warp and two idle
+// warps.  The fifth warpgroup gives registers to the compute warpgroups: launched at 96 per
+// thread, it keeps 64 and they take 104.
+constexpr int NCG_KV = 4, NCOMP_KV = 128 * NCG_KV, NTHR_KV = NCOMP_KV + 128;
+constexpr int MMA_WARP_KV = NCOMP_KV / 32, PRODUCER_WARP_KV = MMA_WARP_KV + 1;
+constexpr int REG_LAUNCH_KV = 96, REG_COMP_KV = 104, REG_AUX_KV = 64;
+static_assert(NCOMP_KV * REG_COMP_KV + 128 * REG_AUX_KV <= NTHR_KV * REG_LAUNCH_KV,
+              "register shares exceed the launch allocation");
+
 // ---------------------------------------------------------------------------
 // dK/dV kernel element work on one 32-query chunk of one key j: the forward
 // probability P_ij and dS_ij = gamma_ij Delta_ij plus, at the arg-max / arg-min
 // key of row i, c_M / n_max and c_m / n_min (Eq. full).  Row constants come
 // from the RowRec array of the tile in shared memory (broadcast loads).
 // ---------------------------------------------------------------------------
-template <int CAL, int REC, bool FULLG, bool PROJ, bool MASKED, bool TIES, int W>
+// DV / DK: which of P and dS the launch feeds to a product; the other is not formed (its record
+// words and table entries are not read either: the shared-memory loads are this chunk's
+// largest cost).
+template <int CAL, int REC, bool FULLG, bool PROJ, bool MASKED, bool TIES, bool DV, bool DK, int W>
 __device__ __forceinline__ void kv_chunk(const float (&sv)[W], const float (&gv)[W], float (&pa)[W],
                                          float (&da)[W], int j, int i0, int T, uint32_t recs, uint32_t tabs,
                                          uint32_t fwtab, uint32_t tstride, float Kf, float fwm_inv_h,
@@ -21,18 +34,20 @@ __device__ __forceinline__ void kv_chunk(const float (&sv)[W], const float (&gv)
   for (int ii = 0; ii < W; ++ii) {
     const uint32_t ra = recs + ii * 64u;  // RowRec of query row i0 + ii
     const float4 r0 = lds_f4(ra);          // c0, k1, invWf, ga
-    const float4 r1 = lds_f4(ra + 16);     // gb, cMn, amax, flags
-    float4 r2 = make_float4(0.f, 0.f, 0.f, 0.f);
-    if constexpr (CAL == CAL_MINMAX) r2 = lds_f4(ra + 32);  // inv_h, cmn, amin, -
-    const float gam = __fmaf_rn(gv[ii], r0.w, r1.x);
-    float pv, ds;
+    float4 r1 = make_float4(0.f, 0.f, 0.f, 0.f), r2 = r1;
+    if constexpr (DK) r1 = lds_f4(ra + 16);                         // gb, cMn, amax, flags
+    else if constexpr (CAL == CAL_MINMAX) r1.w = lds_f32(ra + 28);  // flags
+    if constexpr (DK && CAL == CAL_MINMAX) r2 = lds_f4(ra + 32);    // inv_h, cmn, amin, -
+    float gam = 0.f;
+    if constexpr (DK) gam = __fmaf_rn(gv[ii], r0.w, r1.x);
+    float pv = 0.f, ds = 0.f;
     if constexpr (CAL == CAL_SOFTMAX) {
       pv = ex2_approx(__fmaf_rn(sv[ii], r0.y, r0.x)) * r0.z;
       ds = pv * gam;
     } else if constexpr (CAL == CAL_EXP8) {
       // forward P from the E4M3-rounded weight; dS from the exponential itself
       const float we = ex2_approx(__fmaf_rn(sv[ii], r0.y, r0.x));
-      pv = e4m3_rn(we) * r0.z;
+      if constexpr (DV) pv = e4m3_rn(we) * r0.z;
       ds = gam * we;
     } else if constexpr (CAL == CAL_EXPB) {
       // record holds -M, scale: z = acc * scale - M; the bfloat16 chain rule
@@ -44,7 +59,10 @@ __device__ __forceinline__ void kv_chunk(const float (&sv)[W], const float (&gv)
       // record holds 2k1, 2c0; Kf = 2K; fwtab: the half-bin table of (w^N, Delta_r / h)
       const float v = __fmaf_rn(sv[ii], r0.y, r0.x);
       const uint32_t qb = fwm_half_bits(v, Kf);
-      float2 e = lds_f2(fwtab + qb * 8u);
+      float2 e = make_float2(0.f, 0.f);
+      if constexpr (DV && DK) e = lds_f2(fwtab + qb * 8u);
+      else if constexpr (DV) e.x = lds_f32(fwtab + qb * 8u);
+      else e.y = lds_f32(fwtab + qb * 8u + 4u);
       if constexpr (CAL == CAL_FWMR) {
         // resolved: below the window, (w^N, Delta_r / h) of the continued grid (u = v / 2 exactly)
         const BelowPair bp = resolved_below(__fmul_rn(v, 0.5f), hl, b0l);
@@ -82,10 +100,10 @@ __device__ __forceinline__ void kv_chunk(const float (&sv)[W], const float (&gv)
       }
       pv = w * r0.z;
     }
-    if constexpr (FULLG && CAL != CAL_SOFTMAX) {
+    if constexpr (DK && FULLG && CAL != CAL_SOFTMAX) {
       ds += (j == __float_as_int(r1.z)) ? r1.y : 0.f;
       if constexpr (CAL == CAL_MINMAX) ds += (j == __float_as_int(r2.z)) ? r2.y : 0.f;
-    } else if constexpr (PROJ && CAL != CAL_SOFTMAX) {
+    } else if constexpr (DK && PROJ && CAL != CAL_SOFTMAX) {
       ds = __fsub_rn(ds, r1.y);  // detached, P1 projection: minus the row mean
     }
     if constexpr (MASKED) {
@@ -94,7 +112,7 @@ __device__ __forceinline__ void kv_chunk(const float (&sv)[W], const float (&gv)
       pv = ok ? pv : 0.f;
       ds = ok ? ds : 0.f;
     }
-    if constexpr (FULLG && TIES && CAL != CAL_SOFTMAX) {
+    if constexpr (DK && FULLG && TIES && CAL != CAL_SOFTMAX) {
       // rows with tied extrema (flagged per 64-row query tile by the dQ kernel): the tie set
       // is found by equality on the recomputed scores (rare, kept off the common path)
       const int fl = __float_as_int(r1.w);
@@ -107,8 +125,8 @@ __device__ __forceinline__ void kv_chunk(const float (&sv)[W], const float (&gv)
         if (CAL == CAL_MINMAX && (fl & REC_TIEMIN) && sc == ext.y) ds += r2.y;
       }
     }
-    pa[ii] = pv;
-    da[ii] = ds;
+    if constexpr (DV) pa[ii] = pv;
+    if constexpr (DK) da[ii] = ds;
   }
 }
 
@@ -146,29 +164,40 @@ __device__ __forceinline__ void rowsum_add(const float (&v)[16], float* dsum, fl
   }
 }
 
-// MMA thread of k_bwd_dkdv: wait for the query tile in stage st (ring position), then
-// S^T_b = K Q^T and (dK launches) g^T_b = V dO^T into score buffer b.
+// MMA warp of k_bwd_dkdv: the products of the query tile in stage s (landed) into score buffer b.
+__device__ __forceinline__ void kv_issue_s(const Params& p, const uint8_t* st, int b, uint32_t cKa, uint32_t cSG,
+                                           int qtile) {
+  const int D = p.d;
+  const uint32_t cS = cSG + 128 * b;
+  if (p.x3) {
+    mma_tmem_smem(cS, cKa + D, st, BT, D, false);
+    mma_tmem_smem(cS, cKa, st + qtile, BT, D, true);
+    mma_tmem_smem(cS, cKa, st, BT, D, true);
+  } else {
+    mma_tmem_smem(cS, cKa, st, BT, D, false);
+  }
+}
+__device__ __forceinline__ void kv_issue_g(const Params& p, const uint8_t* st, int b, uint32_t cVa, uint32_t cSG,
+                                           int qtile, int odO) {
+  const int D = p.d;
+  const uint32_t cG = cSG + 128 * b + 64;
+  if (p.x3) {
+    mma_tmem_smem(cG, cVa + D, st + odO, BT, D, false);
+    mma_tmem_smem(cG, cVa, st + odO + qtile, BT, D, true);
+    mma_tmem_smem(cG, cVa, st + odO, BT, D, true);
+  } else {
+    mma_tmem_smem(cG, cVa, st + odO, BT, D, false);
+  }
+}
+// Both (S^T_b = K Q^T and, with V, g^T_b = V dO^T) once the tile in stage stg has landed.
 __device__ __forceinline__ bool kv_issue_sg(const Params& p, RingPos stg, int b, uint64_t* bar_full,
                                             uint64_t* bar_sfull, const uint8_t* st0, uint32_t cKa, uint32_t cVa,
-                                            uint32_t cSG, int qtile, bool needV, int oQ, int odO) {
-  const int D = p.d, s = stg.i;
-  if (!mbar_wait_warp(&bar_full[s], stg.ph, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA)) return false;
+                                            uint32_t cSG, int qtile, bool needV, int odO) {
+  if (!mbar_wait_warp(&bar_full[stg.i], stg.ph, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA)) return false;
   tc_fence_after();
-  const uint8_t* st = st0 + s * p.sm_stage_bytes;
-  const uint32_t cS = cSG + 128 * b, cG = cS + 64;
-  if (p.x3) {
-    mma_tmem_smem(cS, cKa + D, st + oQ, BT, D, false);
-    mma_tmem_smem(cS, cKa, st + oQ + qtile, BT, D, true);
-    mma_tmem_smem(cS, cKa, st + oQ, BT, D, true);
-    if (needV) {
-      mma_tmem_smem(cG, cVa + D, st + odO, BT, D, false);
-      mma_tmem_smem(cG, cVa, st + odO + qtile, BT, D, true);
-      mma_tmem_smem(cG, cVa, st + odO, BT, D, true);
-    }
-  } else {
-    mma_tmem_smem(cS, cKa, st + oQ, BT, D, false);
-    if (needV) mma_tmem_smem(cG, cVa, st + odO, BT, D, false);
-  }
+  const uint8_t* st = st0 + stg.i * p.sm_stage_bytes;
+  kv_issue_s(p, st, b, cKa, cSG, qtile);
+  if (needV) kv_issue_g(p, st, b, cVa, cSG, qtile, odO);
   mma_commit(&bar_sfull[b]);
   return true;
 }
@@ -186,16 +215,26 @@ __device__ __forceinline__ bool store_staged_dkdv(const Maps& maps, const Params
 }
 
 // ---------------------------------------------------------------------------
-// k_bwd_dkdv.  Thread t (< 256) owns key j = kb*128 + t%128 and the query half
-// t/128 of each 64-query tile.  TMEM: K [0, dp), V [dp, 2dp) (dK launches),
+// k_bwd_dkdv.  TMEM: K [0, dp), V [dp, 2dp) (dK launches),
 // then per buffer b: S^T_b (64 columns) and g^T_b (64 columns) from `base`,
 // dV, dK.  P^T overwrites S^T_b and dS^T overwrites g^T_b (3xTF32: the single
 // product's hi part goes to S^T_b, its lo part to g^T_b).
-// smem stage: Q | dO | Q^T | dO^T tiles (hi[, lo]), the 64 RowRecs of the tile,
-// and (MinMax) their grid pair tables; FWM's shared table at sm_table.
+// smem stage: the tiles the launch reads of Q | dO | Q^T | dO^T (hi[, lo]): Q, and dO and Q^T
+// for dK, dO^T for dV; the 64 RowRecs of the tile, and (MinMax) their grid pair tables;
+// FWM's shared table at sm_table.  (With all four in every stage a one-product launch at
+// d = 128 or under 3xTF32 had one stage and nothing overlapped.)
+// What bounds it: the issue of the products by one warp and, at one score buffer, the chain
+// products -> element work -> products; shared-memory loads of the row records come next.
+// Measured on GB300 against eight compute warps and stages of all four tiles: B=4 H=16 T=2048
+// d=128 FWM Weight-STE dV 340 -> 178 us, dK 403 -> 330; H=16 T=16384 d=128 MinMax K=16 LERP
+// 5097 -> 2252, 5878 -> 4178; 3xTF32 B=8 H=12 T=1024 168 -> 98, 203 -> 190; MinMax B=4 H=12
+// T=1024 d=64 (both products) 73.6 -> 71.6.
+// With one score buffer (dK alone at d = 128, TF32) the next tile's S^T is formed under the
+// element work of the current one, once every warp has loaded its scores (bar_sread): dS
+// overwrites g^T, so S^T's columns are free from then on.
 // ---------------------------------------------------------------------------
-template <int CAL, int REC, bool FULLG, bool PROJ = false, bool RS = false>
-__global__ void __launch_bounds__(NTHR, 1) k_bwd_dkdv(const __grid_constant__ Maps maps, const Params p) {
+template <int CAL, int REC, bool FULLG, bool PROJ, bool RS, int SEL>
+__global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__ Maps maps, const Params p) {
   uint8_t* sm = smem_base();
   if (p.gate != nullptr) {
     // launched on one side of a device-side decision: when the single-pass backward ran
@@ -205,7 +244,7 @@ __global__ void __launch_bounds__(NTHR, 1) k_bwd_dkdv(const __grid_constant__ Ma
   }
   const int D = p.d, Kq = p.Kint, parts = p.x3 ? 2 : 1, NS = p.nstage, nbuf = p.nbuf;
   const int qtile = BT * D * 4;
-  const bool doDV = p.dkv_sel != DKV_DK, doDK = p.dkv_sel != DKV_DV, needV = doDK;
+  constexpr bool doDV = SEL != DKV_DK, doDK = SEL != DKV_DV, needV = doDK;
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm + p.sm_bars);
   uint64_t* bar_full = bars;
   uint64_t* bar_empty = bars + NS;
@@ -223,7 +262,8 @@ __global__ void __launch_bounds__(NTHR, 1) k_bwd_dkdv(const __grid_constant__ Ma
   // products dV, dK that read it complete (bar_empty)
   uint64_t* bar_emptyA = bars + 3 * NS + 8;  // [NS]
   uint64_t* bar_drain = bars + 4 * NS + 8;   // the MMA warp's clean-up commit
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 4 * NS + 9);
+  uint64_t* bar_sread = bars + 4 * NS + 9;   // S^T of the tile in every compute warp's registers (early_s)
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 4 * NS + 10);
   const int tid = threadIdx.x, warp = warp_id_uniform();
   const int dp = D * parts;
   const int cK = 0, cV = dp, base = needV ? 2 * dp : dp;
@@ -235,28 +275,31 @@ __global__ void __launch_bounds__(NTHR, 1) k_bwd_dkdv(const __grid_constant__ Ma
   // steps by three, and the two sums meet in fp32 in the epilogue.
   const int cdC = cdK + (doDK ? D : 0);
   const int nqt = (p.T + BT - 1) / BT;
-  const int oQ = 0, odO = parts * qtile, oQT = 2 * parts * qtile, odOT = 3 * parts * qtile;
-  const int oRec = 4 * parts * qtile, oTab = oRec + BT * 64;
+  const int oQ = 0, odO = parts * qtile, oQT = (needV ? 2 : 1) * parts * qtile,
+            odOT = oQT + (doDK ? parts * qtile : 0);
+  const int oRec = odOT + (doDV ? parts * qtile : 0), oTab = oRec + BT * 64;
+  const bool early_s = nbuf == 1 && !p.x3 && !doDV && NS > 1;
   const uint32_t tstride = (uint32_t)p.Kp * 8u;
-  constexpr int W = BT / NCG;  // query columns per thread per tile
-  constexpr int WS = 16;       // columns per register chunk
+  constexpr int W = BT / NCG_KV;  // query columns per thread per tile
+  static_assert(W == 16, "the element work and the row sums take 16 columns");
 
   if (tid == 0) {
     for (int s = 0; s < NS; ++s) {
       mbar_init(&bar_full[s], 1);
       mbar_init(&bar_fullT[s], 1);
       mbar_init(&bar_empty[s], 1);
-      mbar_init(&bar_emptyA[s], NCOMP / 32);
+      mbar_init(&bar_emptyA[s], NCOMP_KV / 32);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&bar_sfull[b], 1);
-      mbar_init(&bar_pready[b], NCOMP / 32);
+      mbar_init(&bar_pready[b], NCOMP_KV / 32);
     }
     mbar_init(bar_done, 1);
-    mbar_init(bar_ops, NCOMP / 32);
+    mbar_init(bar_ops, NCOMP_KV / 32);
     mbar_init(bar_stg, 1);
-    mbar_init(bar_ostg, NCOMP / 32);
+    mbar_init(bar_ostg, NCOMP_KV / 32);
     mbar_init(bar_drain, 1);
+    mbar_init(bar_sread, NCOMP_KV / 32);
     fence_mbar_init();
   }
   if (warp == 0) {
@@ -276,7 +319,9 @@ __global__ void __launch_bounds__(NTHR, 1) k_bwd_dkdv(const __grid_constant__ Ma
   // Work items are (128-key block kb, head) pairs, longest first (kb = 0 meets every
   // query tile); a CTA takes the items snake_item(0), snake_item(1), ...  Tile counters
   // (stage ring, score buffers) run on across items.
-  if (warp == PRODUCER_WARP) {
+  if (warp >= NCOMP_KV / 32) {
+  setmaxnreg_dec<REG_AUX_KV>();
+  if (warp == PRODUCER_WARP_KV) {
     int gt = 0, n = 0;
     RingPos ld;  // stage of the next tile loaded
     RingPos nf, nT;  // ring positions after the last first-half and transposed-half loads issued
@@ -356,10 +401,11 @@ __global__ void __launch_bounds__(NTHR, 1) k_bwd_dkdv(const __grid_constant__ Ma
     drain_ring(bar_full, nf, cf, NS, p.wait_ns, p.status);
     drain_ring(bar_fullT, nT, cT, NS, p.wait_ns, p.status);
     if (staged > 0) mbar_wait_warp(bar_stg, (staged - 1) & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA);
-  } else if (warp == MMA_WARP) {
+  } else if (warp == MMA_WARP_KV) {
     const uint8_t* st0 = sm + p.sm_stage0;
     const uint32_t cKa = tmem + cK, cVa = tmem + cV, cSG = tmem + base;
     int n = 0;
+    uint32_t gt = 0;         // tiles of the CTA's earlier items (early_s)
     RingPos is, ib, cs, cb;  // stage / buffer of the next S^T, g^T product and of the tile being finished
     bool ok = true;
     for (int item = snake_item(n); item < p.nitems && ok; item = snake_item(++n)) {
@@ -368,15 +414,23 @@ __global__ void __launch_bounds__(NTHR, 1) k_bwd_dkdv(const __grid_constant__ Ma
       // item's last S, g were read)
       ok = mbar_wait_warp(bar_ops, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_SYNC);
       if (ok) tc_fence_after();
-      ok = ok && kv_issue_sg(p, is, ib.i, bar_full, bar_sfull, st0, cKa, cVa, cSG, qtile, needV, oQ, odO);
+      ok = ok && kv_issue_sg(p, is, ib.i, bar_full, bar_sfull, st0, cKa, cVa, cSG, qtile, needV, odO);
       is.next(NS);
       ib.next(nbuf);
       for (int it = 0; it < nit && ok; ++it, cs.next(NS), cb.next(nbuf)) {
         const int b = cb.i, s = cs.i;
         if (nbuf == 2 && it + 1 < nit) {
-          ok = kv_issue_sg(p, is, ib.i, bar_full, bar_sfull, st0, cKa, cVa, cSG, qtile, needV, oQ, odO);
+          ok = kv_issue_sg(p, is, ib.i, bar_full, bar_sfull, st0, cKa, cVa, cSG, qtile, needV, odO);
           is.next(NS);
           ib.next(nbuf);
+        }
+        if (ok && early_s && it + 1 < nit) {
+          ok = mbar_wait_warp(&bar_full[is.i], is.ph, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA) &&
+               mbar_wait_warp(bar_sread, (gt + it) & 1u, p.wait_ns, p.status, DEV_ERR_TIMEOUT_SYNC);
+          if (ok) {
+            tc_fence_after();
+            kv_issue_s(p, st0 + is.i * p.sm_stage_bytes, 0, cKa, cSG, qtile);
+          }
         }
         if (!ok) break;
         if (!mbar_wait_warp(&bar_pready[b], cb.ph, p.wait_ns, p.status, DEV_ERR_TIMEOUT_SYNC) ||
@@ -399,31 +453,44 @@ __global__ void __launch_bounds__(NTHR, 1) k_bwd_dkdv(const __grid_constant__ Ma
           if (doDK) mma_tmem_smem(tmem + cdK, cG, st + oQT, D, BT, acc);
         }
         mma_commit(&bar_empty[s]);
-        if (nbuf == 1 && it + 1 < nit) {
-          ok = kv_issue_sg(p, is, ib.i, bar_full, bar_sfull, st0, cKa, cVa, cSG, qtile, needV, oQ, odO);
+        if (early_s && it + 1 < nit) {  // (the wait for the tile, ahead of its S^T, covered dO too)
+          kv_issue_g(p, st0 + is.i * p.sm_stage_bytes, 0, cVa, cSG, qtile, odO);
+          mma_commit(&bar_sfull[0]);
+          is.next(NS);
+          ib.next(nbuf);
+        } else if (nbuf == 1 && it + 1 < nit) {
+          ok = kv_issue_sg(p, is, ib.i, bar_full, bar_sfull, st0, cKa, cVa, cSG, qtile, needV, odO);
           is.next(NS);
           ib.next(nbuf);
         }
       }
+      gt += (uint32_t)nit;
       mma_commit(bar_done);
     }
     drain_mma(bar_drain, p.wait_ns, p.status);  // clean-up: no product still writes TMEM
+  }
   } else {
-    const int row = tid & 127, cg = (tid >> 7) & (NCG - 1);
-    // K / V rows of the n-th item into TMEM (column group 0 takes K, group 1 takes V),
-    // handed to the MMA warp through bar_ops: TF32 at d = 64 from the tiles the producer
-    // staged in smem, otherwise from global rows.  The next item's rows go in as soon as
-    // the current item's last S^T, g^T have been read, so its first products run under
-    // the current item's epilogue.
+    setmaxnreg_inc<REG_COMP_KV>();
+    const int row = tid & 127, cg = tid >> 7;
+    // K / V rows of the n-th item into TMEM (each thread a share of its key's columns: with V two
+    // column groups take K and two take V), handed to the MMA warp through bar_ops: TF32 at
+    // d = 64 from the tiles the producer staged in smem, otherwise from global rows.  The
+    // next item's rows go in as soon as the current item's last S^T, g^T have been read, so
+    // its first products run under the current item's epilogue.
     auto ops_to_tmem = [&](int n) {
       const int item = snake_item(n), kb = item / p.BH, bh = item % p.BH, j = kb * 128 + row;
-      if (p.ops_smem) {
-        if (mbar_wait(bar_stg, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA) && (cg == 0 || needV))
-          staged_row_to_tmem(tmem, cg == 0 ? cK : cV, sm + p.sm_a + (cg == 0 ? 0 : 128 * D * 4), row, D);
-      } else {
-        const size_t lim = j < p.T ? (size_t)(bh + 1) * p.T : 0;
-        if (cg == 0) row_to_tmem(tmem, cK, p.K, bh * p.T + j, lim, D, p.x3 != 0);
-        else if (needV) row_to_tmem(tmem, cV, p.V, bh * p.T + j, lim, D, p.x3 != 0);
+      const bool isV = needV && cg >= 2;
+      const int nc = needV ? D / 2 : D / NCG_KV, c0 = (needV ? cg & 1 : cg) * nc;
+      const bool ok = !p.ops_smem || mbar_wait(bar_stg, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA);
+      if (ok) {
+        const int lim = j < p.T ? (bh + 1) * p.T : 0;
+#pragma unroll 1
+        for (int c = c0; c < c0 + nc; c += 16) {
+          if (p.ops_smem)
+            staged16_to_tmem(tmem, isV ? cV : cK, sm + p.sm_a + (isV ? 128 * D * 4 : 0), row, c);
+          else
+            row_to_tmem_part<16>(tmem, isV ? cV : cK, isV ? p.V : p.K, bh * p.T + j, lim, D, c, p.x3 != 0);
+        }
       }
       tmem_st_wait();
       tc_fence_before();
@@ -443,7 +510,7 @@ __global__ void __launch_bounds__(NTHR, 1) k_bwd_dkdv(const __grid_constant__ Ma
     }
     const float Kf = (float)(half ? 2 * Kq : Kq);
     const uint32_t fwtab = smem_u32(sm + p.sm_table) + (half ? 8u * kHalfTail : 0u) - 0x58000000u;
-    group_sync(BAR_COMPUTE, NCOMP);  // the FWM table
+    group_sync(BAR_COMPUTE, NCOMP_KV);  // the FWM table
     bool failed = false;
     int n = 0;
     RingPos cs, cb;  // stage and score buffer of the current tile
@@ -452,11 +519,11 @@ __global__ void __launch_bounds__(NTHR, 1) k_bwd_dkdv(const __grid_constant__ Ma
       const int qt0 = (kb * 128) / BT, nit = nqt - qt0;
       const int j = kb * 128 + row;
       const int* tflags = p.tileflags + (size_t)bh * p.nqt + qt0;
-      int tie_next = (FULLG && CAL != CAL_SOFTMAX) ? __ldg(tflags) : 0;
+      int tie_next = (doDK && FULLG && CAL != CAL_SOFTMAX) ? __ldg(tflags) : 0;
       for (int it = 0; it < nit; ++it, cs.next(NS), cb.next(nbuf)) {
         // the tie flag of this 64-row query tile, loaded one tile ahead
         const int tie_here = tie_next;
-        if (FULLG && CAL != CAL_SOFTMAX && it + 1 < nit) tie_next = __ldg(tflags + it + 1);
+        if (doDK && FULLG && CAL != CAL_SOFTMAX && it + 1 < nit) tie_next = __ldg(tflags + it + 1);
         const int b = cb.i, s = cs.i;
         const int q0 = (qt0 + it) * BT;
         const bool ok1 = mbar_wait(&bar_sfull[b], cb.ph, p.wait_ns, p.status, DEV_ERR_TIMEOUT_MMA);
@@ -468,50 +535,58 @@ __global__ void __launch_bounds__(NTHR, 1) k_bwd_dkdv(const __grid_constant__ Ma
         }
         tc_fence_after();
         const uint8_t* st = sm + p.sm_stage0 + s * p.sm_stage_bytes;
-        // two 16-column halves of the thread's W columns (bounds the live registers)
-#pragma unroll 1
-        for (int h = 0; h < W / WS; ++h) {
-          const int c0 = cg * W + h * WS, i0h = q0 + c0;
-          const uint32_t recs = smem_u32(st + oRec) + c0 * 64;
-          const uint32_t tabs = smem_u32(st + oTab) + c0 * tstride - 0x58000000u;
-          const int cS = base + 128 * b + c0, cG = cS + 64;
-          float sv[WS], gv[WS], pa[WS], da[WS];
-          tmem_ldw<WS>(lane_addr(tmem, cS), sv);
-          if (needV) {
-            tmem_ldw<WS>(lane_addr(tmem, cG), gv);
-          } else {
+        const int c0 = cg * W, i0h = q0 + c0;
+        const uint32_t recs = smem_u32(st + oRec) + c0 * 64;
+        const uint32_t tabs = smem_u32(st + oTab) + c0 * tstride - 0x58000000u;
+        const int cS = base + 128 * b + c0, cG = cS + 64;
+        float sv[W], gv[W], pa[W], da[W];
+        tmem_ldw<W>(lane_addr(tmem, cS), sv);
+        if (needV) {
+          tmem_ldw<W>(lane_addr(tmem, cG), gv);
+        } else {
 #pragma unroll
-            for (int q = 0; q < WS; ++q) gv[q] = 0.f;
-          }
-          tmem_ld_wait();
-          const bool masked = (i0h < kb * 128 + 128) || (i0h + WS > p.T);
-          if (FULLG && CAL != CAL_SOFTMAX && tie_here)
-            kv_chunk<CAL, REC, FULLG, PROJ, true, true, WS>(sv, gv, pa, da, j, i0h, p.T, recs, tabs, fwtab, tstride, Kf,
-                                                      p.fwm_inv_h, p.scale, p.fwm_hl, p.fwm_b0l);
+          for (int q = 0; q < W; ++q) gv[q] = 0.f;
+        }
+        tmem_ld_wait();
+        if (early_s) {  // the next tile's S^T may overwrite the scores
+          tc_fence_before();
+          __syncwarp();
+          if ((tid & 31) == 0) mbar_arrive(bar_sread);
+        }
+        // this warp's keys against its queries: all pairs masked, some, or none
+        const int j0w = kb * 128 + (warp & 3) * 32;
+        if (i0h + W <= j0w) {
+#pragma unroll
+          for (int q = 0; q < W; ++q) pa[q] = da[q] = 0.f;
+        } else {
+          const bool masked = i0h < j0w + 31 || i0h + W > p.T;
+          if (doDK && FULLG && CAL != CAL_SOFTMAX && tie_here)
+            kv_chunk<CAL, REC, FULLG, PROJ, true, true, doDV, doDK, W>(sv, gv, pa, da, j, i0h, p.T, recs, tabs, fwtab, tstride, Kf,
+                                                     p.fwm_inv_h, p.scale, p.fwm_hl, p.fwm_b0l);
           else if (masked)
-            kv_chunk<CAL, REC, FULLG, PROJ, true, false, WS>(sv, gv, pa, da, j, i0h, p.T, recs, tabs, fwtab, tstride,
-                                                       Kf, p.fwm_inv_h, p.scale, p.fwm_hl, p.fwm_b0l);
+            kv_chunk<CAL, REC, FULLG, PROJ, true, false, doDV, doDK, W>(sv, gv, pa, da, j, i0h, p.T, recs, tabs, fwtab, tstride,
+                                                      Kf, p.fwm_inv_h, p.scale, p.fwm_hl, p.fwm_b0l);
           else
-            kv_chunk<CAL, REC, FULLG, PROJ, false, false, WS>(sv, gv, pa, da, j, i0h, p.T, recs, tabs, fwtab, tstride,
-                                                        Kf, p.fwm_inv_h, p.scale, p.fwm_hl, p.fwm_b0l);
+            kv_chunk<CAL, REC, FULLG, PROJ, false, false, doDV, doDK, W>(sv, gv, pa, da, j, i0h, p.T, recs, tabs, fwtab, tstride,
+                                                       Kf, p.fwm_inv_h, p.scale, p.fwm_hl, p.fwm_b0l);
           // optional side outputs: per-query-row sums of dS and |dS| over this warp's 32 keys
           if constexpr (RS) {
-            if (doDK) rowsum_add(da, p.dsum_out, p.dabs_out, (size_t)bh * p.T + i0h, min(WS, p.T - i0h));
+            if (doDK) rowsum_add(da, p.dsum_out, p.dabs_out, (size_t)bh * p.T + i0h, min(W, p.T - i0h));
           }
-          if (p.x3) {
+        }
+        if (p.x3) {
 #pragma unroll
-            for (int q = 0; q < WS; ++q) {
-              const float x = doDV ? pa[q] : da[q];
-              const float hh = tf32_rna(x);
-              pa[q] = hh;
-              da[q] = __fsub_rn(x, hh);
-            }
-            tmem_stw<WS>(lane_addr(tmem, cS), pa);
-            tmem_stw<WS>(lane_addr(tmem, cG), da);
-          } else {
-            if (doDV) tmem_stw<WS>(lane_addr(tmem, cS), pa);
-            if (doDK) tmem_stw<WS>(lane_addr(tmem, cG), da);
+          for (int q = 0; q < W; ++q) {
+            const float x = doDV ? pa[q] : da[q];
+            const float hh = tf32_rna(x);
+            pa[q] = hh;
+            da[q] = __fsub_rn(x, hh);
           }
+          tmem_stw<W>(lane_addr(tmem, cS), pa);
+          tmem_stw<W>(lane_addr(tmem, cG), da);
+        } else {
+          if (doDV) tmem_stw<W>(lane_addr(tmem, cS), pa);
+          if (doDK) tmem_stw<W>(lane_addr(tmem, cG), da);
         }
         __syncwarp();
         if ((tid & 31) == 0) mbar_arrive(&bar_emptyA[s]);  // the stage's records are read
@@ -523,7 +598,7 @@ __global__ void __launch_bounds__(NTHR, 1) k_bwd_dkdv(const __grid_constant__ Ma
       // the next item's K / V (this item's S^T, g^T have all been read: the last tile's were)
       if (!failed && snake_item(n + 1) < p.nitems) ops_to_tmem(n + 1);
       const bool dok = !failed && mbar_wait(bar_done, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_MMA);
-      failed = group_any(BAR_COMPUTE, NCOMP, !dok);
+      failed = group_any(BAR_COMPUTE, NCOMP_KV, !dok);
       if (!failed) {
         tc_fence_after();
         // dV, dK rows into swizzled tiles for TMA stores: in the K / V staging area (free now
@@ -538,32 +613,32 @@ __global__ void __launch_bounds__(NTHR, 1) k_bwd_dkdv(const __grid_constant__ Ma
           const int col = pass == 0 ? cdV : cdK;
           const float mul = pass == 0 ? 1.0f : p.scale;
           float* out = (pass == 0 ? p.dV : p.dK) + ((size_t)bh * p.T + j) * D;
-          for (int c = cg * (D / NCG); c < (cg + 1) * (D / NCG); c += 32) {
-            float v[32];
-            tmem_ld32(lane_addr(tmem, col + c), v);
+          for (int c = cg * (D / NCG_KV); c < (cg + 1) * (D / NCG_KV); c += 16) {
+            float v[16];
+            tmem_ld16(lane_addr(tmem, col + c), v);
             if (p.x3) {
-              float w[32];
-              tmem_ld32(lane_addr(tmem, cdC + c), w);
+              float w[16];
+              tmem_ld16(lane_addr(tmem, cdC + c), w);
               tmem_ld_wait();
 #pragma unroll
-              for (int q = 0; q < 32; ++q) v[q] += w[q];
+              for (int q = 0; q < 16; ++q) v[q] += w[q];
             }
             tmem_ld_wait();
 #pragma unroll
-            for (int q = 0; q < 32; ++q) v[q] *= mul;
+            for (int q = 0; q < 16; ++q) v[q] *= mul;
             if (p.ops_smem) {
-              row_to_staged(stg + pass * 128 * D * 4, row, c / 32, v);
+              row16_to_staged(stg + pass * 128 * D * 4, row, c, v);
             } else if (j < p.T) {
               float4* dst = reinterpret_cast<float4*>(out + c);
 #pragma unroll
-              for (int q = 0; q < 8; ++q) dst[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+              for (int q = 0; q < 4; ++q) dst[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
             }
           }
         }
         if (p.ops_smem) {
           fence_async_smem();
           if (last) {
-            group_sync(BAR_COMPUTE, NCOMP);
+            group_sync(BAR_COMPUTE, NCOMP_KV);
             if (warp == 0 && doDV) store_rows_tile_boxed(stg, &maps.dv, D, 64, kb * 128, bh, false);
             if (warp == 1 && doDK) store_rows_tile_boxed(stg + 128 * D * 4, &maps.dk, D, 64, kb * 128, bh, false);
           } else {
@@ -580,39 +655,45 @@ __global__ void __launch_bounds__(NTHR, 1) k_bwd_dkdv(const __grid_constant__ Ma
   if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
-// Every backward mode of one calibration and reconstruction; softmax ignores the mode.
-template <int CAL, int REC, bool RS>
+// Every backward mode of one calibration and reconstruction; softmax ignores the mode, and a dV
+// launch does not depend on it.
+template <int CAL, int REC, bool RS, int SEL>
 cudaError_t launch_dkdv_modes(dim3 grid, const Maps& maps, const Params& p, int smem_bytes, cudaStream_t s) {
-  if constexpr (CAL == CAL_SOFTMAX) {
-    return launch3(k_bwd_dkdv<CAL_SOFTMAX, REC_LERP, false, false, RS>, grid, maps, p, smem_bytes, s);
+  if constexpr (CAL == CAL_SOFTMAX || SEL == DKV_DV) {
+    return launch3(k_bwd_dkdv<CAL, REC, false, false, RS, SEL>, grid, maps, p, smem_bytes, s, NTHR_KV);
   } else {
     const bool proj = p.grad == GRAD_DETACH_PROJ, full = p.grad != GRAD_DETACH && !proj;
-    return full ? launch3(k_bwd_dkdv<CAL, REC, true, false, RS>, grid, maps, p, smem_bytes, s)
-           : proj ? launch3(k_bwd_dkdv<CAL, REC, false, true, RS>, grid, maps, p, smem_bytes, s)
-                  : launch3(k_bwd_dkdv<CAL, REC, false, false, RS>, grid, maps, p, smem_bytes, s);
+    return full ? launch3(k_bwd_dkdv<CAL, REC, true, false, RS, SEL>, grid, maps, p, smem_bytes, s, NTHR_KV)
+           : proj ? launch3(k_bwd_dkdv<CAL, REC, false, true, RS, SEL>, grid, maps, p, smem_bytes, s, NTHR_KV)
+                  : launch3(k_bwd_dkdv<CAL, REC, false, false, RS, SEL>, grid, maps, p, smem_bytes, s, NTHR_KV);
   }
 }
 
-// The dK/dV launch of p's configuration; RS: the instantiation that also accumulates the
-// per-row sums of dS and |dS| (p.dsum_out, p.dabs_out).
-template <bool RS>
+// The dK/dV launch of p's configuration.  RS: the instantiation that also accumulates the
+// per-row sums of dS and |dS| (p.dsum_out, p.dabs_out); SEL: its products (DkvSel).
+template <bool RS, int SEL>
 cudaError_t launch_bwd_dkdv_t(const Maps& maps, const Params& p, int smem_bytes, cudaStream_t s) {
   const dim3 grid((unsigned)p.ngrid);
   const bool near = p.recon == REC_NEAREST;
   switch (p.calib) {
-    case CAL_SOFTMAX: return launch_dkdv_modes<CAL_SOFTMAX, REC_LERP, RS>(grid, maps, p, smem_bytes, s);
-    case CAL_EXP8: return launch_dkdv_modes<CAL_EXP8, REC_LERP, RS>(grid, maps, p, smem_bytes, s);
-    case CAL_EXPB: return launch_dkdv_modes<CAL_EXPB, REC_LERP, RS>(grid, maps, p, smem_bytes, s);
+    case CAL_SOFTMAX: return launch_dkdv_modes<CAL_SOFTMAX, REC_LERP, RS, SEL>(grid, maps, p, smem_bytes, s);
+    case CAL_EXP8: return launch_dkdv_modes<CAL_EXP8, REC_LERP, RS, SEL>(grid, maps, p, smem_bytes, s);
+    case CAL_EXPB: return launch_dkdv_modes<CAL_EXPB, REC_LERP, RS, SEL>(grid, maps, p, smem_bytes, s);
     case CAL_MINMAX:
-      return near ? launch_dkdv_modes<CAL_MINMAX, REC_NEAREST, RS>(grid, maps, p, smem_bytes, s)
-                  : launch_dkdv_modes<CAL_MINMAX, REC_LERP, RS>(grid, maps, p, smem_bytes, s);
+      return near ? launch_dkdv_modes<CAL_MINMAX, REC_NEAREST, RS, SEL>(grid, maps, p, smem_bytes, s)
+                  : launch_dkdv_modes<CAL_MINMAX, REC_LERP, RS, SEL>(grid, maps, p, smem_bytes, s);
     case CAL_FWMR:
-      return near ? launch_dkdv_modes<CAL_FWMR, REC_NEAREST, RS>(grid, maps, p, smem_bytes, s)
-                  : launch_dkdv_modes<CAL_FWMR, REC_LERP, RS>(grid, maps, p, smem_bytes, s);
+      return near ? launch_dkdv_modes<CAL_FWMR, REC_NEAREST, RS, SEL>(grid, maps, p, smem_bytes, s)
+                  : launch_dkdv_modes<CAL_FWMR, REC_LERP, RS, SEL>(grid, maps, p, smem_bytes, s);
     default:
-      return near ? launch_dkdv_modes<CAL_FWM, REC_NEAREST, RS>(grid, maps, p, smem_bytes, s)
-                  : launch_dkdv_modes<CAL_FWM, REC_LERP, RS>(grid, maps, p, smem_bytes, s);
+      return near ? launch_dkdv_modes<CAL_FWM, REC_NEAREST, RS, SEL>(grid, maps, p, smem_bytes, s)
+                  : launch_dkdv_modes<CAL_FWM, REC_LERP, RS, SEL>(grid, maps, p, smem_bytes, s);
   }
 }
+extern template cudaError_t launch_bwd_dkdv_t<false, DKV_BOTH>(const Maps&, const Params&, int, cudaStream_t);
+extern template cudaError_t launch_bwd_dkdv_t<false, DKV_DV>(const Maps&, const Params&, int, cudaStream_t);
+extern template cudaError_t launch_bwd_dkdv_t<false, DKV_DK>(const Maps&, const Params&, int, cudaStream_t);
+extern template cudaError_t launch_bwd_dkdv_t<true, DKV_BOTH>(const Maps&, const Params&, int, cudaStream_t);
+extern template cudaError_t launch_bwd_dkdv_t<true, DKV_DK>(const Maps&, const Params&, int, cudaStream_t);
 
 }  // namespace kint

@@ -241,35 +241,6 @@ __device__ __forceinline__ bool main_issue_s(const Params& p, RingPos stg, int b
   return true;
 }
 
-// 16 columns [c0, c0 + 16) of the calling thread's row into a 128-row staging tile laid out
-// as TMA reads it (128-byte swizzle, 32-column panels).
-__device__ __forceinline__ void row16_to_staged(uint8_t* tile, int row, int c0, const float (&v)[16]) {
-  const uint32_t base = smem_u32(tile) + (uint32_t)(c0 >> 5) * 128u * SW + (uint32_t)row * SW;
-  const int ch0 = (c0 & 31) >> 2;
-#pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    const uint32_t a = base + (uint32_t)(((ch0 + c) ^ (row & 7)) << 4);
-    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v[4 * c]), "f"(v[4 * c + 1]),
-                 "f"(v[4 * c + 2]), "f"(v[4 * c + 3])
-                 : "memory");
-  }
-}
-// The same columns of a 128-row tile that TMA loaded, into the thread's TMEM lane at `col`.
-__device__ __forceinline__ void staged16_to_tmem(uint32_t tmem_base, int col, const uint8_t* tile, int row, int c0) {
-  const uint32_t base = smem_u32(tile) + (uint32_t)(c0 >> 5) * 128u * SW + (uint32_t)row * SW;
-  const int ch0 = (c0 & 31) >> 2;
-  float v[16];
-#pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    const float4 x = lds_f4(base + (uint32_t)(((ch0 + c) ^ (row & 7)) << 4));
-    v[4 * c] = x.x;
-    v[4 * c + 1] = x.y;
-    v[4 * c + 2] = x.z;
-    v[4 * c + 3] = x.w;
-  }
-  tmem_st16(lane_addr(tmem_base, col + c0), v);
-}
-
 template <int CAL, int REC, int MODE, bool X3, int NG>
 __global__ void __launch_bounds__(MainT<NG>::NTHR, MainT<NG>::CTAS) k_fwd_main(const __grid_constant__ Maps maps, const Params p,
                                                       const __grid_constant__ Sched sch) {

@@ -127,6 +127,7 @@ __device__ __forceinline__ void add_tied_keys(uint32_t mask, float* acc, const f
 
 // MMA thread of k_bwd_dq: wait for key tile kt, then S_b = Q K^T and g_b = dO V^T
 // into score buffer b = kt % nbuf.
+template <int BK>
 __device__ __forceinline__ bool dq_issue_sg(const Params& p, RingPos stg, int b, uint64_t* bar_full,
                                             uint64_t* bar_sfull, const uint8_t* st0, uint32_t cQa, uint32_t cdOa,
                                             uint32_t cSG, int ktile) {
@@ -135,17 +136,17 @@ __device__ __forceinline__ bool dq_issue_sg(const Params& p, RingPos stg, int b,
   tc_fence_after();
   const uint8_t* sk = st0 + s * p.sm_stage_bytes;
   const uint8_t* sv = sk + parts * ktile;
-  const uint32_t cS = cSG + 128 * b, cG = cS + 64;
+  const uint32_t cS = cSG + 2 * BK * b, cG = cS + BK;
   if (p.x3) {
-    mma_tmem_smem(cS, cQa + D, sk, BT, D, false);     // Q_lo K_hi
-    mma_tmem_smem(cS, cQa, sk + ktile, BT, D, true);  // Q_hi K_lo
-    mma_tmem_smem(cS, cQa, sk, BT, D, true);          // Q_hi K_hi
-    mma_tmem_smem(cG, cdOa + D, sv, BT, D, false);
-    mma_tmem_smem(cG, cdOa, sv + ktile, BT, D, true);
-    mma_tmem_smem(cG, cdOa, sv, BT, D, true);
+    mma_tmem_smem(cS, cQa + D, sk, BK, D, false);     // Q_lo K_hi
+    mma_tmem_smem(cS, cQa, sk + ktile, BK, D, true);  // Q_hi K_lo
+    mma_tmem_smem(cS, cQa, sk, BK, D, true);          // Q_hi K_hi
+    mma_tmem_smem(cG, cdOa + D, sv, BK, D, false);
+    mma_tmem_smem(cG, cdOa, sv + ktile, BK, D, true);
+    mma_tmem_smem(cG, cdOa, sv, BK, D, true);
   } else {
-    mma_tmem_smem(cS, cQa, sk, BT, D, false);
-    mma_tmem_smem(cG, cdOa, sv, BT, D, false);
+    mma_tmem_smem(cS, cQa, sk, BK, D, false);
+    mma_tmem_smem(cG, cdOa, sv, BK, D, false);
   }
   mma_commit(&bar_sfull[b]);
   return true;
@@ -153,11 +154,19 @@ __device__ __forceinline__ bool dq_issue_sg(const Params& p, RingPos stg, int b,
 
 // ---------------------------------------------------------------------------
 // k_bwd_dq.
+// BK: keys per tile.  64 at d = 64 in TF32: a thread takes half of a tile's columns of its row.  32
+// at d = 128 and under 3xTF32, where Q, dO and dQ leave 128 TMEM columns, one pair of
+// 64-key score buffers or two of 32: with one, products and element work took turns; with
+// two, the groups of four compute warps take the tiles in turn, under each other's
+// products (a thread takes all of a tile's columns, every other tile: the same keys in the
+// same order as half of every 64-key tile, so the row sums keep their bits).  (Against 64-key tiles and one
+// buffer: B=4 H=16 T=2048 d=128 303 -> 272 us, H=16 T=16384 d=128 MinMax 4730 -> 4137, 3xTF32
+// B=8 H=12 T=1024 172 -> 158.)
 // TMEM: Q [0, dp), dO [dp, 2dp) (dp = d, or 2d for 3xTF32 hi|lo; loaded by the
-// compute threads), then per score buffer b: S_b at 2dp + 128 b (64 columns), g_b
-// right after it (64 columns); dQ at 2dp + 128 nbuf.  dS overwrites S_b (its tf32
+// compute threads), then per score buffer b: S_b at 2dp + 2 BK b (BK columns), g_b
+// right after it (BK columns); dQ at 2dp + 2 BK nbuf.  dS overwrites S_b (its tf32
 // lo part, under 3xTF32, overwrites g_b).
-// smem: stages {K [64 x d], V [64 x d], K^T [d x 64]} (hi[, lo] each) at
+// smem: stages {K [BK x d], V [BK x d], K^T [d x BK]} (hi[, lo] each) at
 // sm_stage0; the grid pair table at sm_table; exchange words at sm_rows.
 // ---------------------------------------------------------------------------
 // Producer warp of k_bwd_dq: TMA-stores the dQ tile of its k-th item, which the compute
@@ -171,7 +180,7 @@ __device__ __forceinline__ bool store_staged_dq(const Maps& maps, const Params& 
   return true;
 }
 
-template <int CAL, bool FULLG>
+template <int CAL, bool FULLG, int BK>
 __global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ Maps maps, const Params p) {
   uint8_t* sm = smem_base();
   if (p.gate != nullptr) {
@@ -181,7 +190,8 @@ __global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ M
     if (gated_off(p)) return;
   }
   const int D = p.d, Kq = p.Kint, parts = p.x3 ? 2 : 1, NS = p.nstage, nbuf = p.nbuf;
-  const int ktile = BT * D * 4;
+  const int ktile = BK * D * 4;
+  constexpr int NGRP = 64 / BK, NWT = NCOMP / 32 / NGRP;  // groups of compute warps taking tiles in turn; warps per tile
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm + p.sm_bars);
   uint64_t* bar_full = bars;               // [NS]
   uint64_t* bar_empty = bars + NS;         // [NS]
@@ -200,19 +210,19 @@ __global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ M
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 3 * NS + 11);
   float* xch = reinterpret_cast<float*>(sm + p.sm_rows);  // [8][128]
   const int tid = threadIdx.x, warp = warp_id_uniform();
-  constexpr int W = BT / NCG;  // key columns per thread per tile
+  constexpr int W = 32;  // key columns per thread per tile
   const int dp = D * parts;
-  const int cQ = 0, cdO = dp, cSG0 = 2 * dp, cdQ = cSG0 + 128 * nbuf;
+  const int cQ = 0, cdO = dp, cSG0 = 2 * dp, cdQ = cSG0 + 2 * BK * nbuf;
 
   if (tid == 0) {
     for (int s = 0; s < NS; ++s) {
       mbar_init(&bar_full[s], 1);
       mbar_init(&bar_empty[s], 1);
-      mbar_init(&bar_emptyA[s], NCOMP / 32);
+      mbar_init(&bar_emptyA[s], NWT);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&bar_sfull[b], 1);
-      mbar_init(&bar_pready[b], NCOMP / 32);
+      mbar_init(&bar_pready[b], NWT);
       mbar_init(&bar_dqdone[b], 1);
     }
     mbar_init(bar_done, 1);
@@ -252,7 +262,7 @@ __global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ M
     if (p.ops_smem && snake_item(0) < p.nitems) stage_ops(0);
     for (int item = snake_item(n); item < p.nitems && ok; item = snake_item(++n)) {
       const int qb = p.nqb - 1 - item / p.BH, bh = item % p.BH;
-      const int nkt = min(2 * qb + 2, (p.T + BT - 1) / BT);
+      const int nkt = min((128 / BK) * (qb + 1), (p.T + BK - 1) / BK);
       for (int kt = 0; kt < nkt; ++kt, ++gt, ld.next(NS)) {
         const int s = ld.i;
         if (gt >= NS && !mbar_wait_warp(&bar_emptyA[s], ld.ph ^ 1u, p.wait_ns, p.status, DEV_ERR_TIMEOUT_SYNC)) {
@@ -262,18 +272,18 @@ __global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ M
         uint8_t* dst = sm + p.sm_stage0 + s * p.sm_stage_bytes;
         uint64_t* b = &bar_full[s];
         mbar_arrive_expect_tx(b, 3 * parts * ktile);
-        load_rows_tile(dst, &maps.k, b, D, BT, 0, kt * BT, bh);
-        load_rows_tile(dst + parts * ktile, &maps.v, b, D, BT, 0, kt * BT, bh);
+        load_rows_tile(dst, &maps.k, b, D, BK, 0, kt * BK, bh);
+        load_rows_tile(dst + parts * ktile, &maps.v, b, D, BK, 0, kt * BK, bh);
         if (p.x3) {
-          load_rows_tile(dst + ktile, &maps.k_lo, b, D, BT, 0, kt * BT, bh);
-          load_rows_tile(dst + parts * ktile + ktile, &maps.v_lo, b, D, BT, 0, kt * BT, bh);
+          load_rows_tile(dst + ktile, &maps.k_lo, b, D, BK, 0, kt * BK, bh);
+          load_rows_tile(dst + parts * ktile + ktile, &maps.v_lo, b, D, BK, 0, kt * BK, bh);
         }
         if (gt >= NS && !mbar_wait_warp(&bar_empty[s], ld.ph ^ 1u, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA)) {
           ok = false;
           break;
         }
-        load_rows_tile(dst + 2 * parts * ktile, &maps.kt, b, BT, D, kt * BT, 0, bh);
-        if (p.x3) load_rows_tile(dst + 2 * parts * ktile + ktile, &maps.kt_lo, b, BT, D, kt * BT, 0, bh);
+        load_rows_tile(dst + 2 * parts * ktile, &maps.kt, b, BK, D, kt * BK, 0, bh);
+        if (p.x3) load_rows_tile(dst + 2 * parts * ktile + ktile, &maps.kt_lo, b, BK, D, kt * BK, 0, bh);
         // The next item's Q / dO, as soon as the stage ring holds this item's first tiles: it needs
         // this item's Q / dO copied out into TMEM and the previous item's dQ tile, staged in the
         // same area since, stored; both happen at the end of the previous item, so the load has
@@ -304,7 +314,7 @@ __global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ M
     bool ok = true;
     for (int item = snake_item(n); item < p.nitems && ok; item = snake_item(++n)) {
       const int qb = p.nqb - 1 - item / p.BH;
-      const int nkt = min(2 * qb + 2, (p.T + BT - 1) / BT);
+      const int nkt = min((128 / BK) * (qb + 1), (p.T + BK - 1) / BK);
       // Q / dO of the item in TMEM (copied by the compute warps once the previous item's
       // last S, g were read)
       ok = mbar_wait_warp(bar_ops, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_SYNC);
@@ -315,7 +325,7 @@ __global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ M
           ok = false;
           break;
         }
-        ok = dq_issue_sg(p, is, ib.i, bar_full, bar_sfull, st0, cQa, cdOa, cSG, ktile);
+        ok = dq_issue_sg<BK>(p, is, ib.i, bar_full, bar_sfull, st0, cQa, cdOa, cSG, ktile);
       }
     }
     drain_mma(bar_drain, p.wait_ns, p.status);  // clean-up: no product still writes TMEM
@@ -326,7 +336,7 @@ __global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ M
     bool ok = true;
     for (int item = snake_item(n); item < p.nitems && ok; item = snake_item(++n)) {
       const int qb = p.nqb - 1 - item / p.BH;
-      const int nkt = min(2 * qb + 2, (p.T + BT - 1) / BT);
+      const int nkt = min((128 / BK) * (qb + 1), (p.T + BK - 1) / BK);
       for (int kt = 0; kt < nkt && ok; ++kt, cs.next(NS), cb.next(nbuf)) {
         const int b = cb.i, s = cs.i;
         if (!mbar_wait_warp(&bar_pready[b], cb.ph, p.wait_ns, p.status, DEV_ERR_TIMEOUT_SYNC)) {
@@ -335,14 +345,14 @@ __global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ M
         }
         tc_fence_after();
         const uint8_t* skt = sm + p.sm_stage0 + s * p.sm_stage_bytes + 2 * parts * ktile;
-        const uint32_t cS = tmem + cSG0 + 128 * b, cG = cS + 64;
+        const uint32_t cS = tmem + cSG0 + 2 * BK * b, cG = cS + BK;
         const bool acc = kt > 0;
         if (p.x3) {
-          mma_tmem_smem(tmem + cdQ, cS, skt, D, BT, acc);           // dS_hi K_hi
-          mma_tmem_smem(tmem + cdQ, cS, skt + ktile, D, BT, true);  // dS_hi K_lo
-          mma_tmem_smem(tmem + cdQ, cG, skt, D, BT, true);          // dS_lo K_hi
+          mma_tmem_tile<BK>(tmem + cdQ, cS, skt, D, acc);           // dS_hi K_hi
+          mma_tmem_tile<BK>(tmem + cdQ, cS, skt + ktile, D, true);  // dS_hi K_lo
+          mma_tmem_tile<BK>(tmem + cdQ, cG, skt, D, true);          // dS_lo K_hi
         } else {
-          mma_tmem_smem(tmem + cdQ, cS, skt, D, BT, acc);
+          mma_tmem_tile<BK>(tmem + cdQ, cS, skt, D, acc);
         }
         mma_commit(&bar_empty[s]);
         mma_commit(&bar_dqdone[b]);
@@ -353,6 +363,7 @@ __global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ M
   } else {
     // ---- compute warps: items one after the other ----
     const int row = tid & 127, cg = (tid >> 7) & (NCG - 1);
+    int gt = 0;  // tiles so far
     // Operand rows of the n-th item into TMEM (column group 0 takes Q, group 1 takes dO),
     // handed to the MMA warp through bar_ops.  TF32 at d = 64: from the tiles the producer
     // staged in smem; otherwise from global rows.  The next item's rows go in as soon as
@@ -427,7 +438,7 @@ __global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ M
     for (int item = snake_item(n); item < p.nitems && !failed; item = snake_item(++n)) {
       // ---- set-up: row constants, grid table (the operands are in TMEM already) ----
       const int qb = p.nqb - 1 - item / p.BH, bh = item % p.BH;
-      const int nkt = min(2 * qb + 2, (p.T + BT - 1) / BT);
+      const int nkt = min((128 / BK) * (qb + 1), (p.T + BK - 1) / BK);
       const int i = qb * 128 + row;
       const bool row_ok = i < p.T;
       const size_t rw = (size_t)bh * p.T + (row_ok ? i : 0);
@@ -472,7 +483,9 @@ __global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ M
       // the grid table, and the zeroed tie sums (every column group of a row may add to them)
       group_sync(BAR_COMPUTE, NCOMP);
       float own = 0.f, cm = 0.f;
-      for (int kt = 0; kt < nkt; ++kt, cb.next(nbuf)) {
+      const int i0w = qb * 128 + (warp & 3) * 32;  // this warp's first row
+      for (int kt = 0; kt < nkt; ++kt, cb.next(nbuf), cs.next(NS), ++gt) {
+        if (NGRP == 2 && (gt & 1) != cg) continue;
         const int b = cb.i;
         const bool ok = mbar_wait(&bar_sfull[b], cb.ph, p.wait_ns, p.status, DEV_ERR_TIMEOUT_MMA);
         if (!ok) {
@@ -481,20 +494,23 @@ __global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ M
         }
         // S, g of the tile completed: its K and V may be reloaded
         if ((tid & 31) == 0) mbar_arrive(&bar_emptyA[cs.i]);
-        cs.next(NS);
         tc_fence_after();
-        const int cS = cSG0 + 128 * b + cg * W, cG = cS + 64;
+        const int cS = cSG0 + 2 * BK * b + (NGRP == 2 ? 0 : cg * W), cG = cS + BK;
         float sv[W], gv[W], out[W];
         tmem_ldw<W>(lane_addr(tmem, cS), sv);
         tmem_ldw<W>(lane_addr(tmem, cG), gv);
         tmem_ld_wait();
-        const int j0 = kt * BT + cg * W;
-        if (j0 + W - 1 > qb * 128)
+        const int j0 = kt * BK + (NGRP == 2 ? 0 : cg * W);
+        if (BK == 32 && j0 > i0w + 31) {  // every key lies after every row of the warp
+#pragma unroll
+          for (int q = 0; q < W; ++q) out[q] = 0.f;
+        } else if (j0 + W - 1 > (BK == 32 ? i0w : qb * 128)) {
           dq_chunk<CAL, FULLG, true, W>(sv, gv, out, j0, i, k1q, c0q, g.inv_h, ga, gb, g.nogrid, Kf, fk, tab, sk1,
                                         sc0, invWf, g.hl, g.b0l, own, cm);
-        else
+        } else {
           dq_chunk<CAL, FULLG, false, W>(sv, gv, out, j0, i, k1q, c0q, g.inv_h, ga, gb, g.nogrid, Kf, fk, tab,
                                          sk1, sc0, invWf, g.hl, g.b0l, own, cm);
+        }
         if (__any_sync(0xffffffffu, track)) {
           // rare: tied extrema, the tie set is found by equality on the recomputed scores
           uint32_t mk_max = 0, mk_min = 0;
@@ -526,6 +542,11 @@ __global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ M
       }
       // the next item's Q / dO (this item's S, g have all been read: the last tile's were)
       // and its row statistics
+      // (a group has seen its own last tile's S, g, and waits for the other group's here: products
+      // complete in order, so the barrier's phase before is over)
+      if (NGRP == 2 && !failed && ((gt - 1) & 1) != cg)
+        failed = !mbar_wait(&bar_sfull[(gt - 1) & 1], (uint32_t)((gt - 1) >> 1) & 1u, p.wait_ns, p.status,
+                            DEV_ERR_TIMEOUT_MMA);
       if (!failed && snake_item(n + 1) < p.nitems) {
         ops_to_tmem(n + 1);
         nx = load_row_stats(n + 1);
@@ -705,24 +726,29 @@ cudaError_t launch_kcum(const float* K, float* C, int BH, int T, int d, cudaStre
   return launch_pdl(k_kcum, dim3((unsigned)(BH * (d / 32))), dim3(KCUM_WARPS * 32), 0, s, K, C, T, d);
 }
 
-cudaError_t launch_bwd_dq(const Maps& maps, const Params& p, int smem_bytes, cudaStream_t s) {
+template <int BK>
+static cudaError_t launch_dq_bk(const Maps& maps, const Params& p, int smem_bytes, cudaStream_t s) {
   const dim3 grid((unsigned)p.ngrid);
   const bool full = p.grad != GRAD_DETACH && p.grad != GRAD_DETACH_PROJ;
-  if (p.calib == CAL_SOFTMAX) return launch3(k_bwd_dq<CAL_SOFTMAX, false>, grid, maps, p, smem_bytes, s, NTHR_DQ);
+  if (p.calib == CAL_SOFTMAX) return launch3(k_bwd_dq<CAL_SOFTMAX, false, BK>, grid, maps, p, smem_bytes, s, NTHR_DQ);
   if (p.calib == CAL_EXP8)
-    return full ? launch3(k_bwd_dq<CAL_EXP8, true>, grid, maps, p, smem_bytes, s, NTHR_DQ)
-                : launch3(k_bwd_dq<CAL_EXP8, false>, grid, maps, p, smem_bytes, s, NTHR_DQ);
+    return full ? launch3(k_bwd_dq<CAL_EXP8, true, BK>, grid, maps, p, smem_bytes, s, NTHR_DQ)
+                : launch3(k_bwd_dq<CAL_EXP8, false, BK>, grid, maps, p, smem_bytes, s, NTHR_DQ);
   if (p.calib == CAL_EXPB)
-    return full ? launch3(k_bwd_dq<CAL_EXPB, true>, grid, maps, p, smem_bytes, s, NTHR_DQ)
-                : launch3(k_bwd_dq<CAL_EXPB, false>, grid, maps, p, smem_bytes, s, NTHR_DQ);
+    return full ? launch3(k_bwd_dq<CAL_EXPB, true, BK>, grid, maps, p, smem_bytes, s, NTHR_DQ)
+                : launch3(k_bwd_dq<CAL_EXPB, false, BK>, grid, maps, p, smem_bytes, s, NTHR_DQ);
   if (p.calib == CAL_MINMAX)
-    return full ? launch3(k_bwd_dq<CAL_MINMAX, true>, grid, maps, p, smem_bytes, s, NTHR_DQ)
-                : launch3(k_bwd_dq<CAL_MINMAX, false>, grid, maps, p, smem_bytes, s, NTHR_DQ);
+    return full ? launch3(k_bwd_dq<CAL_MINMAX, true, BK>, grid, maps, p, smem_bytes, s, NTHR_DQ)
+                : launch3(k_bwd_dq<CAL_MINMAX, false, BK>, grid, maps, p, smem_bytes, s, NTHR_DQ);
   if (p.calib == CAL_FWMR)
-    return full ? launch3(k_bwd_dq<CAL_FWMR, true>, grid, maps, p, smem_bytes, s, NTHR_DQ)
-                : launch3(k_bwd_dq<CAL_FWMR, false>, grid, maps, p, smem_bytes, s, NTHR_DQ);
-  return full ? launch3(k_bwd_dq<CAL_FWM, true>, grid, maps, p, smem_bytes, s, NTHR_DQ)
-              : launch3(k_bwd_dq<CAL_FWM, false>, grid, maps, p, smem_bytes, s, NTHR_DQ);
+    return full ? launch3(k_bwd_dq<CAL_FWMR, true, BK>, grid, maps, p, smem_bytes, s, NTHR_DQ)
+                : launch3(k_bwd_dq<CAL_FWMR, false, BK>, grid, maps, p, smem_bytes, s, NTHR_DQ);
+  return full ? launch3(k_bwd_dq<CAL_FWM, true, BK>, grid, maps, p, smem_bytes, s, NTHR_DQ)
+              : launch3(k_bwd_dq<CAL_FWM, false, BK>, grid, maps, p, smem_bytes, s, NTHR_DQ);
+}
+
+cudaError_t launch_bwd_dq(const Maps& maps, const Params& p, int smem_bytes, cudaStream_t s) {
+  return p.bk == 32 ? launch_dq_bk<32>(maps, p, smem_bytes, s) : launch_dq_bk<64>(maps, p, smem_bytes, s);
 }
 
 }  // namespace kint

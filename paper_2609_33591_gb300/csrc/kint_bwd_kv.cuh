@@ -6,8 +6,9 @@
 
 namespace kint {
 
-// Thread roles: sixteen compute warps (thread t owns key kb*128 + t%128 and the 16 query columns
-// 16 (t/128) .. + 15 of each 64-query tile), the MMA warp, the producer warp and two idle
+// Thread roles: sixteen compute warps (thread t owns key kb*128 + t%128 and 16 query columns:
+// 16 (t/128) .. + 15 of each 64-query tile, or, with 32-query tiles, 16 (t/128 % 2) .. + 15 of
+// every other tile, the two groups of eight warps taking the tiles in turn), the MMA warp, the producer warp and two idle
 // warps.  The fifth warpgroup gives registers to the compute warpgroups: launched at 96 per
 // thread, it keeps 64 and they take 104.
 constexpr int NCG_KV = 4, NCOMP_KV = 128 * NCG_KV, NTHR_KV = NCOMP_KV + 128;
@@ -165,39 +166,42 @@ __device__ __forceinline__ void rowsum_add(const float (&v)[16], float* dsum, fl
 }
 
 // MMA warp of k_bwd_dkdv: the products of the query tile in stage s (landed) into score buffer b.
+template <int BQ>
 __device__ __forceinline__ void kv_issue_s(const Params& p, const uint8_t* st, int b, uint32_t cKa, uint32_t cSG,
                                            int qtile) {
   const int D = p.d;
-  const uint32_t cS = cSG + 128 * b;
+  const uint32_t cS = cSG + 2 * BQ * b;
   if (p.x3) {
-    mma_tmem_smem(cS, cKa + D, st, BT, D, false);
-    mma_tmem_smem(cS, cKa, st + qtile, BT, D, true);
-    mma_tmem_smem(cS, cKa, st, BT, D, true);
+    mma_tmem_smem(cS, cKa + D, st, BQ, D, false);
+    mma_tmem_smem(cS, cKa, st + qtile, BQ, D, true);
+    mma_tmem_smem(cS, cKa, st, BQ, D, true);
   } else {
-    mma_tmem_smem(cS, cKa, st, BT, D, false);
+    mma_tmem_smem(cS, cKa, st, BQ, D, false);
   }
 }
+template <int BQ>
 __device__ __forceinline__ void kv_issue_g(const Params& p, const uint8_t* st, int b, uint32_t cVa, uint32_t cSG,
                                            int qtile, int odO) {
   const int D = p.d;
-  const uint32_t cG = cSG + 128 * b + 64;
+  const uint32_t cG = cSG + 2 * BQ * b + BQ;
   if (p.x3) {
-    mma_tmem_smem(cG, cVa + D, st + odO, BT, D, false);
-    mma_tmem_smem(cG, cVa, st + odO + qtile, BT, D, true);
-    mma_tmem_smem(cG, cVa, st + odO, BT, D, true);
+    mma_tmem_smem(cG, cVa + D, st + odO, BQ, D, false);
+    mma_tmem_smem(cG, cVa, st + odO + qtile, BQ, D, true);
+    mma_tmem_smem(cG, cVa, st + odO, BQ, D, true);
   } else {
-    mma_tmem_smem(cG, cVa, st + odO, BT, D, false);
+    mma_tmem_smem(cG, cVa, st + odO, BQ, D, false);
   }
 }
 // Both (S^T_b = K Q^T and, with V, g^T_b = V dO^T) once the tile in stage stg has landed.
+template <int BQ>
 __device__ __forceinline__ bool kv_issue_sg(const Params& p, RingPos stg, int b, uint64_t* bar_full,
                                             uint64_t* bar_sfull, const uint8_t* st0, uint32_t cKa, uint32_t cVa,
                                             uint32_t cSG, int qtile, bool needV, int odO) {
   if (!mbar_wait_warp(&bar_full[stg.i], stg.ph, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA)) return false;
   tc_fence_after();
   const uint8_t* st = st0 + stg.i * p.sm_stage_bytes;
-  kv_issue_s(p, st, b, cKa, cSG, qtile);
-  if (needV) kv_issue_g(p, st, b, cVa, cSG, qtile, odO);
+  kv_issue_s<BQ>(p, st, b, cKa, cSG, qtile);
+  if (needV) kv_issue_g<BQ>(p, st, b, cVa, cSG, qtile, odO);
   mma_commit(&bar_sfull[b]);
   return true;
 }
@@ -226,12 +230,12 @@ __device__ __forceinline__ bool store_staged_dkdv(const Maps& maps, const Params
 // What bounds it: the issue of the products by one warp and, at one score buffer, the chain
 // products -> element work -> products; shared-memory loads of the row records come next.
 // Measured on GB300 against eight compute warps and stages of all four tiles: B=4 H=16 T=2048
-// d=128 FWM Weight-STE dV 340 -> 178 us, dK 403 -> 330; H=16 T=16384 d=128 MinMax K=16 LERP
-// 5097 -> 2252, 5878 -> 4178; 3xTF32 B=8 H=12 T=1024 168 -> 98, 203 -> 190; MinMax B=4 H=12
+// d=128 FWM Weight-STE dV 340 -> 178 us, dK 403 -> 313; H=16 T=16384 d=128 MinMax K=16 LERP
+// 5097 -> 2252, 5878 -> 3785; 3xTF32 B=8 H=12 T=1024 168 -> 98, 203 -> 170; MinMax B=4 H=12
 // T=1024 d=64 (both products) 73.6 -> 71.6.
-// With one score buffer (dK alone at d = 128, TF32) the next tile's S^T is formed under the
-// element work of the current one, once every warp has loaded its scores (bar_sread): dS
-// overwrites g^T, so S^T's columns are free from then on.
+// dK alone takes 32-query tiles: at d = 128 and under 3xTF32 K, V and the accumulators leave 128
+// columns, one pair of 64-query score buffers or two of 32.  With one, products and element
+// work took turns; with two, the groups work on alternate tiles under each other's products.
 // ---------------------------------------------------------------------------
 template <int CAL, int REC, bool FULLG, bool PROJ, bool RS, int SEL>
 __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__ Maps maps, const Params p) {
@@ -243,8 +247,10 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
     if (gated_off(p)) return;
   }
   const int D = p.d, Kq = p.Kint, parts = p.x3 ? 2 : 1, NS = p.nstage, nbuf = p.nbuf;
-  const int qtile = BT * D * 4;
+  
   constexpr bool doDV = SEL != DKV_DK, doDK = SEL != DKV_DV, needV = doDK;
+  constexpr int BQ = SEL == DKV_DK ? 32 : BT;  // queries per tile
+  const int qtile = BQ * D * 4;
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm + p.sm_bars);
   uint64_t* bar_full = bars;
   uint64_t* bar_empty = bars + NS;
@@ -262,44 +268,42 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
   // products dV, dK that read it complete (bar_empty)
   uint64_t* bar_emptyA = bars + 3 * NS + 8;  // [NS]
   uint64_t* bar_drain = bars + 4 * NS + 8;   // the MMA warp's clean-up commit
-  uint64_t* bar_sread = bars + 4 * NS + 9;   // S^T of the tile in every compute warp's registers (early_s)
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 4 * NS + 10);
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 4 * NS + 9);
   const int tid = threadIdx.x, warp = warp_id_uniform();
   const int dp = D * parts;
   const int cK = 0, cV = dp, base = needV ? 2 * dp : dp;
-  const int cdV = base + 128 * nbuf, cdK = cdV + (doDV ? D : 0);
+  const int cdV = base + 2 * BQ * nbuf, cdK = cdV + (doDV ? D : 0);
   // 3xTF32 (one product per launch): the two cross terms accumulate apart from hi x hi.
   // The tensor core rounds each accumulation step toward zero, so a dK / dV row summed
   // over a whole causal column (up to T / 8 x 3 steps) drifts by about one unit in the
   // last place per step; keeping the cross terms out of the main accumulator cuts its
   // steps by three, and the two sums meet in fp32 in the epilogue.
   const int cdC = cdK + (doDK ? D : 0);
-  const int nqt = (p.T + BT - 1) / BT;
+  const int nqt = (p.T + BQ - 1) / BQ;
   const int oQ = 0, odO = parts * qtile, oQT = (needV ? 2 : 1) * parts * qtile,
             odOT = oQT + (doDK ? parts * qtile : 0);
-  const int oRec = odOT + (doDV ? parts * qtile : 0), oTab = oRec + BT * 64;
-  const bool early_s = nbuf == 1 && !p.x3 && !doDV && NS > 1;
+  const int oRec = odOT + (doDV ? parts * qtile : 0), oTab = oRec + BQ * 64;
   const uint32_t tstride = (uint32_t)p.Kp * 8u;
-  constexpr int W = BT / NCG_KV;  // query columns per thread per tile
-  static_assert(W == 16, "the element work and the row sums take 16 columns");
+  constexpr int W = 16;            // query columns per thread per tile
+  constexpr int NGRP = 64 / BQ;    // groups of compute warps taking tiles in turn
+  constexpr int NWT = NCOMP_KV / 32 / NGRP;  // compute warps per tile
 
   if (tid == 0) {
     for (int s = 0; s < NS; ++s) {
       mbar_init(&bar_full[s], 1);
       mbar_init(&bar_fullT[s], 1);
       mbar_init(&bar_empty[s], 1);
-      mbar_init(&bar_emptyA[s], NCOMP_KV / 32);
+      mbar_init(&bar_emptyA[s], NWT);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&bar_sfull[b], 1);
-      mbar_init(&bar_pready[b], NCOMP_KV / 32);
+      mbar_init(&bar_pready[b], NWT);
     }
     mbar_init(bar_done, 1);
     mbar_init(bar_ops, NCOMP_KV / 32);
     mbar_init(bar_stg, 1);
     mbar_init(bar_ostg, NCOMP_KV / 32);
     mbar_init(bar_drain, 1);
-    mbar_init(bar_sread, NCOMP_KV / 32);
     fence_mbar_init();
   }
   if (warp == 0) {
@@ -339,9 +343,9 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
     if (p.ops_smem && snake_item(0) < p.nitems) stage_ops(0);
     for (int item = snake_item(n); item < p.nitems && ok; item = snake_item(++n)) {
       const int kb = item / p.BH, bh = item % p.BH;
-      const int qt0 = (kb * 128) / BT, nit = nqt - qt0;
+      const int qt0 = (kb * 128) / BQ, nit = nqt - qt0;
       for (int it = 0; it < nit; ++it, ++gt, ld.next(NS)) {
-        const int s = ld.i, q0 = (qt0 + it) * BT;
+        const int s = ld.i, q0 = (qt0 + it) * BQ;
         if (gt >= NS && !mbar_wait_warp(&bar_emptyA[s], ld.ph ^ 1u, p.wait_ns, p.status, DEV_ERR_TIMEOUT_SYNC)) {
           ok = false;
           break;
@@ -349,15 +353,15 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
         uint8_t* dst = sm + p.sm_stage0 + s * p.sm_stage_bytes;
         // first the operands of S^T, g^T and the row records, then the transposed tiles
         uint64_t* b = &bar_full[s];
-        const int nrows = min(BT, p.T - q0);
+        const int nrows = min(BQ, p.T - q0);
         uint32_t bytes = (1 + (needV ? 1 : 0)) * parts * qtile + nrows * 64;
         if (CAL == CAL_MINMAX) bytes += nrows * tstride;
         mbar_arrive_expect_tx(b, bytes);
-        load_rows_tile(dst + oQ, &maps.q, b, D, BT, 0, q0, bh);
-        if (p.x3) load_rows_tile(dst + oQ + qtile, &maps.q_lo, b, D, BT, 0, q0, bh);
+        load_rows_tile(dst + oQ, &maps.q, b, D, BQ, 0, q0, bh);
+        if (p.x3) load_rows_tile(dst + oQ + qtile, &maps.q_lo, b, D, BQ, 0, q0, bh);
         if (needV) {
-          load_rows_tile(dst + odO, &maps.dout, b, D, BT, 0, q0, bh);
-          if (p.x3) load_rows_tile(dst + odO + qtile, &maps.dout_lo, b, D, BT, 0, q0, bh);
+          load_rows_tile(dst + odO, &maps.dout, b, D, BQ, 0, q0, bh);
+          if (p.x3) load_rows_tile(dst + odO + qtile, &maps.dout_lo, b, D, BQ, 0, q0, bh);
         }
         const size_t r0 = (size_t)bh * p.T + q0;
         bulk_load(dst + oRec, reinterpret_cast<const RowRec*>(p.rec) + r0, nrows * 64, b);
@@ -371,12 +375,12 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
         uint64_t* bt = &bar_fullT[s];
         mbar_arrive_expect_tx(bt, ((doDK ? 1 : 0) + (doDV ? 1 : 0)) * parts * qtile);
         if (doDK) {
-          load_rows_tile(dst + oQT, &maps.qt, bt, BT, D, q0, 0, bh);
-          if (p.x3) load_rows_tile(dst + oQT + qtile, &maps.qt_lo, bt, BT, D, q0, 0, bh);
+          load_rows_tile(dst + oQT, &maps.qt, bt, BQ, D, q0, 0, bh);
+          if (p.x3) load_rows_tile(dst + oQT + qtile, &maps.qt_lo, bt, BQ, D, q0, 0, bh);
         }
         if (doDV) {
-          load_rows_tile(dst + odOT, &maps.dot, bt, BT, D, q0, 0, bh);
-          if (p.x3) load_rows_tile(dst + odOT + qtile, &maps.dot_lo, bt, BT, D, q0, 0, bh);
+          load_rows_tile(dst + odOT, &maps.dot, bt, BQ, D, q0, 0, bh);
+          if (p.x3) load_rows_tile(dst + odOT + qtile, &maps.dot_lo, bt, BQ, D, q0, 0, bh);
         }
         nT.next(NS);
         ++cT;
@@ -405,32 +409,23 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
     const uint8_t* st0 = sm + p.sm_stage0;
     const uint32_t cKa = tmem + cK, cVa = tmem + cV, cSG = tmem + base;
     int n = 0;
-    uint32_t gt = 0;         // tiles of the CTA's earlier items (early_s)
     RingPos is, ib, cs, cb;  // stage / buffer of the next S^T, g^T product and of the tile being finished
     bool ok = true;
     for (int item = snake_item(n); item < p.nitems && ok; item = snake_item(++n)) {
-      const int kb = item / p.BH, nit = nqt - (kb * 128) / BT;
+      const int kb = item / p.BH, nit = nqt - (kb * 128) / BQ;
       // K / V of the item in TMEM (the compute warps copy them only after the previous
       // item's last S, g were read)
       ok = mbar_wait_warp(bar_ops, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_SYNC);
       if (ok) tc_fence_after();
-      ok = ok && kv_issue_sg(p, is, ib.i, bar_full, bar_sfull, st0, cKa, cVa, cSG, qtile, needV, odO);
+      ok = ok && kv_issue_sg<BQ>(p, is, ib.i, bar_full, bar_sfull, st0, cKa, cVa, cSG, qtile, needV, odO);
       is.next(NS);
       ib.next(nbuf);
       for (int it = 0; it < nit && ok; ++it, cs.next(NS), cb.next(nbuf)) {
         const int b = cb.i, s = cs.i;
         if (nbuf == 2 && it + 1 < nit) {
-          ok = kv_issue_sg(p, is, ib.i, bar_full, bar_sfull, st0, cKa, cVa, cSG, qtile, needV, odO);
+          ok = kv_issue_sg<BQ>(p, is, ib.i, bar_full, bar_sfull, st0, cKa, cVa, cSG, qtile, needV, odO);
           is.next(NS);
           ib.next(nbuf);
-        }
-        if (ok && early_s && it + 1 < nit) {
-          ok = mbar_wait_warp(&bar_full[is.i], is.ph, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA) &&
-               mbar_wait_warp(bar_sread, (gt + it) & 1u, p.wait_ns, p.status, DEV_ERR_TIMEOUT_SYNC);
-          if (ok) {
-            tc_fence_after();
-            kv_issue_s(p, st0 + is.i * p.sm_stage_bytes, 0, cKa, cSG, qtile);
-          }
         }
         if (!ok) break;
         if (!mbar_wait_warp(&bar_pready[b], cb.ph, p.wait_ns, p.status, DEV_ERR_TIMEOUT_SYNC) ||
@@ -440,31 +435,25 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
         }
         tc_fence_after();
         const uint8_t* st = sm + p.sm_stage0 + s * p.sm_stage_bytes;
-        const uint32_t cS = tmem + base + 128 * b, cG = cS + 64;
+        const uint32_t cS = tmem + base + 2 * BQ * b, cG = cS + BQ;
         const bool acc = it > 0;
         if (p.x3) {
           const uint32_t cacc = tmem + (doDV ? cdV : cdK);
           const uint8_t* bt = st + (doDV ? odOT : oQT);
-          mma_tmem_smem(cacc, cS, bt, D, BT, acc);                   // hi x hi
-          mma_tmem_smem(tmem + cdC, cS, bt + qtile, D, BT, acc);     // hi x lo
-          mma_tmem_smem(tmem + cdC, cG, bt, D, BT, true);            // lo x hi
+          mma_tmem_tile<BQ>(cacc, cS, bt, D, acc);                   // hi x hi
+          mma_tmem_tile<BQ>(tmem + cdC, cS, bt + qtile, D, acc);     // hi x lo
+          mma_tmem_tile<BQ>(tmem + cdC, cG, bt, D, true);            // lo x hi
         } else {
-          if (doDV) mma_tmem_smem(tmem + cdV, cS, st + odOT, D, BT, acc);
-          if (doDK) mma_tmem_smem(tmem + cdK, cG, st + oQT, D, BT, acc);
+          if (doDV) mma_tmem_tile<BQ>(tmem + cdV, cS, st + odOT, D, acc);
+          if (doDK) mma_tmem_tile<BQ>(tmem + cdK, cG, st + oQT, D, acc);
         }
         mma_commit(&bar_empty[s]);
-        if (early_s && it + 1 < nit) {  // (the wait for the tile, ahead of its S^T, covered dO too)
-          kv_issue_g(p, st0 + is.i * p.sm_stage_bytes, 0, cVa, cSG, qtile, odO);
-          mma_commit(&bar_sfull[0]);
-          is.next(NS);
-          ib.next(nbuf);
-        } else if (nbuf == 1 && it + 1 < nit) {
-          ok = kv_issue_sg(p, is, ib.i, bar_full, bar_sfull, st0, cKa, cVa, cSG, qtile, needV, odO);
+        if (nbuf == 1 && it + 1 < nit) {
+          ok = kv_issue_sg<BQ>(p, is, ib.i, bar_full, bar_sfull, st0, cKa, cVa, cSG, qtile, needV, odO);
           is.next(NS);
           ib.next(nbuf);
         }
       }
-      gt += (uint32_t)nit;
       mma_commit(bar_done);
     }
     drain_mma(bar_drain, p.wait_ns, p.status);  // clean-up: no product still writes TMEM
@@ -472,6 +461,7 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
   } else {
     setmaxnreg_inc<REG_COMP_KV>();
     const int row = tid & 127, cg = tid >> 7;
+    const int grp = NGRP == 2 ? cg >> 1 : 0;
     // K / V rows of the n-th item into TMEM (each thread a share of its key's columns: with V two
     // column groups take K and two take V), handed to the MMA warp through bar_ops: TF32 at
     // d = 64 from the tiles the producer staged in smem, otherwise from global rows.  The
@@ -513,19 +503,23 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
     group_sync(BAR_COMPUTE, NCOMP_KV);  // the FWM table
     bool failed = false;
     int n = 0;
+    int gt = 0;      // tiles so far
     RingPos cs, cb;  // stage and score buffer of the current tile
     for (int item = snake_item(n); item < p.nitems && !failed; item = snake_item(++n)) {
       const int kb = item / p.BH, bh = item % p.BH;
-      const int qt0 = (kb * 128) / BT, nit = nqt - qt0;
+      const int qt0 = (kb * 128) / BQ, nit = nqt - qt0;
       const int j = kb * 128 + row;
-      const int* tflags = p.tileflags + (size_t)bh * p.nqt + qt0;
-      int tie_next = (doDK && FULLG && CAL != CAL_SOFTMAX) ? __ldg(tflags) : 0;
-      for (int it = 0; it < nit; ++it, cs.next(NS), cb.next(nbuf)) {
-        // the tie flag of this 64-row query tile, loaded one tile ahead
+      // the tie flags are per 64 query rows
+      constexpr bool ties = doDK && FULLG && CAL != CAL_SOFTMAX;
+      const int* tflags = p.tileflags + (size_t)bh * p.nqt + qt0 * BQ / 64;
+      int tie_next = ties ? __ldg(tflags) : 0;
+      for (int it = 0; it < nit; ++it, cs.next(NS), cb.next(nbuf), ++gt) {
+        // the next tile's tie flag, loaded one tile ahead
         const int tie_here = tie_next;
-        if (doDK && FULLG && CAL != CAL_SOFTMAX && it + 1 < nit) tie_next = __ldg(tflags + it + 1);
+        if (ties && it + 1 < nit) tie_next = __ldg(tflags + (it + 1) * BQ / 64);
+        if (NGRP == 2 && (gt & 1) != grp) continue;
         const int b = cb.i, s = cs.i;
-        const int q0 = (qt0 + it) * BT;
+        const int q0 = (qt0 + it) * BQ;
         const bool ok1 = mbar_wait(&bar_sfull[b], cb.ph, p.wait_ns, p.status, DEV_ERR_TIMEOUT_MMA);
         // the stage's row records arrived with its tiles (bar_full), before the products were issued
         const bool ok2 = ok1 && mbar_wait(&bar_full[s], cs.ph, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA);
@@ -535,10 +529,10 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
         }
         tc_fence_after();
         const uint8_t* st = sm + p.sm_stage0 + s * p.sm_stage_bytes;
-        const int c0 = cg * W, i0h = q0 + c0;
+        const int c0 = (NGRP == 2 ? cg & 1 : cg) * W, i0h = q0 + c0;
         const uint32_t recs = smem_u32(st + oRec) + c0 * 64;
         const uint32_t tabs = smem_u32(st + oTab) + c0 * tstride - 0x58000000u;
-        const int cS = base + 128 * b + c0, cG = cS + 64;
+        const int cS = base + 2 * BQ * b + c0, cG = cS + BQ;
         float sv[W], gv[W], pa[W], da[W];
         tmem_ldw<W>(lane_addr(tmem, cS), sv);
         if (needV) {
@@ -548,11 +542,6 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
           for (int q = 0; q < W; ++q) gv[q] = 0.f;
         }
         tmem_ld_wait();
-        if (early_s) {  // the next tile's S^T may overwrite the scores
-          tc_fence_before();
-          __syncwarp();
-          if ((tid & 31) == 0) mbar_arrive(bar_sread);
-        }
         // this warp's keys against its queries: all pairs masked, some, or none
         const int j0w = kb * 128 + (warp & 3) * 32;
         if (i0h + W <= j0w) {
@@ -595,7 +584,12 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
         __syncwarp();
         if ((tid & 31) == 0) mbar_arrive(&bar_pready[b]);
       }
-      // the next item's K / V (this item's S^T, g^T have all been read: the last tile's were)
+      // the next item's K / V, once this item's S^T, g^T are all complete: a group has seen its own
+      // last tile's, and waits for the other group's here (products complete in order, so the
+      // barrier's phase before is over)
+      if (NGRP == 2 && !failed && ((gt - 1) & 1) != grp)
+        failed = !mbar_wait(&bar_sfull[(gt - 1) & 1], (uint32_t)((gt - 1) >> 1) & 1u, p.wait_ns, p.status,
+                            DEV_ERR_TIMEOUT_MMA);
       if (!failed && snake_item(n + 1) < p.nitems) ops_to_tmem(n + 1);
       const bool dok = !failed && mbar_wait(bar_done, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_MMA);
       failed = group_any(BAR_COMPUTE, NCOMP_KV, !dok);

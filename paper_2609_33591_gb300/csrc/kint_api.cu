@@ -404,18 +404,44 @@ int plan_main(Params& p, int mode) {
   return -1;
 }
 
+// The rings of the product pipeline of kint_pair.cuh (d = 128, 3xTF32), with `rest` bytes of other
+// areas to come: two slots of Y where they fit (g, with its A operand in smem, holds its tile
+// longest).  Returns the end of the rings.
+int plan_pair(Params& p, int rest) {
+  const int parts = p.x3 ? 2 : 1, tile = parts * 64 * p.d * 4;
+  p.pair = 1;
+  p.sm_a = 0;
+  p.sm_x = parts * 128 * p.d * 4;
+  p.nx = p.nxt = 1;
+  p.ny = p.sm_x + 4 * tile + rest <= kSmemLimit - 2048 ? 2 : 1;
+  p.sm_y = p.sm_x + p.nx * tile;
+  p.sm_xt = p.sm_y + p.ny * tile;
+  p.nitems = p.nqb * p.BH;
+  p.ngrid = std::min(p.nitems, num_sms());
+  return p.sm_xt + p.nxt * tile;
+}
+
 // Backward kernels: compute warps + MMA warp + producer warp.  A second score
 // buffer (S/g of tile t+1 computed under the element work of tile t) needs TMEM
 // room and at least two stages.
 int plan_dq(Params& p) {
-  p.bk = (!p.x3 && p.d == 64) ? 64 : 32;
-  const int parts = p.x3 ? 2 : 1, ktile = p.bk * p.d * 4, dp = p.d * parts;
+  const int parts = p.x3 ? 2 : 1, ktile = 64 * p.d * 4, dp = p.d * parts;
   const int table = p.calib == KINT_CALIB_MINMAX ? p.Kint * 1024 : 1024;
+  p.pair = 0;
+  if (p.x3 || p.d == 128) {
+    p.sm_table = plan_pair(p, table + 8 * 128 * 4 + 9 * NCOMP_THREADS * 4);
+    p.sm_rows = p.sm_table + table;
+    p.sm_rstat = p.sm_rows + 8 * 128 * 4;
+    p.ops_smem = 0;
+    p.sm_ostage = 0;
+    const int total = std::max(finish_plan(p, p.sm_rstat + 9 * NCOMP_THREADS * 4, 28), kOneCtaPerSm);
+    return total <= kSmemLimit ? total : -1;
+  }
   // TF32 at d = 64: Q and dO arrive as TMA tiles staged in smem (64 KB) and are copied
   // to TMEM from there; otherwise (3xTF32 hi/lo, d = 128) the staging area would not fit
   // next to the K/V stages and the rows are read from global memory.
   p.ops_smem = (!p.x3 && p.d == 64) ? 1 : 0;
-  p.nbuf = (2 * dp + 4 * p.bk + p.d <= 512) ? 2 : 1;  // (always 2 with 32-key tiles)
+  p.nbuf = (2 * dp + 256 + p.d <= 512) ? 2 : 1;
   p.nitems = p.nqb * p.BH;
   p.sm_a = 0;
   p.sm_stage0 = p.ops_smem ? 2 * 128 * p.d * 4 : 0;
@@ -430,7 +456,6 @@ int plan_dq(Params& p) {
     const int total = std::max(finish_plan(p, p.sm_rstat + 9 * NCOMP_THREADS * 4, 3 * p.nstage + 11), kOneCtaPerSm);
     if (total <= kSmemLimit) {
       if (p.nstage == 1) p.nbuf = 1;
-      if (p.bk == 32 && p.nbuf != 2) return -1;  // its two groups need a buffer each
       p.ngrid = std::min(p.nitems, num_sms());
       return total;
     }
@@ -439,23 +464,29 @@ int plan_dq(Params& p) {
 }
 
 int plan_dkdv(Params& p, int sel) {
-  const int bq = sel == DKV_DK ? 32 : 64;  // queries per tile
-  const int parts = p.x3 ? 2 : 1, qtile = bq * p.d * 4, dp = p.d * parts;
+  const int parts = p.x3 ? 2 : 1, qtile = 64 * p.d * 4, dp = p.d * parts;
   const bool doDV = sel != DKV_DK, doDK = sel != DKV_DV;
   // TF32 at d = 64, both products: K and V staged in smem by TMA (see plan_dq)
   p.ops_smem = (!p.x3 && p.d == 64 && doDV && doDK) ? 1 : 0;
+  p.dkv_sel = sel;
+  if (sel == DKV_DK) {  // (launched for d = 128 and 3xTF32 only)
+    p.rec_bytes = round_up(64 * 64 + (p.calib == KINT_CALIB_MINMAX ? 64 * p.Kp * 8 : 0), 1024);
+    p.sm_rec = plan_pair(p, 2 * p.rec_bytes + 2048);
+    p.sm_table = p.sm_rec + 2 * p.rec_bytes;
+    const int total = std::max(finish_plan(p, p.sm_table + 2048, 28), kOneCtaPerSm);
+    return total <= kSmemLimit ? total : -1;
+  }
   const int base = doDK ? 2 * dp : dp;
   // accumulators, and under 3xTF32 (one product per launch) the cross-term accumulator
   const int acc = (doDV ? p.d : 0) + (doDK ? p.d : 0) + (p.x3 ? p.d : 0);
   if (p.x3 && doDV && doDK) return -1;
-  if (base + 2 * bq + acc > 512) return -1;
-  p.dkv_sel = sel;
-  p.nbuf = (base + 4 * bq + acc <= 512) ? 2 : 1;  // (always 2 with 32-query tiles)
+  if (base + 128 + acc > 512) return -1;
+  p.nbuf = (base + 256 + acc <= 512) ? 2 : 1;
   p.sm_a = 0;
   p.sm_stage0 = p.ops_smem ? 2 * 128 * p.d * 4 : 0;
   // the tiles this launch reads: Q; dO, Q^T for dK; dO^T for dV
   const int tiles = 1 + (doDK ? 2 : 0) + (doDV ? 1 : 0);
-  p.sm_stage_bytes = round_up(tiles * parts * qtile + bq * 64 + (p.calib == KINT_CALIB_MINMAX ? bq * p.Kp * 8 : 0), 1024);
+  p.sm_stage_bytes = round_up(tiles * parts * qtile + 64 * 64 + (p.calib == KINT_CALIB_MINMAX ? 64 * p.Kp * 8 : 0), 1024);
   for (p.nstage = 4; p.nstage >= 1; --p.nstage) {
     p.sm_table = p.sm_stage0 + p.nstage * p.sm_stage_bytes;
     // FWM Nearest: the half-bin table, 2K + 3 entries of 8 bytes
@@ -463,7 +494,6 @@ int plan_dkdv(Params& p, int sel) {
     const int total = std::max(finish_plan(p, p.sm_table + table, 4 * p.nstage + 9), kOneCtaPerSm);
     if (total <= kSmemLimit) {
       if (p.nstage == 1) p.nbuf = 1;
-      if (bq == 32 && p.nbuf != 2) return -1;  // its two groups need a buffer each
       // one CTA per SM looping over the (key block, head) items
       p.nitems = p.nqb * p.BH;
       p.ngrid = std::min(p.nitems, num_sms());
@@ -739,20 +769,17 @@ int kint_attn_bwd(const float* Q, const float* K, const float* V, const float* O
   Maps maps;
   std::memset(&maps, 0, sizeof(maps));
   bool ok = true;
-  // d = 128 and 3xTF32: the dQ and dK kernels take 32-row tiles of K, V and Q, dO (the dV
-  // kernel, whose Q tiles have 64 rows, comes before dK: see below)
-  const int rows = (p.x3 || d == 128) ? 32 : 64;
   if (p.x3) {
-    ok = ok && map_nat(&maps.k, w.kh, BH, T, d, rows) && map_nat(&maps.k_lo, w.kl, BH, T, d, rows);
-    ok = ok && map_nat(&maps.v, w.vh, BH, T, d, rows) && map_nat(&maps.v_lo, w.vl, BH, T, d, rows);
+    ok = ok && map_nat(&maps.k, w.kh, BH, T, d, 64) && map_nat(&maps.k_lo, w.kl, BH, T, d, 64);
+    ok = ok && map_nat(&maps.v, w.vh, BH, T, d, 64) && map_nat(&maps.v_lo, w.vl, BH, T, d, 64);
     ok = ok && map_nat(&maps.q, w.qh, BH, T, d, 64) && map_nat(&maps.q_lo, w.ql, BH, T, d, 64);
-    ok = ok && map_nat(&maps.dout, w.doh, BH, T, d, rows) && map_nat(&maps.dout_lo, w.dol, BH, T, d, rows);
+    ok = ok && map_nat(&maps.dout, w.doh, BH, T, d, 64) && map_nat(&maps.dout_lo, w.dol, BH, T, d, 64);
     ok = ok && map_tr(&maps.kt, w.kth, BH, T, Tp, d) && map_tr(&maps.kt_lo, w.ktl, BH, T, Tp, d);
     ok = ok && map_tr(&maps.qt, w.qth, BH, T, Tp, d) && map_tr(&maps.qt_lo, w.qtl, BH, T, Tp, d);
     ok = ok && map_tr(&maps.dot, w.doth, BH, T, Tp, d) && map_tr(&maps.dot_lo, w.dotl, BH, T, Tp, d);
   } else {
-    ok = ok && map_nat(&maps.k, K, BH, T, d, rows) && map_nat(&maps.v, V, BH, T, d, rows);
-    ok = ok && map_nat(&maps.q, Q, BH, T, d, 64) && map_nat(&maps.dout, dO, BH, T, d, rows);
+    ok = ok && map_nat(&maps.k, K, BH, T, d, 64) && map_nat(&maps.v, V, BH, T, d, 64);
+    ok = ok && map_nat(&maps.q, Q, BH, T, d, 64) && map_nat(&maps.dout, dO, BH, T, d, 64);
     ok = ok && map_tr(&maps.kt, w.kth, BH, T, Tp, d) && map_tr(&maps.qt, w.qth, BH, T, Tp, d);
     ok = ok && map_tr(&maps.dot, w.doth, BH, T, Tp, d);
   }
@@ -805,8 +832,6 @@ int kint_attn_bwd(const float* Q, const float* K, const float* V, const float* O
   Params pk2 = p;
   const int smem_kv2 = plan_dkdv(pk2, DKV_DK);
   if (smem_kv2 < 0) return KINT_ERR_UNSUPPORTED;
-  if (!map_nat(&maps.q, p.x3 ? w.qh : Q, BH, T, d, rows) || (p.x3 && !map_nat(&maps.q_lo, w.ql, BH, T, d, rows)))
-    return KINT_ERR_LAUNCH;
   return launch_rc(traced("k_bwd_dkdv", s, [&] { return launch_bwd_dkdv(maps, pk2, smem_kv2, s); }));
 }
 

@@ -11,9 +11,9 @@
 // k_bwd_dkdv (one CTA per 128-key block, a thread per key and column half): per
 //   64-query tile, S^T and g^T, the forward P and the full dS (extremum terms
 //   now known), and dV += P^T dO, dK += dS^T Q.
-// Both: compute warps 0-7, an MMA-issuing warp 8, a TMA/bulk-copy producer warp
-// 9; tiles change hands through mbarriers only.
-#include "kint_bwd_common.cuh"
+// k_bwd_dq: compute warps 0-7; k_bwd_dkdv: 0-15.  MMA-issuing and TMA / bulk-copy producer
+// warps follow; tiles change hands through mbarriers only.
+#include "kint_pair.cuh"
 
 namespace kint {
 
@@ -127,7 +127,6 @@ __device__ __forceinline__ void add_tied_keys(uint32_t mask, float* acc, const f
 
 // MMA thread of k_bwd_dq: wait for key tile kt, then S_b = Q K^T and g_b = dO V^T
 // into score buffer b = kt % nbuf.
-template <int BK>
 __device__ __forceinline__ bool dq_issue_sg(const Params& p, RingPos stg, int b, uint64_t* bar_full,
                                             uint64_t* bar_sfull, const uint8_t* st0, uint32_t cQa, uint32_t cdOa,
                                             uint32_t cSG, int ktile) {
@@ -136,17 +135,17 @@ __device__ __forceinline__ bool dq_issue_sg(const Params& p, RingPos stg, int b,
   tc_fence_after();
   const uint8_t* sk = st0 + s * p.sm_stage_bytes;
   const uint8_t* sv = sk + parts * ktile;
-  const uint32_t cS = cSG + 2 * BK * b, cG = cS + BK;
+  const uint32_t cS = cSG + 128 * b, cG = cS + 64;
   if (p.x3) {
-    mma_tmem_smem(cS, cQa + D, sk, BK, D, false);     // Q_lo K_hi
-    mma_tmem_smem(cS, cQa, sk + ktile, BK, D, true);  // Q_hi K_lo
-    mma_tmem_smem(cS, cQa, sk, BK, D, true);          // Q_hi K_hi
-    mma_tmem_smem(cG, cdOa + D, sv, BK, D, false);
-    mma_tmem_smem(cG, cdOa, sv + ktile, BK, D, true);
-    mma_tmem_smem(cG, cdOa, sv, BK, D, true);
+    mma_tmem_smem(cS, cQa + D, sk, BT, D, false);     // Q_lo K_hi
+    mma_tmem_smem(cS, cQa, sk + ktile, BT, D, true);  // Q_hi K_lo
+    mma_tmem_smem(cS, cQa, sk, BT, D, true);          // Q_hi K_hi
+    mma_tmem_smem(cG, cdOa + D, sv, BT, D, false);
+    mma_tmem_smem(cG, cdOa, sv + ktile, BT, D, true);
+    mma_tmem_smem(cG, cdOa, sv, BT, D, true);
   } else {
-    mma_tmem_smem(cS, cQa, sk, BK, D, false);
-    mma_tmem_smem(cG, cdOa, sv, BK, D, false);
+    mma_tmem_smem(cS, cQa, sk, BT, D, false);
+    mma_tmem_smem(cG, cdOa, sv, BT, D, false);
   }
   mma_commit(&bar_sfull[b]);
   return true;
@@ -154,19 +153,16 @@ __device__ __forceinline__ bool dq_issue_sg(const Params& p, RingPos stg, int b,
 
 // ---------------------------------------------------------------------------
 // k_bwd_dq.
-// BK: keys per tile.  64 at d = 64 in TF32: a thread takes half of a tile's columns of its row.  32
-// at d = 128 and under 3xTF32, where Q, dO and dQ leave 128 TMEM columns, one pair of
-// 64-key score buffers or two of 32: with one, products and element work took turns; with
-// two, the groups of four compute warps take the tiles in turn, under each other's
-// products (a thread takes all of a tile's columns, every other tile: the same keys in the
-// same order as half of every 64-key tile, so the row sums keep their bits).  (Against 64-key tiles and one
-// buffer: B=4 H=16 T=2048 d=128 303 -> 272 us, H=16 T=16384 d=128 MinMax 4730 -> 4137, 3xTF32
-// B=8 H=12 T=1024 172 -> 158.)
+// PAIR (d = 128, 3xTF32): the product pipeline of kint_pair.cuh (A1 = Q in TMEM, A2 = dO in smem,
+// K, V and K^T in rings of their own).  One score buffer and one stage of all three tiles, the
+// products and the element work in turns, took at B=4 H=16 T=2048 d=128 FWM 303 us (now 248),
+// at H=16 T=16384 d=128 MinMax K=16 LERP 4710 (now 3165), at B=8 H=12 T=1024 under 3xTF32 180
+// (now 147); tiles of 32 keys in two buffers 272, 4137 and 158.  Otherwise:
 // TMEM: Q [0, dp), dO [dp, 2dp) (dp = d, or 2d for 3xTF32 hi|lo; loaded by the
-// compute threads), then per score buffer b: S_b at 2dp + 2 BK b (BK columns), g_b
-// right after it (BK columns); dQ at 2dp + 2 BK nbuf.  dS overwrites S_b (its tf32
+// compute threads), then per score buffer b: S_b at 2dp + 128 b (64 columns), g_b
+// right after it (64 columns); dQ at 2dp + 128 nbuf.  dS overwrites S_b (its tf32
 // lo part, under 3xTF32, overwrites g_b).
-// smem: stages {K [BK x d], V [BK x d], K^T [d x BK]} (hi[, lo] each) at
+// smem: stages {K [64 x d], V [64 x d], K^T [d x 64]} (hi[, lo] each) at
 // sm_stage0; the grid pair table at sm_table; exchange words at sm_rows.
 // ---------------------------------------------------------------------------
 // Producer warp of k_bwd_dq: TMA-stores the dQ tile of its k-th item, which the compute
@@ -180,8 +176,8 @@ __device__ __forceinline__ bool store_staged_dq(const Maps& maps, const Params& 
   return true;
 }
 
-template <int CAL, bool FULLG, int BK>
-__global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ Maps maps, const Params p) {
+template <int CAL, bool FULLG, bool PAIR>
+__global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ Maps maps, const Params p) {
   uint8_t* sm = smem_base();
   if (p.gate != nullptr) {
     // launched on one side of a device-side decision: when the single-pass backward ran
@@ -190,8 +186,7 @@ __global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ M
     if (gated_off(p)) return;
   }
   const int D = p.d, Kq = p.Kint, parts = p.x3 ? 2 : 1, NS = p.nstage, nbuf = p.nbuf;
-  const int ktile = BK * D * 4;
-  constexpr int NGRP = 64 / BK, NWT = NCOMP / 32 / NGRP;  // groups of compute warps taking tiles in turn; warps per tile
+  const int ktile = BT * D * 4;
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm + p.sm_bars);
   uint64_t* bar_full = bars;               // [NS]
   uint64_t* bar_empty = bars + NS;         // [NS]
@@ -207,22 +202,27 @@ __global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ M
   // score buffer b free again: the dQ product that read its dS completed (MMA2 -> MMA warp)
   uint64_t* bar_dqdone = bars + 3 * NS + 8;  // [2]
   uint64_t* bar_drain = bars + 3 * NS + 10;  // the clean-up commits of the two MMA warps
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 3 * NS + 11);
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + (PAIR ? PAIR_NBARS : 3 * NS + 11));
+  const PairBars B = pair_bars(bars);
   float* xch = reinterpret_cast<float*>(sm + p.sm_rows);  // [8][128]
   const int tid = threadIdx.x, warp = warp_id_uniform();
-  constexpr int W = 32;  // key columns per thread per tile
+  constexpr int W = BT / NCG;  // key columns per thread per tile
   const int dp = D * parts;
-  const int cQ = 0, cdO = dp, cSG0 = 2 * dp, cdQ = cSG0 + 2 * BK * nbuf;
+  const int cQ = 0, cdO = dp, cSG0 = PAIR ? 128 : 2 * dp, cdQ = cSG0 + 128 * (PAIR ? 2 : nbuf);
 
-  if (tid == 0) {
+  if (PAIR && tid == 0) {
+    pair_init(B, NCOMP / 32);
+    fence_mbar_init();
+  }
+  if (!PAIR && tid == 0) {
     for (int s = 0; s < NS; ++s) {
       mbar_init(&bar_full[s], 1);
       mbar_init(&bar_empty[s], 1);
-      mbar_init(&bar_emptyA[s], NWT);
+      mbar_init(&bar_emptyA[s], NCOMP / 32);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&bar_sfull[b], 1);
-      mbar_init(&bar_pready[b], NWT);
+      mbar_init(&bar_pready[b], NCOMP / 32);
       mbar_init(&bar_dqdone[b], 1);
     }
     mbar_init(bar_done, 1);
@@ -246,7 +246,29 @@ __global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ M
   if (threadIdx.x == 0 && *tslot != 0u) dev_flag(p.status, DEV_ERR_BOUNDS);
   constexpr uint32_t tmem = 0;
 
-  if (warp == PRODUCER_WARP) {
+  if (PAIR && warp >= NCOMP / 32) {
+    auto get = [&](int n) {
+      const int item = snake_item(n), qb = p.nqb - 1 - item / p.BH;
+      return PairItem{item % p.BH, qb * 128, 0, min(2 * qb + 2, (p.T + BT - 1) / BT), item < p.nitems};
+    };
+    const PairMaps m{&maps.q, &maps.q_lo, &maps.dout, &maps.dout_lo, &maps.k, &maps.k_lo, &maps.v, &maps.v_lo,
+                     &maps.kt, &maps.kt_lo};
+    if (warp == PRODUCER_WARP) {
+      pair_producer<false>(p, m, B, sm, get, [](const PairItem&, int, uint8_t*, uint64_t*) {});
+    } else if (warp == MMA_WARP) {
+      pair_mma_sg(p, B, sm, get);
+    } else if (warp == MMA2_WARP) {
+      pair_mma_acc(p, B, sm, get, [&](uint32_t cS, uint32_t cG, const uint8_t* kt, bool first) {
+        mma_tmem_smem(cdQ, cS, kt, D, BT, !first);  // dS_hi K_hi
+        if (p.x3) {
+          mma_tmem_smem(cdQ, cS, kt + ktile, D, BT, true);  // dS_hi K_lo
+          mma_tmem_smem(cdQ, cG, kt, D, BT, true);          // dS_lo K_hi
+        }
+      });
+    } else {
+      pair_producer_t(p, m, B, sm, get);
+    }
+  } else if (warp == PRODUCER_WARP) {
     int gt = 0, n = 0;
     RingPos ld;  // stage of the next tile loaded
     bool ok = true;
@@ -262,7 +284,7 @@ __global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ M
     if (p.ops_smem && snake_item(0) < p.nitems) stage_ops(0);
     for (int item = snake_item(n); item < p.nitems && ok; item = snake_item(++n)) {
       const int qb = p.nqb - 1 - item / p.BH, bh = item % p.BH;
-      const int nkt = min((128 / BK) * (qb + 1), (p.T + BK - 1) / BK);
+      const int nkt = min(2 * qb + 2, (p.T + BT - 1) / BT);
       for (int kt = 0; kt < nkt; ++kt, ++gt, ld.next(NS)) {
         const int s = ld.i;
         if (gt >= NS && !mbar_wait_warp(&bar_emptyA[s], ld.ph ^ 1u, p.wait_ns, p.status, DEV_ERR_TIMEOUT_SYNC)) {
@@ -272,18 +294,18 @@ __global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ M
         uint8_t* dst = sm + p.sm_stage0 + s * p.sm_stage_bytes;
         uint64_t* b = &bar_full[s];
         mbar_arrive_expect_tx(b, 3 * parts * ktile);
-        load_rows_tile(dst, &maps.k, b, D, BK, 0, kt * BK, bh);
-        load_rows_tile(dst + parts * ktile, &maps.v, b, D, BK, 0, kt * BK, bh);
+        load_rows_tile(dst, &maps.k, b, D, BT, 0, kt * BT, bh);
+        load_rows_tile(dst + parts * ktile, &maps.v, b, D, BT, 0, kt * BT, bh);
         if (p.x3) {
-          load_rows_tile(dst + ktile, &maps.k_lo, b, D, BK, 0, kt * BK, bh);
-          load_rows_tile(dst + parts * ktile + ktile, &maps.v_lo, b, D, BK, 0, kt * BK, bh);
+          load_rows_tile(dst + ktile, &maps.k_lo, b, D, BT, 0, kt * BT, bh);
+          load_rows_tile(dst + parts * ktile + ktile, &maps.v_lo, b, D, BT, 0, kt * BT, bh);
         }
         if (gt >= NS && !mbar_wait_warp(&bar_empty[s], ld.ph ^ 1u, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA)) {
           ok = false;
           break;
         }
-        load_rows_tile(dst + 2 * parts * ktile, &maps.kt, b, BK, D, kt * BK, 0, bh);
-        if (p.x3) load_rows_tile(dst + 2 * parts * ktile + ktile, &maps.kt_lo, b, BK, D, kt * BK, 0, bh);
+        load_rows_tile(dst + 2 * parts * ktile, &maps.kt, b, BT, D, kt * BT, 0, bh);
+        if (p.x3) load_rows_tile(dst + 2 * parts * ktile + ktile, &maps.kt_lo, b, BT, D, kt * BT, 0, bh);
         // The next item's Q / dO, as soon as the stage ring holds this item's first tiles: it needs
         // this item's Q / dO copied out into TMEM and the previous item's dQ tile, staged in the
         // same area since, stored; both happen at the end of the previous item, so the load has
@@ -314,7 +336,7 @@ __global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ M
     bool ok = true;
     for (int item = snake_item(n); item < p.nitems && ok; item = snake_item(++n)) {
       const int qb = p.nqb - 1 - item / p.BH;
-      const int nkt = min((128 / BK) * (qb + 1), (p.T + BK - 1) / BK);
+      const int nkt = min(2 * qb + 2, (p.T + BT - 1) / BT);
       // Q / dO of the item in TMEM (copied by the compute warps once the previous item's
       // last S, g were read)
       ok = mbar_wait_warp(bar_ops, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_SYNC);
@@ -325,7 +347,7 @@ __global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ M
           ok = false;
           break;
         }
-        ok = dq_issue_sg<BK>(p, is, ib.i, bar_full, bar_sfull, st0, cQa, cdOa, cSG, ktile);
+        ok = dq_issue_sg(p, is, ib.i, bar_full, bar_sfull, st0, cQa, cdOa, cSG, ktile);
       }
     }
     drain_mma(bar_drain, p.wait_ns, p.status);  // clean-up: no product still writes TMEM
@@ -336,7 +358,7 @@ __global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ M
     bool ok = true;
     for (int item = snake_item(n); item < p.nitems && ok; item = snake_item(++n)) {
       const int qb = p.nqb - 1 - item / p.BH;
-      const int nkt = min((128 / BK) * (qb + 1), (p.T + BK - 1) / BK);
+      const int nkt = min(2 * qb + 2, (p.T + BT - 1) / BT);
       for (int kt = 0; kt < nkt && ok; ++kt, cs.next(NS), cb.next(nbuf)) {
         const int b = cb.i, s = cs.i;
         if (!mbar_wait_warp(&bar_pready[b], cb.ph, p.wait_ns, p.status, DEV_ERR_TIMEOUT_SYNC)) {
@@ -345,14 +367,14 @@ __global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ M
         }
         tc_fence_after();
         const uint8_t* skt = sm + p.sm_stage0 + s * p.sm_stage_bytes + 2 * parts * ktile;
-        const uint32_t cS = tmem + cSG0 + 2 * BK * b, cG = cS + BK;
+        const uint32_t cS = tmem + cSG0 + 128 * b, cG = cS + 64;
         const bool acc = kt > 0;
         if (p.x3) {
-          mma_tmem_tile<BK>(tmem + cdQ, cS, skt, D, acc);           // dS_hi K_hi
-          mma_tmem_tile<BK>(tmem + cdQ, cS, skt + ktile, D, true);  // dS_hi K_lo
-          mma_tmem_tile<BK>(tmem + cdQ, cG, skt, D, true);          // dS_lo K_hi
+          mma_tmem_smem(tmem + cdQ, cS, skt, D, BT, acc);           // dS_hi K_hi
+          mma_tmem_smem(tmem + cdQ, cS, skt + ktile, D, BT, true);  // dS_hi K_lo
+          mma_tmem_smem(tmem + cdQ, cG, skt, D, BT, true);          // dS_lo K_hi
         } else {
-          mma_tmem_tile<BK>(tmem + cdQ, cS, skt, D, acc);
+          mma_tmem_smem(tmem + cdQ, cS, skt, D, BT, acc);
         }
         mma_commit(&bar_empty[s]);
         mma_commit(&bar_dqdone[b]);
@@ -363,13 +385,16 @@ __global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ M
   } else {
     // ---- compute warps: items one after the other ----
     const int row = tid & 127, cg = (tid >> 7) & (NCG - 1);
-    int gt = 0;  // tiles so far
     // Operand rows of the n-th item into TMEM (column group 0 takes Q, group 1 takes dO),
     // handed to the MMA warp through bar_ops.  TF32 at d = 64: from the tiles the producer
     // staged in smem; otherwise from global rows.  The next item's rows go in as soon as
     // the current item's last S, g have been read (before its dQ epilogue), so the next
     // item's first products run under that epilogue.
     auto ops_to_tmem = [&](int n) {
+      if constexpr (PAIR) {
+        pair_ops_to_tmem(p, B, sm, n, row, cg * (D / NCG), D / NCG);
+        return;
+      }
       const int item = snake_item(n);
       const int qb = p.nqb - 1 - item / p.BH, bh = item % p.BH, i = qb * 128 + row;
       if (p.ops_smem) {
@@ -438,7 +463,7 @@ __global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ M
     for (int item = snake_item(n); item < p.nitems && !failed; item = snake_item(++n)) {
       // ---- set-up: row constants, grid table (the operands are in TMEM already) ----
       const int qb = p.nqb - 1 - item / p.BH, bh = item % p.BH;
-      const int nkt = min((128 / BK) * (qb + 1), (p.T + BK - 1) / BK);
+      const int nkt = min(2 * qb + 2, (p.T + BT - 1) / BT);
       const int i = qb * 128 + row;
       const bool row_ok = i < p.T;
       const size_t rw = (size_t)bh * p.T + (row_ok ? i : 0);
@@ -484,33 +509,34 @@ __global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ M
       group_sync(BAR_COMPUTE, NCOMP);
       float own = 0.f, cm = 0.f;
       const int i0w = qb * 128 + (warp & 3) * 32;  // this warp's first row
-      for (int kt = 0; kt < nkt; ++kt, cb.next(nbuf), cs.next(NS), ++gt) {
-        if (NGRP == 2 && (gt & 1) != cg) continue;
+      for (int kt = 0; kt < nkt; ++kt, cb.next(PAIR ? 2 : nbuf)) {
         const int b = cb.i;
-        const bool ok = mbar_wait(&bar_sfull[b], cb.ph, p.wait_ns, p.status, DEV_ERR_TIMEOUT_MMA);
+        const bool ok = mbar_wait(PAIR ? &B.sfull[b] : &bar_sfull[b], cb.ph, p.wait_ns, p.status, DEV_ERR_TIMEOUT_MMA);
         if (!ok) {
           failed = true;
           break;
         }
         // S, g of the tile completed: its K and V may be reloaded
-        if ((tid & 31) == 0) mbar_arrive(&bar_emptyA[cs.i]);
+        if constexpr (!PAIR) {
+          if ((tid & 31) == 0) mbar_arrive(&bar_emptyA[cs.i]);
+          cs.next(NS);
+        }
         tc_fence_after();
-        const int cS = cSG0 + 2 * BK * b + (NGRP == 2 ? 0 : cg * W), cG = cS + BK;
+        const int cS = cSG0 + 128 * b + cg * W, cG = cS + 64;
         float sv[W], gv[W], out[W];
         tmem_ldw<W>(lane_addr(tmem, cS), sv);
         tmem_ldw<W>(lane_addr(tmem, cG), gv);
         tmem_ld_wait();
-        const int j0 = kt * BK + (NGRP == 2 ? 0 : cg * W);
-        if (BK == 32 && j0 > i0w + 31) {  // every key lies after every row of the warp
+        const int j0 = kt * BT + cg * W;
+        if (PAIR && j0 > i0w + 31) {  // every key lies after every row of the warp
 #pragma unroll
           for (int q = 0; q < W; ++q) out[q] = 0.f;
-        } else if (j0 + W - 1 > (BK == 32 ? i0w : qb * 128)) {
+        } else if (j0 + W - 1 > (PAIR ? i0w : qb * 128))
           dq_chunk<CAL, FULLG, true, W>(sv, gv, out, j0, i, k1q, c0q, g.inv_h, ga, gb, g.nogrid, Kf, fk, tab, sk1,
                                         sc0, invWf, g.hl, g.b0l, own, cm);
-        } else {
+        else
           dq_chunk<CAL, FULLG, false, W>(sv, gv, out, j0, i, k1q, c0q, g.inv_h, ga, gb, g.nogrid, Kf, fk, tab,
                                          sk1, sc0, invWf, g.hl, g.b0l, own, cm);
-        }
         if (__any_sync(0xffffffffu, track)) {
           // rare: tied extrema, the tie set is found by equality on the recomputed scores
           uint32_t mk_max = 0, mk_min = 0;
@@ -538,15 +564,10 @@ __global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ M
         tmem_st_wait();
         tc_fence_before();
         __syncwarp();
-        if ((tid & 31) == 0) mbar_arrive(&bar_pready[b]);
+        if ((tid & 31) == 0) mbar_arrive(PAIR ? &B.pready[b] : &bar_pready[b]);
       }
       // the next item's Q / dO (this item's S, g have all been read: the last tile's were)
       // and its row statistics
-      // (a group has seen its own last tile's S, g, and waits for the other group's here: products
-      // complete in order, so the barrier's phase before is over)
-      if (NGRP == 2 && !failed && ((gt - 1) & 1) != cg)
-        failed = !mbar_wait(&bar_sfull[(gt - 1) & 1], (uint32_t)((gt - 1) >> 1) & 1u, p.wait_ns, p.status,
-                            DEV_ERR_TIMEOUT_MMA);
       if (!failed && snake_item(n + 1) < p.nitems) {
         ops_to_tmem(n + 1);
         nx = load_row_stats(n + 1);
@@ -560,7 +581,7 @@ __global__ void __launch_bounds__(NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ M
         gather_rows128_issue(own_row ? p.K + ((size_t)bh * p.T + amax) * D + cg * (D / NCG) : nullptr,
                              reinterpret_cast<float4*>(sm + p.sm_a + 128 * D * 4) + warp * 256);
       }
-      const bool dok = !failed && mbar_wait(bar_done, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_MMA);
+      const bool dok = !failed && mbar_wait(PAIR ? B.done : bar_done, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_MMA);
       failed = group_any(BAR_COMPUTE, NCOMP, !dok);
       if (!failed) {
         tc_fence_after();
@@ -726,29 +747,30 @@ cudaError_t launch_kcum(const float* K, float* C, int BH, int T, int d, cudaStre
   return launch_pdl(k_kcum, dim3((unsigned)(BH * (d / 32))), dim3(KCUM_WARPS * 32), 0, s, K, C, T, d);
 }
 
-template <int BK>
-static cudaError_t launch_dq_bk(const Maps& maps, const Params& p, int smem_bytes, cudaStream_t s) {
+template <bool PAIR>
+static cudaError_t launch_dq_t(const Maps& maps, const Params& p, int smem_bytes, cudaStream_t s) {
   const dim3 grid((unsigned)p.ngrid);
+  const int nthr = PAIR ? NTHR_DQ + 32 : NTHR_DQ;
   const bool full = p.grad != GRAD_DETACH && p.grad != GRAD_DETACH_PROJ;
-  if (p.calib == CAL_SOFTMAX) return launch3(k_bwd_dq<CAL_SOFTMAX, false, BK>, grid, maps, p, smem_bytes, s, NTHR_DQ);
+  if (p.calib == CAL_SOFTMAX) return launch3(k_bwd_dq<CAL_SOFTMAX, false, PAIR>, grid, maps, p, smem_bytes, s, nthr);
   if (p.calib == CAL_EXP8)
-    return full ? launch3(k_bwd_dq<CAL_EXP8, true, BK>, grid, maps, p, smem_bytes, s, NTHR_DQ)
-                : launch3(k_bwd_dq<CAL_EXP8, false, BK>, grid, maps, p, smem_bytes, s, NTHR_DQ);
+    return full ? launch3(k_bwd_dq<CAL_EXP8, true, PAIR>, grid, maps, p, smem_bytes, s, nthr)
+                : launch3(k_bwd_dq<CAL_EXP8, false, PAIR>, grid, maps, p, smem_bytes, s, nthr);
   if (p.calib == CAL_EXPB)
-    return full ? launch3(k_bwd_dq<CAL_EXPB, true, BK>, grid, maps, p, smem_bytes, s, NTHR_DQ)
-                : launch3(k_bwd_dq<CAL_EXPB, false, BK>, grid, maps, p, smem_bytes, s, NTHR_DQ);
+    return full ? launch3(k_bwd_dq<CAL_EXPB, true, PAIR>, grid, maps, p, smem_bytes, s, nthr)
+                : launch3(k_bwd_dq<CAL_EXPB, false, PAIR>, grid, maps, p, smem_bytes, s, nthr);
   if (p.calib == CAL_MINMAX)
-    return full ? launch3(k_bwd_dq<CAL_MINMAX, true, BK>, grid, maps, p, smem_bytes, s, NTHR_DQ)
-                : launch3(k_bwd_dq<CAL_MINMAX, false, BK>, grid, maps, p, smem_bytes, s, NTHR_DQ);
+    return full ? launch3(k_bwd_dq<CAL_MINMAX, true, PAIR>, grid, maps, p, smem_bytes, s, nthr)
+                : launch3(k_bwd_dq<CAL_MINMAX, false, PAIR>, grid, maps, p, smem_bytes, s, nthr);
   if (p.calib == CAL_FWMR)
-    return full ? launch3(k_bwd_dq<CAL_FWMR, true, BK>, grid, maps, p, smem_bytes, s, NTHR_DQ)
-                : launch3(k_bwd_dq<CAL_FWMR, false, BK>, grid, maps, p, smem_bytes, s, NTHR_DQ);
-  return full ? launch3(k_bwd_dq<CAL_FWM, true, BK>, grid, maps, p, smem_bytes, s, NTHR_DQ)
-              : launch3(k_bwd_dq<CAL_FWM, false, BK>, grid, maps, p, smem_bytes, s, NTHR_DQ);
+    return full ? launch3(k_bwd_dq<CAL_FWMR, true, PAIR>, grid, maps, p, smem_bytes, s, nthr)
+                : launch3(k_bwd_dq<CAL_FWMR, false, PAIR>, grid, maps, p, smem_bytes, s, nthr);
+  return full ? launch3(k_bwd_dq<CAL_FWM, true, PAIR>, grid, maps, p, smem_bytes, s, nthr)
+              : launch3(k_bwd_dq<CAL_FWM, false, PAIR>, grid, maps, p, smem_bytes, s, nthr);
 }
 
 cudaError_t launch_bwd_dq(const Maps& maps, const Params& p, int smem_bytes, cudaStream_t s) {
-  return p.bk == 32 ? launch_dq_bk<32>(maps, p, smem_bytes, s) : launch_dq_bk<64>(maps, p, smem_bytes, s);
+  return p.pair ? launch_dq_t<true>(maps, p, smem_bytes, s) : launch_dq_t<false>(maps, p, smem_bytes, s);
 }
 
 }  // namespace kint

@@ -15,12 +15,6 @@ __device__ __forceinline__ int4 lds_i4(uint32_t addr) {
   return v;
 }
 
-// D[tmem, 128 x N] (+)= A B^T over K = 32 or 64 columns, A in TMEM, B a tile in smem.
-template <int K>
-__device__ __forceinline__ void mma_tmem_tile(uint32_t d_tmem, uint32_t a_tmem, const uint8_t* b, int N, bool acc) {
-  mma_ts_k<K / 8>(d_tmem, a_tmem, b, N * SW, idesc_tf32(128, N, 0, 0), acc);
-}
-
 template <class K>
 static cudaError_t launch3(K kern, dim3 grid, const Maps& maps, const Params& p, int smem_bytes, cudaStream_t s,
                            int nthr = NTHR) {

@@ -2,15 +2,15 @@
 // translation unit of the plain kernels and by the one of the kernels that also
 // accumulate the per-row score-gradient sums (RS), so the two compile in parallel.
 #pragma once
-#include "kint_bwd_common.cuh"
+#include "kint_pair.cuh"
 
 namespace kint {
 
-// Thread roles: sixteen compute warps (thread t owns key kb*128 + t%128 and 16 query columns:
-// 16 (t/128) .. + 15 of each 64-query tile, or, with 32-query tiles, 16 (t/128 % 2) .. + 15 of
-// every other tile, the two groups of eight warps taking the tiles in turn), the MMA warp, the producer warp and two idle
-// warps.  The fifth warpgroup gives registers to the compute warpgroups: launched at 96 per
-// thread, it keeps 64 and they take 104.
+// Thread roles: sixteen compute warps (thread t owns key kb*128 + t%128 and the 16 query columns
+// 16 (t/128) .. + 15 of each 64-query tile), the MMA warp, the producer warp and two idle
+// warps (dK alone: a second MMA and a second producer warp, kint_pair.cuh).  The fifth
+// warpgroup gives registers to the compute warpgroups: launched at 96 per thread, it keeps 64
+// and they take 104.
 constexpr int NCG_KV = 4, NCOMP_KV = 128 * NCG_KV, NTHR_KV = NCOMP_KV + 128;
 constexpr int MMA_WARP_KV = NCOMP_KV / 32, PRODUCER_WARP_KV = MMA_WARP_KV + 1;
 constexpr int REG_LAUNCH_KV = 96, REG_COMP_KV = 104, REG_AUX_KV = 64;
@@ -166,42 +166,39 @@ __device__ __forceinline__ void rowsum_add(const float (&v)[16], float* dsum, fl
 }
 
 // MMA warp of k_bwd_dkdv: the products of the query tile in stage s (landed) into score buffer b.
-template <int BQ>
 __device__ __forceinline__ void kv_issue_s(const Params& p, const uint8_t* st, int b, uint32_t cKa, uint32_t cSG,
                                            int qtile) {
   const int D = p.d;
-  const uint32_t cS = cSG + 2 * BQ * b;
+  const uint32_t cS = cSG + 128 * b;
   if (p.x3) {
-    mma_tmem_smem(cS, cKa + D, st, BQ, D, false);
-    mma_tmem_smem(cS, cKa, st + qtile, BQ, D, true);
-    mma_tmem_smem(cS, cKa, st, BQ, D, true);
+    mma_tmem_smem(cS, cKa + D, st, BT, D, false);
+    mma_tmem_smem(cS, cKa, st + qtile, BT, D, true);
+    mma_tmem_smem(cS, cKa, st, BT, D, true);
   } else {
-    mma_tmem_smem(cS, cKa, st, BQ, D, false);
+    mma_tmem_smem(cS, cKa, st, BT, D, false);
   }
 }
-template <int BQ>
 __device__ __forceinline__ void kv_issue_g(const Params& p, const uint8_t* st, int b, uint32_t cVa, uint32_t cSG,
                                            int qtile, int odO) {
   const int D = p.d;
-  const uint32_t cG = cSG + 2 * BQ * b + BQ;
+  const uint32_t cG = cSG + 128 * b + 64;
   if (p.x3) {
-    mma_tmem_smem(cG, cVa + D, st + odO, BQ, D, false);
-    mma_tmem_smem(cG, cVa, st + odO + qtile, BQ, D, true);
-    mma_tmem_smem(cG, cVa, st + odO, BQ, D, true);
+    mma_tmem_smem(cG, cVa + D, st + odO, BT, D, false);
+    mma_tmem_smem(cG, cVa, st + odO + qtile, BT, D, true);
+    mma_tmem_smem(cG, cVa, st + odO, BT, D, true);
   } else {
-    mma_tmem_smem(cG, cVa, st + odO, BQ, D, false);
+    mma_tmem_smem(cG, cVa, st + odO, BT, D, false);
   }
 }
 // Both (S^T_b = K Q^T and, with V, g^T_b = V dO^T) once the tile in stage stg has landed.
-template <int BQ>
 __device__ __forceinline__ bool kv_issue_sg(const Params& p, RingPos stg, int b, uint64_t* bar_full,
                                             uint64_t* bar_sfull, const uint8_t* st0, uint32_t cKa, uint32_t cVa,
                                             uint32_t cSG, int qtile, bool needV, int odO) {
   if (!mbar_wait_warp(&bar_full[stg.i], stg.ph, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA)) return false;
   tc_fence_after();
   const uint8_t* st = st0 + stg.i * p.sm_stage_bytes;
-  kv_issue_s<BQ>(p, st, b, cKa, cSG, qtile);
-  if (needV) kv_issue_g<BQ>(p, st, b, cVa, cSG, qtile, odO);
+  kv_issue_s(p, st, b, cKa, cSG, qtile);
+  if (needV) kv_issue_g(p, st, b, cVa, cSG, qtile, odO);
   mma_commit(&bar_sfull[b]);
   return true;
 }
@@ -227,15 +224,15 @@ __device__ __forceinline__ bool store_staged_dkdv(const Maps& maps, const Params
 // for dK, dO^T for dV; the 64 RowRecs of the tile, and (MinMax) their grid pair tables;
 // FWM's shared table at sm_table.  (With all four in every stage a one-product launch at
 // d = 128 or under 3xTF32 had one stage and nothing overlapped.)
-// What bounds it: the issue of the products by one warp and, at one score buffer, the chain
-// products -> element work -> products; shared-memory loads of the row records come next.
+// dK alone (d = 128, 3xTF32) runs the product pipeline of kint_pair.cuh instead of the stage
+// ring: K in TMEM, V as an operand in smem, Q, dO and Q^T in rings of their own.
+// What bounds it: the issue of the products by one warp, then the shared-memory loads of the
+// row records.
 // Measured on GB300 against eight compute warps and stages of all four tiles: B=4 H=16 T=2048
-// d=128 FWM Weight-STE dV 340 -> 178 us, dK 403 -> 313; H=16 T=16384 d=128 MinMax K=16 LERP
-// 5097 -> 2252, 5878 -> 3785; 3xTF32 B=8 H=12 T=1024 168 -> 98, 203 -> 170; MinMax B=4 H=12
-// T=1024 d=64 (both products) 73.6 -> 71.6.
-// dK alone takes 32-query tiles: at d = 128 and under 3xTF32 K, V and the accumulators leave 128
-// columns, one pair of 64-query score buffers or two of 32.  With one, products and element
-// work took turns; with two, the groups work on alternate tiles under each other's products.
+// d=128 FWM Weight-STE dV 340 -> 178 us, dK 403 -> 238; H=16 T=16384 d=128 MinMax K=16 LERP
+// 5097 -> 2250, 5878 -> 3047; 3xTF32 B=8 H=12 T=1024 168 -> 98, 203 -> 131; MinMax B=4 H=12
+// T=1024 d=64 (both products) 73.6 -> 71.6.  (dK in the stage ring with 32-query tiles: 313,
+// 3785 and 170.)
 // ---------------------------------------------------------------------------
 template <int CAL, int REC, bool FULLG, bool PROJ, bool RS, int SEL>
 __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__ Maps maps, const Params p) {
@@ -247,10 +244,9 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
     if (gated_off(p)) return;
   }
   const int D = p.d, Kq = p.Kint, parts = p.x3 ? 2 : 1, NS = p.nstage, nbuf = p.nbuf;
-  
   constexpr bool doDV = SEL != DKV_DK, doDK = SEL != DKV_DV, needV = doDK;
-  constexpr int BQ = SEL == DKV_DK ? 32 : BT;  // queries per tile
-  const int qtile = BQ * D * 4;
+  constexpr bool PAIR = SEL == DKV_DK;  // the product pipeline of kint_pair.cuh
+  const int qtile = BT * D * 4;
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm + p.sm_bars);
   uint64_t* bar_full = bars;
   uint64_t* bar_empty = bars + NS;
@@ -268,36 +264,39 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
   // products dV, dK that read it complete (bar_empty)
   uint64_t* bar_emptyA = bars + 3 * NS + 8;  // [NS]
   uint64_t* bar_drain = bars + 4 * NS + 8;   // the MMA warp's clean-up commit
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 4 * NS + 9);
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + (PAIR ? PAIR_NBARS : 4 * NS + 9));
+  const PairBars B = pair_bars(bars);
   const int tid = threadIdx.x, warp = warp_id_uniform();
   const int dp = D * parts;
-  const int cK = 0, cV = dp, base = needV ? 2 * dp : dp;
-  const int cdV = base + 2 * BQ * nbuf, cdK = cdV + (doDV ? D : 0);
+  const int cK = 0, cV = dp, base = PAIR ? 128 : needV ? 2 * dp : dp;
+  const int cdV = base + 128 * (PAIR ? 2 : nbuf), cdK = cdV + (doDV ? D : 0);
   // 3xTF32 (one product per launch): the two cross terms accumulate apart from hi x hi.
   // The tensor core rounds each accumulation step toward zero, so a dK / dV row summed
   // over a whole causal column (up to T / 8 x 3 steps) drifts by about one unit in the
   // last place per step; keeping the cross terms out of the main accumulator cuts its
   // steps by three, and the two sums meet in fp32 in the epilogue.
   const int cdC = cdK + (doDK ? D : 0);
-  const int nqt = (p.T + BQ - 1) / BQ;
+  const int nqt = (p.T + BT - 1) / BT;
   const int oQ = 0, odO = parts * qtile, oQT = (needV ? 2 : 1) * parts * qtile,
             odOT = oQT + (doDK ? parts * qtile : 0);
-  const int oRec = odOT + (doDV ? parts * qtile : 0), oTab = oRec + BQ * 64;
+  const int oRec = odOT + (doDV ? parts * qtile : 0), oTab = oRec + BT * 64;
   const uint32_t tstride = (uint32_t)p.Kp * 8u;
   constexpr int W = 16;            // query columns per thread per tile
-  constexpr int NGRP = 64 / BQ;    // groups of compute warps taking tiles in turn
-  constexpr int NWT = NCOMP_KV / 32 / NGRP;  // compute warps per tile
 
-  if (tid == 0) {
+  if (PAIR && tid == 0) {
+    pair_init(B, NCOMP_KV / 32);
+    fence_mbar_init();
+  }
+  if (!PAIR && tid == 0) {
     for (int s = 0; s < NS; ++s) {
       mbar_init(&bar_full[s], 1);
       mbar_init(&bar_fullT[s], 1);
       mbar_init(&bar_empty[s], 1);
-      mbar_init(&bar_emptyA[s], NWT);
+      mbar_init(&bar_emptyA[s], NCOMP_KV / 32);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&bar_sfull[b], 1);
-      mbar_init(&bar_pready[b], NWT);
+      mbar_init(&bar_pready[b], NCOMP_KV / 32);
     }
     mbar_init(bar_done, 1);
     mbar_init(bar_ops, NCOMP_KV / 32);
@@ -325,7 +324,37 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
   // (stage ring, score buffers) run on across items.
   if (warp >= NCOMP_KV / 32) {
   setmaxnreg_dec<REG_AUX_KV>();
-  if (warp == PRODUCER_WARP_KV) {
+  if constexpr (PAIR) {
+    auto get = [&](int n) {
+      const int item = snake_item(n), kb = item / p.BH;
+      return PairItem{item % p.BH, kb * 128, kb * 128, nqt - kb * 128 / BT, item < p.nitems};
+    };
+    const PairMaps m{&maps.k, &maps.k_lo, &maps.v, &maps.v_lo, &maps.q, &maps.q_lo, &maps.dout, &maps.dout_lo,
+                     &maps.qt, &maps.qt_lo};
+    if (warp == PRODUCER_WARP_KV) {
+      pair_producer<true>(p, m, B, sm, get, [&](const PairItem& it, int q0, uint8_t* dst, uint64_t* bar) {
+        const int nrows = min(BT, p.T - q0);
+        const size_t r0 = (size_t)it.bh * p.T + q0;
+        mbar_arrive_expect_tx(bar, nrows * 64 + (CAL == CAL_MINMAX ? nrows * (int)tstride : 0));
+        bulk_load(dst, reinterpret_cast<const RowRec*>(p.rec) + r0, nrows * 64, bar);
+        if (CAL == CAL_MINMAX) bulk_load(dst + BT * 64, p.rtab + r0 * p.Kp * 2, nrows * tstride, bar);
+      });
+    } else if (warp == PRODUCER_WARP_KV + 1) {
+      pair_producer_t(p, m, B, sm, get);
+    } else if (warp == MMA_WARP_KV) {
+      pair_mma_sg(p, B, sm, get);
+    } else {
+      pair_mma_acc(p, B, sm, get, [&](uint32_t cS, uint32_t cG, const uint8_t* qt, bool first) {
+        if (p.x3) {
+          mma_tmem_smem(cdK, cS, qt, D, BT, !first);          // hi x hi
+          mma_tmem_smem(cdC, cS, qt + qtile, D, BT, !first);  // hi x lo
+          mma_tmem_smem(cdC, cG, qt, D, BT, true);            // lo x hi
+        } else {
+          mma_tmem_smem(cdK, cG, qt, D, BT, !first);
+        }
+      });
+    }
+  } else if (warp == PRODUCER_WARP_KV) {
     int gt = 0, n = 0;
     RingPos ld;  // stage of the next tile loaded
     RingPos nf, nT;  // ring positions after the last first-half and transposed-half loads issued
@@ -343,9 +372,9 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
     if (p.ops_smem && snake_item(0) < p.nitems) stage_ops(0);
     for (int item = snake_item(n); item < p.nitems && ok; item = snake_item(++n)) {
       const int kb = item / p.BH, bh = item % p.BH;
-      const int qt0 = (kb * 128) / BQ, nit = nqt - qt0;
+      const int qt0 = (kb * 128) / BT, nit = nqt - qt0;
       for (int it = 0; it < nit; ++it, ++gt, ld.next(NS)) {
-        const int s = ld.i, q0 = (qt0 + it) * BQ;
+        const int s = ld.i, q0 = (qt0 + it) * BT;
         if (gt >= NS && !mbar_wait_warp(&bar_emptyA[s], ld.ph ^ 1u, p.wait_ns, p.status, DEV_ERR_TIMEOUT_SYNC)) {
           ok = false;
           break;
@@ -353,15 +382,15 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
         uint8_t* dst = sm + p.sm_stage0 + s * p.sm_stage_bytes;
         // first the operands of S^T, g^T and the row records, then the transposed tiles
         uint64_t* b = &bar_full[s];
-        const int nrows = min(BQ, p.T - q0);
+        const int nrows = min(BT, p.T - q0);
         uint32_t bytes = (1 + (needV ? 1 : 0)) * parts * qtile + nrows * 64;
         if (CAL == CAL_MINMAX) bytes += nrows * tstride;
         mbar_arrive_expect_tx(b, bytes);
-        load_rows_tile(dst + oQ, &maps.q, b, D, BQ, 0, q0, bh);
-        if (p.x3) load_rows_tile(dst + oQ + qtile, &maps.q_lo, b, D, BQ, 0, q0, bh);
+        load_rows_tile(dst + oQ, &maps.q, b, D, BT, 0, q0, bh);
+        if (p.x3) load_rows_tile(dst + oQ + qtile, &maps.q_lo, b, D, BT, 0, q0, bh);
         if (needV) {
-          load_rows_tile(dst + odO, &maps.dout, b, D, BQ, 0, q0, bh);
-          if (p.x3) load_rows_tile(dst + odO + qtile, &maps.dout_lo, b, D, BQ, 0, q0, bh);
+          load_rows_tile(dst + odO, &maps.dout, b, D, BT, 0, q0, bh);
+          if (p.x3) load_rows_tile(dst + odO + qtile, &maps.dout_lo, b, D, BT, 0, q0, bh);
         }
         const size_t r0 = (size_t)bh * p.T + q0;
         bulk_load(dst + oRec, reinterpret_cast<const RowRec*>(p.rec) + r0, nrows * 64, b);
@@ -375,12 +404,12 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
         uint64_t* bt = &bar_fullT[s];
         mbar_arrive_expect_tx(bt, ((doDK ? 1 : 0) + (doDV ? 1 : 0)) * parts * qtile);
         if (doDK) {
-          load_rows_tile(dst + oQT, &maps.qt, bt, BQ, D, q0, 0, bh);
-          if (p.x3) load_rows_tile(dst + oQT + qtile, &maps.qt_lo, bt, BQ, D, q0, 0, bh);
+          load_rows_tile(dst + oQT, &maps.qt, bt, BT, D, q0, 0, bh);
+          if (p.x3) load_rows_tile(dst + oQT + qtile, &maps.qt_lo, bt, BT, D, q0, 0, bh);
         }
         if (doDV) {
-          load_rows_tile(dst + odOT, &maps.dot, bt, BQ, D, q0, 0, bh);
-          if (p.x3) load_rows_tile(dst + odOT + qtile, &maps.dot_lo, bt, BQ, D, q0, 0, bh);
+          load_rows_tile(dst + odOT, &maps.dot, bt, BT, D, q0, 0, bh);
+          if (p.x3) load_rows_tile(dst + odOT + qtile, &maps.dot_lo, bt, BT, D, q0, 0, bh);
         }
         nT.next(NS);
         ++cT;
@@ -412,18 +441,18 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
     RingPos is, ib, cs, cb;  // stage / buffer of the next S^T, g^T product and of the tile being finished
     bool ok = true;
     for (int item = snake_item(n); item < p.nitems && ok; item = snake_item(++n)) {
-      const int kb = item / p.BH, nit = nqt - (kb * 128) / BQ;
+      const int kb = item / p.BH, nit = nqt - (kb * 128) / BT;
       // K / V of the item in TMEM (the compute warps copy them only after the previous
       // item's last S, g were read)
       ok = mbar_wait_warp(bar_ops, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_SYNC);
       if (ok) tc_fence_after();
-      ok = ok && kv_issue_sg<BQ>(p, is, ib.i, bar_full, bar_sfull, st0, cKa, cVa, cSG, qtile, needV, odO);
+      ok = ok && kv_issue_sg(p, is, ib.i, bar_full, bar_sfull, st0, cKa, cVa, cSG, qtile, needV, odO);
       is.next(NS);
       ib.next(nbuf);
       for (int it = 0; it < nit && ok; ++it, cs.next(NS), cb.next(nbuf)) {
         const int b = cb.i, s = cs.i;
         if (nbuf == 2 && it + 1 < nit) {
-          ok = kv_issue_sg<BQ>(p, is, ib.i, bar_full, bar_sfull, st0, cKa, cVa, cSG, qtile, needV, odO);
+          ok = kv_issue_sg(p, is, ib.i, bar_full, bar_sfull, st0, cKa, cVa, cSG, qtile, needV, odO);
           is.next(NS);
           ib.next(nbuf);
         }
@@ -435,21 +464,21 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
         }
         tc_fence_after();
         const uint8_t* st = sm + p.sm_stage0 + s * p.sm_stage_bytes;
-        const uint32_t cS = tmem + base + 2 * BQ * b, cG = cS + BQ;
+        const uint32_t cS = tmem + base + 128 * b, cG = cS + 64;
         const bool acc = it > 0;
         if (p.x3) {
           const uint32_t cacc = tmem + (doDV ? cdV : cdK);
           const uint8_t* bt = st + (doDV ? odOT : oQT);
-          mma_tmem_tile<BQ>(cacc, cS, bt, D, acc);                   // hi x hi
-          mma_tmem_tile<BQ>(tmem + cdC, cS, bt + qtile, D, acc);     // hi x lo
-          mma_tmem_tile<BQ>(tmem + cdC, cG, bt, D, true);            // lo x hi
+          mma_tmem_smem(cacc, cS, bt, D, BT, acc);                   // hi x hi
+          mma_tmem_smem(tmem + cdC, cS, bt + qtile, D, BT, acc);     // hi x lo
+          mma_tmem_smem(tmem + cdC, cG, bt, D, BT, true);            // lo x hi
         } else {
-          if (doDV) mma_tmem_tile<BQ>(tmem + cdV, cS, st + odOT, D, acc);
-          if (doDK) mma_tmem_tile<BQ>(tmem + cdK, cG, st + oQT, D, acc);
+          if (doDV) mma_tmem_smem(tmem + cdV, cS, st + odOT, D, BT, acc);
+          if (doDK) mma_tmem_smem(tmem + cdK, cG, st + oQT, D, BT, acc);
         }
         mma_commit(&bar_empty[s]);
         if (nbuf == 1 && it + 1 < nit) {
-          ok = kv_issue_sg<BQ>(p, is, ib.i, bar_full, bar_sfull, st0, cKa, cVa, cSG, qtile, needV, odO);
+          ok = kv_issue_sg(p, is, ib.i, bar_full, bar_sfull, st0, cKa, cVa, cSG, qtile, needV, odO);
           is.next(NS);
           ib.next(nbuf);
         }
@@ -461,13 +490,16 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
   } else {
     setmaxnreg_inc<REG_COMP_KV>();
     const int row = tid & 127, cg = tid >> 7;
-    const int grp = NGRP == 2 ? cg >> 1 : 0;
     // K / V rows of the n-th item into TMEM (each thread a share of its key's columns: with V two
     // column groups take K and two take V), handed to the MMA warp through bar_ops: TF32 at
     // d = 64 from the tiles the producer staged in smem, otherwise from global rows.  The
     // next item's rows go in as soon as the current item's last S^T, g^T have been read, so
     // its first products run under the current item's epilogue.
     auto ops_to_tmem = [&](int n) {
+      if constexpr (PAIR) {
+        pair_ops_to_tmem(p, B, sm, n, row, cg * (D / NCG_KV), D / NCG_KV);
+        return;
+      }
       const int item = snake_item(n), kb = item / p.BH, bh = item % p.BH, j = kb * 128 + row;
       const bool isV = needV && cg >= 2;
       const int nc = needV ? D / 2 : D / NCG_KV, c0 = (needV ? cg & 1 : cg) * nc;
@@ -503,36 +535,35 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
     group_sync(BAR_COMPUTE, NCOMP_KV);  // the FWM table
     bool failed = false;
     int n = 0;
-    int gt = 0;      // tiles so far
-    RingPos cs, cb;  // stage and score buffer of the current tile
+    RingPos cs, cb;  // stage (dK alone: slot of the record ring) and score buffer of the current tile
+    const int ncs = PAIR ? 2 : NS, ncb = PAIR ? 2 : nbuf;
     for (int item = snake_item(n); item < p.nitems && !failed; item = snake_item(++n)) {
       const int kb = item / p.BH, bh = item % p.BH;
-      const int qt0 = (kb * 128) / BQ, nit = nqt - qt0;
+      const int qt0 = (kb * 128) / BT, nit = nqt - qt0;
       const int j = kb * 128 + row;
       // the tie flags are per 64 query rows
       constexpr bool ties = doDK && FULLG && CAL != CAL_SOFTMAX;
-      const int* tflags = p.tileflags + (size_t)bh * p.nqt + qt0 * BQ / 64;
+      const int* tflags = p.tileflags + (size_t)bh * p.nqt + qt0 * BT / 64;
       int tie_next = ties ? __ldg(tflags) : 0;
-      for (int it = 0; it < nit; ++it, cs.next(NS), cb.next(nbuf), ++gt) {
+      for (int it = 0; it < nit; ++it, cs.next(ncs), cb.next(ncb)) {
         // the next tile's tie flag, loaded one tile ahead
         const int tie_here = tie_next;
-        if (ties && it + 1 < nit) tie_next = __ldg(tflags + (it + 1) * BQ / 64);
-        if (NGRP == 2 && (gt & 1) != grp) continue;
+        if (ties && it + 1 < nit) tie_next = __ldg(tflags + (it + 1) * BT / 64);
         const int b = cb.i, s = cs.i;
-        const int q0 = (qt0 + it) * BQ;
-        const bool ok1 = mbar_wait(&bar_sfull[b], cb.ph, p.wait_ns, p.status, DEV_ERR_TIMEOUT_MMA);
+        const int q0 = (qt0 + it) * BT;
+        const bool ok1 = mbar_wait(PAIR ? &B.sfull[b] : &bar_sfull[b], cb.ph, p.wait_ns, p.status, DEV_ERR_TIMEOUT_MMA);
         // the stage's row records arrived with its tiles (bar_full), before the products were issued
-        const bool ok2 = ok1 && mbar_wait(&bar_full[s], cs.ph, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA);
+        const bool ok2 = ok1 && mbar_wait(PAIR ? &B.fullR[s] : &bar_full[s], cs.ph, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA);
         if (!ok2) {
           failed = true;
           break;
         }
         tc_fence_after();
-        const uint8_t* st = sm + p.sm_stage0 + s * p.sm_stage_bytes;
-        const int c0 = (NGRP == 2 ? cg & 1 : cg) * W, i0h = q0 + c0;
-        const uint32_t recs = smem_u32(st + oRec) + c0 * 64;
-        const uint32_t tabs = smem_u32(st + oTab) + c0 * tstride - 0x58000000u;
-        const int cS = base + 2 * BQ * b + c0, cG = cS + BQ;
+        const uint8_t* st = PAIR ? sm + p.sm_rec + s * p.rec_bytes : sm + p.sm_stage0 + s * p.sm_stage_bytes + oRec;
+        const int c0 = cg * W, i0h = q0 + c0;
+        const uint32_t recs = smem_u32(st) + c0 * 64;
+        const uint32_t tabs = smem_u32(st + BT * 64) + c0 * tstride - 0x58000000u;
+        const int cS = base + 128 * b + c0, cG = cS + 64;
         float sv[W], gv[W], pa[W], da[W];
         tmem_ldw<W>(lane_addr(tmem, cS), sv);
         if (needV) {
@@ -578,20 +609,15 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
           if (doDK) tmem_stw<W>(lane_addr(tmem, cG), da);
         }
         __syncwarp();
-        if ((tid & 31) == 0) mbar_arrive(&bar_emptyA[s]);  // the stage's records are read
+        if ((tid & 31) == 0) mbar_arrive(PAIR ? &B.emptyR[s] : &bar_emptyA[s]);  // the stage's records are read
         tmem_st_wait();
         tc_fence_before();
         __syncwarp();
-        if ((tid & 31) == 0) mbar_arrive(&bar_pready[b]);
+        if ((tid & 31) == 0) mbar_arrive(PAIR ? &B.pready[b] : &bar_pready[b]);
       }
-      // the next item's K / V, once this item's S^T, g^T are all complete: a group has seen its own
-      // last tile's, and waits for the other group's here (products complete in order, so the
-      // barrier's phase before is over)
-      if (NGRP == 2 && !failed && ((gt - 1) & 1) != grp)
-        failed = !mbar_wait(&bar_sfull[(gt - 1) & 1], (uint32_t)((gt - 1) >> 1) & 1u, p.wait_ns, p.status,
-                            DEV_ERR_TIMEOUT_MMA);
+      // the next item's K / V (this item's S^T, g^T have all been read: the last tile's were)
       if (!failed && snake_item(n + 1) < p.nitems) ops_to_tmem(n + 1);
-      const bool dok = !failed && mbar_wait(bar_done, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_MMA);
+      const bool dok = !failed && mbar_wait(PAIR ? B.done : bar_done, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_MMA);
       failed = group_any(BAR_COMPUTE, NCOMP_KV, !dok);
       if (!failed) {
         tc_fence_after();

@@ -155,9 +155,9 @@ __device__ __forceinline__ bool dq_issue_sg(const Params& p, RingPos stg, int b,
 // k_bwd_dq.
 // PAIR (d = 128, 3xTF32): the product pipeline of kint_pair.cuh (A1 = Q in TMEM, A2 = dO in smem,
 // K, V and K^T in rings of their own).  One score buffer and one stage of all three tiles, the
-// products and the element work in turns, took at B=4 H=16 T=2048 d=128 FWM 303 us (now 248),
-// at H=16 T=16384 d=128 MinMax K=16 LERP 4710 (now 3165), at B=8 H=12 T=1024 under 3xTF32 180
-// (now 147); tiles of 32 keys in two buffers 272, 4137 and 158.  Otherwise:
+// products and the element work in turns, took at B=4 H=16 T=2048 d=128 FWM 303 us (now 232),
+// at H=16 T=16384 d=128 MinMax K=16 LERP 4710 (now 3140), at B=8 H=12 T=1024 under 3xTF32 180
+// (now 131); tiles of 32 keys in two buffers 272, 4137 and 158.  Otherwise:
 // TMEM: Q [0, dp), dO [dp, 2dp) (dp = d, or 2d for 3xTF32 hi|lo; loaded by the
 // compute threads), then per score buffer b: S_b at 2dp + 128 b (64 columns), g_b
 // right after it (64 columns); dQ at 2dp + 128 nbuf.  dS overwrites S_b (its tf32
@@ -167,17 +167,19 @@ __device__ __forceinline__ bool dq_issue_sg(const Params& p, RingPos stg, int b,
 // ---------------------------------------------------------------------------
 // Producer warp of k_bwd_dq: TMA-stores the dQ tile of its k-th item, which the compute
 // warps staged at `tile`, and returns once it has been read out.
-__device__ __forceinline__ bool store_staged_dq(const Maps& maps, const Params& p, uint64_t* bar_ostg, int k,
+template <class Order>
+__device__ __forceinline__ bool store_staged_dq(const Maps& maps, const Params& p, const Order& sch, uint64_t* bar_ostg, int k,
                                                 const uint8_t* tile) {
   if (!mbar_wait_warp(bar_ostg, k & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_SYNC)) return false;
-  const int item = snake_item(k), qb = p.nqb - 1 - item / p.BH, bh = item % p.BH;
+  const int item = sched_item(sch, k), qb = p.nqb - 1 - item / p.BH, bh = item % p.BH;
   store_rows_tile_boxed(tile, &maps.dq, p.d, 64, qb * 128, bh, false);
   tma_store_wait_read();
   return true;
 }
 
 template <int CAL, bool FULLG, bool PAIR>
-__global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ Maps maps, const Params p) {
+__global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(const __grid_constant__ Maps maps, const Params p,
+                                                                             const __grid_constant__ ItemOrder<PAIR> sch) {
   uint8_t* sm = smem_base();
   if (p.gate != nullptr) {
     // launched on one side of a device-side decision: when the single-pass backward ran
@@ -248,7 +250,7 @@ __global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(con
 
   if (PAIR && warp >= NCOMP / 32) {
     auto get = [&](int n) {
-      const int item = snake_item(n), qb = p.nqb - 1 - item / p.BH;
+      const int item = sched_item(sch, n), qb = p.nqb - 1 - item / p.BH;
       return PairItem{item % p.BH, qb * 128, 0, min(2 * qb + 2, (p.T + BT - 1) / BT), item < p.nitems};
     };
     const PairMaps m{&maps.q, &maps.q_lo, &maps.dout, &maps.dout_lo, &maps.k, &maps.k_lo, &maps.v, &maps.v_lo,
@@ -275,14 +277,14 @@ __global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(con
     // Q / dO of this CTA's k-th item into the staging area (TF32 at d = 64)
     int staged = 0;  // staging loads issued
     auto stage_ops = [&](int k) {
-      const int it_ = snake_item(k), qb_ = p.nqb - 1 - it_ / p.BH, bh_ = it_ % p.BH;
+      const int it_ = sched_item(sch, k), qb_ = p.nqb - 1 - it_ / p.BH, bh_ = it_ % p.BH;
       mbar_arrive_expect_tx(bar_stg, 2 * 128 * D * 4);
       load_rows_tile_boxed(sm + p.sm_a, &maps.q, bar_stg, D, 128, BT, 0, qb_ * 128, bh_);
       load_rows_tile_boxed(sm + p.sm_a + 128 * D * 4, &maps.dout, bar_stg, D, 128, BT, 0, qb_ * 128, bh_);
       staged = k + 1;
     };
-    if (p.ops_smem && snake_item(0) < p.nitems) stage_ops(0);
-    for (int item = snake_item(n); item < p.nitems && ok; item = snake_item(++n)) {
+    if (p.ops_smem && sched_item(sch, 0) < p.nitems) stage_ops(0);
+    for (int item = sched_item(sch, n); item < p.nitems && ok; item = sched_item(sch, ++n)) {
       const int qb = p.nqb - 1 - item / p.BH, bh = item % p.BH;
       const int nkt = min(2 * qb + 2, (p.T + BT - 1) / BT);
       for (int kt = 0; kt < nkt; ++kt, ++gt, ld.next(NS)) {
@@ -310,9 +312,9 @@ __global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(con
         // this item's Q / dO copied out into TMEM and the previous item's dQ tile, staged in the
         // same area since, stored; both happen at the end of the previous item, so the load has
         // this whole item to land.
-        if (p.ops_smem && kt == min(nkt, NS) - 1 && snake_item(n + 1) < p.nitems) {
+        if (p.ops_smem && kt == min(nkt, NS) - 1 && sched_item(sch, n + 1) < p.nitems) {
           if (!mbar_wait_warp(bar_ops, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_SYNC) ||
-              (n >= 1 && !store_staged_dq(maps, p, bar_ostg, n - 1, sm + p.sm_a))) {
+              (n >= 1 && !store_staged_dq(maps, p, sch, bar_ostg, n - 1, sm + p.sm_a))) {
             ok = false;
             break;
           }
@@ -321,7 +323,7 @@ __global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(con
       }
     }
     // the last-but-one item's tile (the last item's is stored by the compute warps)
-    if (p.ops_smem && ok && n >= 2) store_staged_dq(maps, p, bar_ostg, n - 2, sm + p.sm_a);
+    if (p.ops_smem && ok && n >= 2) store_staged_dq(maps, p, sch, bar_ostg, n - 2, sm + p.sm_a);
     tma_store_wait_all();
     // clean-up: the last tiles issued have landed
     drain_ring(bar_full, ld, gt, NS, p.wait_ns, p.status);
@@ -334,7 +336,7 @@ __global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(con
     int n = 0, g = 0;
     RingPos is, ib;  // stage and buffer of the next S, g product
     bool ok = true;
-    for (int item = snake_item(n); item < p.nitems && ok; item = snake_item(++n)) {
+    for (int item = sched_item(sch, n); item < p.nitems && ok; item = sched_item(sch, ++n)) {
       const int qb = p.nqb - 1 - item / p.BH;
       const int nkt = min(2 * qb + 2, (p.T + BT - 1) / BT);
       // Q / dO of the item in TMEM (copied by the compute warps once the previous item's
@@ -356,7 +358,7 @@ __global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(con
     RingPos cs, cb;  // stage and buffer of the tile being finished
     int n = 0;
     bool ok = true;
-    for (int item = snake_item(n); item < p.nitems && ok; item = snake_item(++n)) {
+    for (int item = sched_item(sch, n); item < p.nitems && ok; item = sched_item(sch, ++n)) {
       const int qb = p.nqb - 1 - item / p.BH;
       const int nkt = min(2 * qb + 2, (p.T + BT - 1) / BT);
       for (int kt = 0; kt < nkt && ok; ++kt, cs.next(NS), cb.next(nbuf)) {
@@ -395,7 +397,7 @@ __global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(con
         pair_ops_to_tmem(p, B, sm, n, row, cg * (D / NCG), D / NCG);
         return;
       }
-      const int item = snake_item(n);
+      const int item = sched_item(sch, n);
       const int qb = p.nqb - 1 - item / p.BH, bh = item % p.BH, i = qb * 128 + row;
       if (p.ops_smem) {
         if (mbar_wait(bar_stg, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA))
@@ -419,7 +421,7 @@ __global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(con
     const bool prob = (p.recon == REC_NEAREST && p.ste == 1 && !gridless(CAL));
     const uint32_t rslot = smem_u32(sm + p.sm_rstat) + 4u * (uint32_t)tid;
     auto prefetch_row_stats = [&](int n) {
-      const int item = snake_item(n);
+      const int item = sched_item(sch, n);
       const int i = (p.nqb - 1 - item / p.BH) * 128 + row;
       if (i < p.T) {
         const size_t rw = (size_t)(item % p.BH) * p.T + i;
@@ -435,7 +437,7 @@ __global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(con
     };
     auto load_row_stats = [&](int n) {
       RowIn r;
-      const int item = snake_item(n);
+      const int item = sched_item(sch, n);
       const int i = (p.nqb - 1 - item / p.BH) * 128 + row;
       asm volatile("cp.async.wait_all;" ::: "memory");
       if (i < p.T) {
@@ -455,12 +457,12 @@ __global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(con
     RingPos cb, cs;  // score buffer and stage of the current tile
     bool failed = false;
     RowIn nx;
-    if (snake_item(0) < p.nitems) {
+    if (sched_item(sch, 0) < p.nitems) {
       prefetch_row_stats(0);
       ops_to_tmem(0);
       nx = load_row_stats(0);
     }
-    for (int item = snake_item(n); item < p.nitems && !failed; item = snake_item(++n)) {
+    for (int item = sched_item(sch, n); item < p.nitems && !failed; item = sched_item(sch, ++n)) {
       // ---- set-up: row constants, grid table (the operands are in TMEM already) ----
       const int qb = p.nqb - 1 - item / p.BH, bh = item % p.BH;
       const int nkt = min(2 * qb + 2, (p.T + BT - 1) / BT);
@@ -469,7 +471,7 @@ __global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(con
       const size_t rw = (size_t)bh * p.T + (row_ok ? i : 0);
       const float M = nx.M, m = nx.m, Wf = nx.Wf, Ws = nx.Ws, Dg = nx.Dg;
       const int nmax = nx.nmax, nmin = nx.nmin, amax = nx.amax, amin = nx.amin;
-      if (snake_item(n + 1) < p.nitems) prefetch_row_stats(n + 1);  // (the slot was just read)
+      if (sched_item(sch, n + 1) < p.nitems) prefetch_row_stats(n + 1);  // (the slot was just read)
       const RowGrid g = row_grid(p, M, m);
       if constexpr (fwm_like(CAL)) {  // the same for every item
         if (n == 0 && tid < 2 * Kq + 1 + kHalfTail)
@@ -568,7 +570,7 @@ __global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(con
       }
       // the next item's Q / dO (this item's S, g have all been read: the last tile's were)
       // and its row statistics
-      if (!failed && snake_item(n + 1) < p.nitems) {
+      if (!failed && sched_item(sch, n + 1) < p.nitems) {
         ops_to_tmem(n + 1);
         nx = load_row_stats(n + 1);
       }
@@ -615,7 +617,7 @@ __global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(con
         // that the next item's Q / dO are in TMEM; the producer stores it before it stages
         // the item after next), or, for the last item, in the idle stage ring (stored here).
         // Without the staging area (3xTF32, d = 128) straight to global memory.
-        const bool last = snake_item(n + 1) >= p.nitems;
+        const bool last = sched_item(sch, n + 1) >= p.nitems;
         uint8_t* stg = last ? sm + p.sm_stage0 : sm + p.sm_a;
         for (int c = cg * (D / NCG); c < (cg + 1) * (D / NCG); c += 32) {
           // the arg-extremum key rows (128 bytes of each: this column half).  With the staging
@@ -748,29 +750,29 @@ cudaError_t launch_kcum(const float* K, float* C, int BH, int T, int d, cudaStre
 }
 
 template <bool PAIR>
-static cudaError_t launch_dq_t(const Maps& maps, const Params& p, int smem_bytes, cudaStream_t s) {
+static cudaError_t launch_dq_t(const Maps& maps, const Params& p, int smem_bytes, cudaStream_t s, const ItemOrder<PAIR>& sch) {
   const dim3 grid((unsigned)p.ngrid);
   const int nthr = PAIR ? NTHR_DQ + 32 : NTHR_DQ;
   const bool full = p.grad != GRAD_DETACH && p.grad != GRAD_DETACH_PROJ;
-  if (p.calib == CAL_SOFTMAX) return launch3(k_bwd_dq<CAL_SOFTMAX, false, PAIR>, grid, maps, p, smem_bytes, s, nthr);
+  if (p.calib == CAL_SOFTMAX) return launch3(k_bwd_dq<CAL_SOFTMAX, false, PAIR>, grid, maps, p, smem_bytes, s, sch, nthr);
   if (p.calib == CAL_EXP8)
-    return full ? launch3(k_bwd_dq<CAL_EXP8, true, PAIR>, grid, maps, p, smem_bytes, s, nthr)
-                : launch3(k_bwd_dq<CAL_EXP8, false, PAIR>, grid, maps, p, smem_bytes, s, nthr);
+    return full ? launch3(k_bwd_dq<CAL_EXP8, true, PAIR>, grid, maps, p, smem_bytes, s, sch, nthr)
+                : launch3(k_bwd_dq<CAL_EXP8, false, PAIR>, grid, maps, p, smem_bytes, s, sch, nthr);
   if (p.calib == CAL_EXPB)
-    return full ? launch3(k_bwd_dq<CAL_EXPB, true, PAIR>, grid, maps, p, smem_bytes, s, nthr)
-                : launch3(k_bwd_dq<CAL_EXPB, false, PAIR>, grid, maps, p, smem_bytes, s, nthr);
+    return full ? launch3(k_bwd_dq<CAL_EXPB, true, PAIR>, grid, maps, p, smem_bytes, s, sch, nthr)
+                : launch3(k_bwd_dq<CAL_EXPB, false, PAIR>, grid, maps, p, smem_bytes, s, sch, nthr);
   if (p.calib == CAL_MINMAX)
-    return full ? launch3(k_bwd_dq<CAL_MINMAX, true, PAIR>, grid, maps, p, smem_bytes, s, nthr)
-                : launch3(k_bwd_dq<CAL_MINMAX, false, PAIR>, grid, maps, p, smem_bytes, s, nthr);
+    return full ? launch3(k_bwd_dq<CAL_MINMAX, true, PAIR>, grid, maps, p, smem_bytes, s, sch, nthr)
+                : launch3(k_bwd_dq<CAL_MINMAX, false, PAIR>, grid, maps, p, smem_bytes, s, sch, nthr);
   if (p.calib == CAL_FWMR)
-    return full ? launch3(k_bwd_dq<CAL_FWMR, true, PAIR>, grid, maps, p, smem_bytes, s, nthr)
-                : launch3(k_bwd_dq<CAL_FWMR, false, PAIR>, grid, maps, p, smem_bytes, s, nthr);
-  return full ? launch3(k_bwd_dq<CAL_FWM, true, PAIR>, grid, maps, p, smem_bytes, s, nthr)
-              : launch3(k_bwd_dq<CAL_FWM, false, PAIR>, grid, maps, p, smem_bytes, s, nthr);
+    return full ? launch3(k_bwd_dq<CAL_FWMR, true, PAIR>, grid, maps, p, smem_bytes, s, sch, nthr)
+                : launch3(k_bwd_dq<CAL_FWMR, false, PAIR>, grid, maps, p, smem_bytes, s, sch, nthr);
+  return full ? launch3(k_bwd_dq<CAL_FWM, true, PAIR>, grid, maps, p, smem_bytes, s, sch, nthr)
+              : launch3(k_bwd_dq<CAL_FWM, false, PAIR>, grid, maps, p, smem_bytes, s, sch, nthr);
 }
 
-cudaError_t launch_bwd_dq(const Maps& maps, const Params& p, int smem_bytes, cudaStream_t s) {
-  return p.pair ? launch_dq_t<true>(maps, p, smem_bytes, s) : launch_dq_t<false>(maps, p, smem_bytes, s);
+cudaError_t launch_bwd_dq(const Maps& maps, const Params& p, int smem_bytes, cudaStream_t s, const Sched& sch) {
+  return p.pair ? launch_dq_t<true>(maps, p, smem_bytes, s, sch) : launch_dq_t<false>(maps, p, smem_bytes, s, SnakeOrder{});
 }
 
 }  // namespace kint

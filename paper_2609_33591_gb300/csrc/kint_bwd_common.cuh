@@ -15,12 +15,12 @@ __device__ __forceinline__ int4 lds_i4(uint32_t addr) {
   return v;
 }
 
-template <class K>
+template <class K, class Order>
 static cudaError_t launch3(K kern, dim3 grid, const Maps& maps, const Params& p, int smem_bytes, cudaStream_t s,
-                           int nthr = NTHR) {
+                           const Order& sch, int nthr) {
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
   if (e != cudaSuccess) return e;
-  return launch_pdl(kern, grid, dim3(nthr), smem_bytes, s, maps, p);
+  return launch_pdl(kern, grid, dim3(nthr), smem_bytes, s, maps, p, sch);
 }
 
 }  // namespace kint

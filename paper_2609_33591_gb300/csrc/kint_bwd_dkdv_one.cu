@@ -3,7 +3,7 @@
 
 namespace kint {
 
-template cudaError_t launch_bwd_dkdv_t<false, DKV_DV>(const Maps&, const Params&, int, cudaStream_t);
-template cudaError_t launch_bwd_dkdv_t<false, DKV_DK>(const Maps&, const Params&, int, cudaStream_t);
+template cudaError_t launch_bwd_dkdv_t<false, DKV_DV>(const Maps&, const Params&, int, cudaStream_t, const SnakeOrder&);
+template cudaError_t launch_bwd_dkdv_t<false, DKV_DK>(const Maps&, const Params&, int, cudaStream_t, const Sched&);
 
 }  // namespace kint

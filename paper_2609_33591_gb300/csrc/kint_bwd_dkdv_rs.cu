@@ -6,6 +6,6 @@
 
 namespace kint {
 
-template cudaError_t launch_bwd_dkdv_t<true, DKV_BOTH>(const Maps&, const Params&, int, cudaStream_t);
+template cudaError_t launch_bwd_dkdv_t<true, DKV_BOTH>(const Maps&, const Params&, int, cudaStream_t, const SnakeOrder&);
 
 }  // namespace kint

@@ -205,10 +205,11 @@ __device__ __forceinline__ bool kv_issue_sg(const Params& p, RingPos stg, int b,
 
 // Producer warp of k_bwd_dkdv: TMA-stores the dV / dK tiles of its k-th item, which the
 // compute warps staged at `tile` (dV, then dK), and returns once they have been read out.
-__device__ __forceinline__ bool store_staged_dkdv(const Maps& maps, const Params& p, uint64_t* bar_ostg, int k,
+template <class Order>
+__device__ __forceinline__ bool store_staged_dkdv(const Maps& maps, const Params& p, const Order& sch, uint64_t* bar_ostg, int k,
                                                   const uint8_t* tile, bool doDV, bool doDK) {
   if (!mbar_wait_warp(bar_ostg, k & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_SYNC)) return false;
-  const int item = snake_item(k), kb = item / p.BH, bh = item % p.BH;
+  const int item = sched_item(sch, k), kb = item / p.BH, bh = item % p.BH;
   if (doDV) store_rows_tile_boxed(tile, &maps.dv, p.d, 64, kb * 128, bh, false);
   if (doDK) store_rows_tile_boxed(tile + 128 * p.d * 4, &maps.dk, p.d, 64, kb * 128, bh, false);
   tma_store_wait_read();
@@ -229,13 +230,14 @@ __device__ __forceinline__ bool store_staged_dkdv(const Maps& maps, const Params
 // What bounds it: the issue of the products by one warp, then the shared-memory loads of the
 // row records.
 // Measured on GB300 against eight compute warps and stages of all four tiles: B=4 H=16 T=2048
-// d=128 FWM Weight-STE dV 340 -> 178 us, dK 403 -> 238; H=16 T=16384 d=128 MinMax K=16 LERP
-// 5097 -> 2250, 5878 -> 3047; 3xTF32 B=8 H=12 T=1024 168 -> 98, 203 -> 131; MinMax B=4 H=12
+// d=128 FWM Weight-STE dV 340 -> 178 us, dK 403 -> 231; H=16 T=16384 d=128 MinMax K=16 LERP
+// 5097 -> 2223, 5878 -> 3010; 3xTF32 B=8 H=12 T=1024 168 -> 98, 203 -> 127; MinMax B=4 H=12
 // T=1024 d=64 (both products) 73.6 -> 71.6.  (dK in the stage ring with 32-query tiles: 313,
 // 3785 and 170.)
 // ---------------------------------------------------------------------------
 template <int CAL, int REC, bool FULLG, bool PROJ, bool RS, int SEL>
-__global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__ Maps maps, const Params p) {
+__global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__ Maps maps, const Params p,
+                                                         const __grid_constant__ ItemOrder<SEL == DKV_DK> sch) {
   uint8_t* sm = smem_base();
   if (p.gate != nullptr) {
     // launched on one side of a device-side decision: when the single-pass backward ran
@@ -320,13 +322,13 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
   constexpr uint32_t tmem = 0;
 
   // Work items are (128-key block kb, head) pairs, longest first (kb = 0 meets every
-  // query tile); a CTA takes the items snake_item(0), snake_item(1), ...  Tile counters
+  // query tile); a CTA takes the items sched_item(sch, 0), sched_item(sch, 1), ...  Tile counters
   // (stage ring, score buffers) run on across items.
   if (warp >= NCOMP_KV / 32) {
   setmaxnreg_dec<REG_AUX_KV>();
   if constexpr (PAIR) {
     auto get = [&](int n) {
-      const int item = snake_item(n), kb = item / p.BH;
+      const int item = sched_item(sch, n), kb = item / p.BH;
       return PairItem{item % p.BH, kb * 128, kb * 128, nqt - kb * 128 / BT, item < p.nitems};
     };
     const PairMaps m{&maps.k, &maps.k_lo, &maps.v, &maps.v_lo, &maps.q, &maps.q_lo, &maps.dout, &maps.dout_lo,
@@ -363,14 +365,14 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
     // K / V of this CTA's k-th item into the staging area (TF32 at d = 64)
     int staged = 0;  // staging loads issued
     auto stage_ops = [&](int k) {
-      const int it_ = snake_item(k), kb_ = it_ / p.BH, bh_ = it_ % p.BH;
+      const int it_ = sched_item(sch, k), kb_ = it_ / p.BH, bh_ = it_ % p.BH;
       mbar_arrive_expect_tx(bar_stg, (needV ? 2 : 1) * 128 * D * 4);
       load_rows_tile_boxed(sm + p.sm_a, &maps.k, bar_stg, D, 128, BT, 0, kb_ * 128, bh_);
       if (needV) load_rows_tile_boxed(sm + p.sm_a + 128 * D * 4, &maps.v, bar_stg, D, 128, BT, 0, kb_ * 128, bh_);
       staged = k + 1;
     };
-    if (p.ops_smem && snake_item(0) < p.nitems) stage_ops(0);
-    for (int item = snake_item(n); item < p.nitems && ok; item = snake_item(++n)) {
+    if (p.ops_smem && sched_item(sch, 0) < p.nitems) stage_ops(0);
+    for (int item = sched_item(sch, n); item < p.nitems && ok; item = sched_item(sch, ++n)) {
       const int kb = item / p.BH, bh = item % p.BH;
       const int qt0 = (kb * 128) / BT, nit = nqt - qt0;
       for (int it = 0; it < nit; ++it, ++gt, ld.next(NS)) {
@@ -417,9 +419,9 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
         // this item's K / V copied out into TMEM and the previous item's dV / dK tiles, staged in
         // the same area since, stored; both happen at the end of the previous item, so the load
         // has this whole item to land.
-        if (p.ops_smem && it == min(nit, NS) - 1 && snake_item(n + 1) < p.nitems) {
+        if (p.ops_smem && it == min(nit, NS) - 1 && sched_item(sch, n + 1) < p.nitems) {
           if (!mbar_wait_warp(bar_ops, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_SYNC) ||
-              (n >= 1 && !store_staged_dkdv(maps, p, bar_ostg, n - 1, sm + p.sm_a, doDV, doDK))) {
+              (n >= 1 && !store_staged_dkdv(maps, p, sch, bar_ostg, n - 1, sm + p.sm_a, doDV, doDK))) {
             ok = false;
             break;
           }
@@ -428,7 +430,7 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
       }
     }
     // the last-but-one item's tiles (the last item's are stored by the compute warps)
-    if (p.ops_smem && ok && n >= 2) store_staged_dkdv(maps, p, bar_ostg, n - 2, sm + p.sm_a, doDV, doDK);
+    if (p.ops_smem && ok && n >= 2) store_staged_dkdv(maps, p, sch, bar_ostg, n - 2, sm + p.sm_a, doDV, doDK);
     tma_store_wait_all();
     // clean-up: the last tiles issued have landed
     drain_ring(bar_full, nf, cf, NS, p.wait_ns, p.status);
@@ -440,7 +442,7 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
     int n = 0;
     RingPos is, ib, cs, cb;  // stage / buffer of the next S^T, g^T product and of the tile being finished
     bool ok = true;
-    for (int item = snake_item(n); item < p.nitems && ok; item = snake_item(++n)) {
+    for (int item = sched_item(sch, n); item < p.nitems && ok; item = sched_item(sch, ++n)) {
       const int kb = item / p.BH, nit = nqt - (kb * 128) / BT;
       // K / V of the item in TMEM (the compute warps copy them only after the previous
       // item's last S, g were read)
@@ -500,7 +502,7 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
         pair_ops_to_tmem(p, B, sm, n, row, cg * (D / NCG_KV), D / NCG_KV);
         return;
       }
-      const int item = snake_item(n), kb = item / p.BH, bh = item % p.BH, j = kb * 128 + row;
+      const int item = sched_item(sch, n), kb = item / p.BH, bh = item % p.BH, j = kb * 128 + row;
       const bool isV = needV && cg >= 2;
       const int nc = needV ? D / 2 : D / NCG_KV, c0 = (needV ? cg & 1 : cg) * nc;
       const bool ok = !p.ops_smem || mbar_wait(bar_stg, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA);
@@ -519,7 +521,7 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
       __syncwarp();
       if ((tid & 31) == 0) mbar_arrive(bar_ops);
     };
-    if (snake_item(0) < p.nitems) ops_to_tmem(0);
+    if (sched_item(sch, 0) < p.nitems) ops_to_tmem(0);
     // FWM Nearest: the half-bin table (entry q at sm_table + 8 (q + 2)) and the doubled
     // position; FWM LERP: the pair table, entry r at sm_table + 8 r (0x4B000000 * 8 =
     // 0x58000000 mod 2^32)
@@ -537,7 +539,7 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
     int n = 0;
     RingPos cs, cb;  // stage (dK alone: slot of the record ring) and score buffer of the current tile
     const int ncs = PAIR ? 2 : NS, ncb = PAIR ? 2 : nbuf;
-    for (int item = snake_item(n); item < p.nitems && !failed; item = snake_item(++n)) {
+    for (int item = sched_item(sch, n); item < p.nitems && !failed; item = sched_item(sch, ++n)) {
       const int kb = item / p.BH, bh = item % p.BH;
       const int qt0 = (kb * 128) / BT, nit = nqt - qt0;
       const int j = kb * 128 + row;
@@ -616,7 +618,7 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
         if ((tid & 31) == 0) mbar_arrive(PAIR ? &B.pready[b] : &bar_pready[b]);
       }
       // the next item's K / V (this item's S^T, g^T have all been read: the last tile's were)
-      if (!failed && snake_item(n + 1) < p.nitems) ops_to_tmem(n + 1);
+      if (!failed && sched_item(sch, n + 1) < p.nitems) ops_to_tmem(n + 1);
       const bool dok = !failed && mbar_wait(PAIR ? B.done : bar_done, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_MMA);
       failed = group_any(BAR_COMPUTE, NCOMP_KV, !dok);
       if (!failed) {
@@ -626,7 +628,7 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
         // the item after next), or, for the last item, in the idle stage ring (stored here).
         // Without the staging area (3xTF32, d = 128, one-product launches) straight to
         // global memory.
-        const bool last = snake_item(n + 1) >= p.nitems;
+        const bool last = sched_item(sch, n + 1) >= p.nitems;
         uint8_t* stg = last ? sm + p.sm_stage0 : sm + p.sm_a;
         for (int pass = 0; pass < 2; ++pass) {
           if (pass == 0 ? !doDV : !doDK) continue;
@@ -678,42 +680,43 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
 // Every backward mode of one calibration and reconstruction; softmax ignores the mode, and a dV
 // launch does not depend on it.
 template <int CAL, int REC, bool RS, int SEL>
-cudaError_t launch_dkdv_modes(dim3 grid, const Maps& maps, const Params& p, int smem_bytes, cudaStream_t s) {
+cudaError_t launch_dkdv_modes(dim3 grid, const Maps& maps, const Params& p, int smem_bytes, cudaStream_t s,
+                              const ItemOrder<SEL == DKV_DK>& sch) {
   if constexpr (CAL == CAL_SOFTMAX || SEL == DKV_DV) {
-    return launch3(k_bwd_dkdv<CAL, REC, false, false, RS, SEL>, grid, maps, p, smem_bytes, s, NTHR_KV);
+    return launch3(k_bwd_dkdv<CAL, REC, false, false, RS, SEL>, grid, maps, p, smem_bytes, s, sch, NTHR_KV);
   } else {
     const bool proj = p.grad == GRAD_DETACH_PROJ, full = p.grad != GRAD_DETACH && !proj;
-    return full ? launch3(k_bwd_dkdv<CAL, REC, true, false, RS, SEL>, grid, maps, p, smem_bytes, s, NTHR_KV)
-           : proj ? launch3(k_bwd_dkdv<CAL, REC, false, true, RS, SEL>, grid, maps, p, smem_bytes, s, NTHR_KV)
-                  : launch3(k_bwd_dkdv<CAL, REC, false, false, RS, SEL>, grid, maps, p, smem_bytes, s, NTHR_KV);
+    return full ? launch3(k_bwd_dkdv<CAL, REC, true, false, RS, SEL>, grid, maps, p, smem_bytes, s, sch, NTHR_KV)
+           : proj ? launch3(k_bwd_dkdv<CAL, REC, false, true, RS, SEL>, grid, maps, p, smem_bytes, s, sch, NTHR_KV)
+                  : launch3(k_bwd_dkdv<CAL, REC, false, false, RS, SEL>, grid, maps, p, smem_bytes, s, sch, NTHR_KV);
   }
 }
 
 // The dK/dV launch of p's configuration.  RS: the instantiation that also accumulates the
 // per-row sums of dS and |dS| (p.dsum_out, p.dabs_out); SEL: its products (DkvSel).
 template <bool RS, int SEL>
-cudaError_t launch_bwd_dkdv_t(const Maps& maps, const Params& p, int smem_bytes, cudaStream_t s) {
+cudaError_t launch_bwd_dkdv_t(const Maps& maps, const Params& p, int smem_bytes, cudaStream_t s, const ItemOrder<SEL == DKV_DK>& sch) {
   const dim3 grid((unsigned)p.ngrid);
   const bool near = p.recon == REC_NEAREST;
   switch (p.calib) {
-    case CAL_SOFTMAX: return launch_dkdv_modes<CAL_SOFTMAX, REC_LERP, RS, SEL>(grid, maps, p, smem_bytes, s);
-    case CAL_EXP8: return launch_dkdv_modes<CAL_EXP8, REC_LERP, RS, SEL>(grid, maps, p, smem_bytes, s);
-    case CAL_EXPB: return launch_dkdv_modes<CAL_EXPB, REC_LERP, RS, SEL>(grid, maps, p, smem_bytes, s);
+    case CAL_SOFTMAX: return launch_dkdv_modes<CAL_SOFTMAX, REC_LERP, RS, SEL>(grid, maps, p, smem_bytes, s, sch);
+    case CAL_EXP8: return launch_dkdv_modes<CAL_EXP8, REC_LERP, RS, SEL>(grid, maps, p, smem_bytes, s, sch);
+    case CAL_EXPB: return launch_dkdv_modes<CAL_EXPB, REC_LERP, RS, SEL>(grid, maps, p, smem_bytes, s, sch);
     case CAL_MINMAX:
-      return near ? launch_dkdv_modes<CAL_MINMAX, REC_NEAREST, RS, SEL>(grid, maps, p, smem_bytes, s)
-                  : launch_dkdv_modes<CAL_MINMAX, REC_LERP, RS, SEL>(grid, maps, p, smem_bytes, s);
+      return near ? launch_dkdv_modes<CAL_MINMAX, REC_NEAREST, RS, SEL>(grid, maps, p, smem_bytes, s, sch)
+                  : launch_dkdv_modes<CAL_MINMAX, REC_LERP, RS, SEL>(grid, maps, p, smem_bytes, s, sch);
     case CAL_FWMR:
-      return near ? launch_dkdv_modes<CAL_FWMR, REC_NEAREST, RS, SEL>(grid, maps, p, smem_bytes, s)
-                  : launch_dkdv_modes<CAL_FWMR, REC_LERP, RS, SEL>(grid, maps, p, smem_bytes, s);
+      return near ? launch_dkdv_modes<CAL_FWMR, REC_NEAREST, RS, SEL>(grid, maps, p, smem_bytes, s, sch)
+                  : launch_dkdv_modes<CAL_FWMR, REC_LERP, RS, SEL>(grid, maps, p, smem_bytes, s, sch);
     default:
-      return near ? launch_dkdv_modes<CAL_FWM, REC_NEAREST, RS, SEL>(grid, maps, p, smem_bytes, s)
-                  : launch_dkdv_modes<CAL_FWM, REC_LERP, RS, SEL>(grid, maps, p, smem_bytes, s);
+      return near ? launch_dkdv_modes<CAL_FWM, REC_NEAREST, RS, SEL>(grid, maps, p, smem_bytes, s, sch)
+                  : launch_dkdv_modes<CAL_FWM, REC_LERP, RS, SEL>(grid, maps, p, smem_bytes, s, sch);
   }
 }
-extern template cudaError_t launch_bwd_dkdv_t<false, DKV_BOTH>(const Maps&, const Params&, int, cudaStream_t);
-extern template cudaError_t launch_bwd_dkdv_t<false, DKV_DV>(const Maps&, const Params&, int, cudaStream_t);
-extern template cudaError_t launch_bwd_dkdv_t<false, DKV_DK>(const Maps&, const Params&, int, cudaStream_t);
-extern template cudaError_t launch_bwd_dkdv_t<true, DKV_BOTH>(const Maps&, const Params&, int, cudaStream_t);
-extern template cudaError_t launch_bwd_dkdv_t<true, DKV_DK>(const Maps&, const Params&, int, cudaStream_t);
+extern template cudaError_t launch_bwd_dkdv_t<false, DKV_BOTH>(const Maps&, const Params&, int, cudaStream_t, const SnakeOrder&);
+extern template cudaError_t launch_bwd_dkdv_t<false, DKV_DV>(const Maps&, const Params&, int, cudaStream_t, const SnakeOrder&);
+extern template cudaError_t launch_bwd_dkdv_t<false, DKV_DK>(const Maps&, const Params&, int, cudaStream_t, const Sched&);
+extern template cudaError_t launch_bwd_dkdv_t<true, DKV_BOTH>(const Maps&, const Params&, int, cudaStream_t, const SnakeOrder&);
+extern template cudaError_t launch_bwd_dkdv_t<true, DKV_DK>(const Maps&, const Params&, int, cudaStream_t, const Sched&);
 
 }  // namespace kint

@@ -167,6 +167,11 @@ __device__ __forceinline__ int sched_item(const Sched& s, int n) {
   return k < s.off[blockIdx.x + 1] ? (int)s.idx[k] : 0x7fffffff;
 }
 
+// The snake order as an argument type of its own, for the launches that have no host schedule
+// (a Sched is 4.7 KB of launch parameters).
+struct SnakeOrder {};
+__device__ __forceinline__ int sched_item(const SnakeOrder&, int n) { return snake_item(n); }
+
 // item / BH (the block of a (block, head) item): the high half of item * ceil(2^64 / BH), which
 // is exact for item * BH < 2^64; a plain division costs a persistent kernel's warps several
 // hundred cycles per item.

@@ -60,8 +60,8 @@ cudaError_t launch_pdl(Kern kern, dim3 grid, dim3 block, int smem, cudaStream_t 
 // sch: the host item schedule of the persistent kernels (Sched::n == 0: snake order)
 cudaError_t launch_fwd_stats(const Maps& maps, const Params& p, int smem_bytes, cudaStream_t s, const Sched& sch);
 cudaError_t launch_fwd_main(const Maps& maps, const Params& p, int smem_bytes, cudaStream_t s, const Sched& sch);
-cudaError_t launch_bwd_dq(const Maps& maps, const Params& p, int smem_bytes, cudaStream_t s);
-cudaError_t launch_bwd_dkdv(const Maps& maps, const Params& p, int smem_bytes, cudaStream_t s);
+cudaError_t launch_bwd_dq(const Maps& maps, const Params& p, int smem_bytes, cudaStream_t s, const Sched& sch);
+cudaError_t launch_bwd_dkdv(const Maps& maps, const Params& p, int smem_bytes, cudaStream_t s, const Sched& sch);
 // Geometry probe: per-row span, width, softmax entropy, share below -6, top-bucket mass,
 // effective buckets and total variation to softmax, into p.probe
 cudaError_t launch_fwd_probe(const Maps& maps, const Params& p, int smem_bytes, cudaStream_t s);

@@ -41,8 +41,9 @@ struct Maps {
 
 // Static item schedule of a persistent kernel, computed on the host (longest processing
 // time first over the launch's CTAs): CTA c takes the items idx[off[c]] .. idx[off[c+1] - 1]
-// in that order.  n == 0: no schedule, the snake order (snake_item) instead.
-constexpr int SCHED_MAX_CTAS = 304, SCHED_MAX_ITEMS = 1536;
+// in that order.  n == 0: no schedule, the snake order (snake_item) instead.  2048 items: 16 heads
+// of 16384 rows.
+constexpr int SCHED_MAX_CTAS = 304, SCHED_MAX_ITEMS = 2048;
 struct Sched {
   int n;
   uint16_t off[SCHED_MAX_CTAS + 1];

@@ -18,6 +18,7 @@ X3, TF = kint.PREC_3XTF32, kint.PREC_TF32
 
 @pytest.mark.parametrize("BH,T,d,c,K,r,s,g,prec", [
     (160, 130, 128, FW, 4, NE, WE, FU, TF),  # d = 128: several items per CTA, odd tile counts
+    (420, 130, 128, FW, 4, NE, WE, FU, TF),  # tiles of all heads past the L2 share: groups of heads
     (90, 193, 128, MM, 16, LE, WE, FU, TF),  # two slots of the second operand beside pair tables
     (80, 257, 128, MM, 32, NE, PR, FU, TF),  # one slot beside the largest tables
     (170, 65, 128, SM, 1, LE, WE, FU, TF),   # a one-row last tile

@@ -553,7 +553,7 @@ int plan_fused(Params& p) {
   p.sm_stage_bytes = 4 * qtile + 64 * 16;
   p.sm_v = p.sm_stage0 + p.nstage * p.sm_stage_bytes;
   p.sm_kt = p.sm_v + 128 * 64 * 4;
-  p.sm_ostage = p.sm_kt + 128 * 64 * 4;  // the compute warps' 1 KB dQ reduce slices
+  p.sm_ostage = p.sm_kt + 128 * 64 * 4;  // the output warps' four 1 KB dQ reduce slices each
   p.sm_table = p.sm_ostage + 16 * 1024;
   const int total = std::max(finish_plan(p, p.sm_table + 2048, 5 * p.nstage + 13), kOneCtaPerSm);
   if (total > kSmemLimit) return -1;

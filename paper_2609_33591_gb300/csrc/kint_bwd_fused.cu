@@ -106,8 +106,8 @@ __device__ __forceinline__ void fused_chunk(const float (&sv)[W], const float (&
   }
 }
 
-// The calling warp holds v[c] for 16 query rows r0 + c at 32 keys (one per lane): the
-// 32-key sum of each row is added to dst[r0 + c] (butterfly reduce-scatter: the xor-16
+// The calling warp holds v[c] for 16 query rows r0 + c, a part of the row per lane: the
+// sum over the lanes of each row is added to dst[r0 + c] (butterfly reduce-scatter: the xor-16
 // step keeps rows 8..15 in the upper half-warp, xor-8 rows +4, xor-4 +2, xor-2 +1, and
 // xor-1 adds the pair; the even lane of each pair adds it).
 __device__ __forceinline__ void rowsum_red(const float (&v)[16], float* dst, size_t r0, int nvalid) {
@@ -132,8 +132,8 @@ __device__ __forceinline__ void rowsum_red(const float (&v)[16], float* dst, siz
 
 
 // ---------------------------------------------------------------------------
-// k_bwd_fused (640 threads: 16 compute warps, the MMA warp, two producer warps, an idle warp).  Work
-// items are (128-key block kb, head) pairs, longest first; a CTA
+// k_bwd_fused (768 threads: 16 compute warps, the MMA warp, two producer warps, an idle warp,
+// four output warps).  Work items are (128-key block kb, head) pairs, longest first; a CTA
 // takes sched_item(sch, 0), sched_item(sch, 1), ...  Thread t (< 512) owns key j = kb*128 + t%128
 // (TMEM lane t%128) and the 16 query columns 16 (t/128) .. +15 of each 64-query tile:
 // four compute warps per SM sub-partition, so that one warp's latencies (TMEM and
@@ -151,17 +151,25 @@ __device__ __forceinline__ void rowsum_red(const float (&v)[16], float* dst, siz
 // operand of g^T) also stages the next item's K rows on their way into TMEM; its K^T tile
 // (B operand of dQ), which the compute warps write from the K rows in TMEM, stages the dV,
 // dK rows of the epilogue (32 keys x 16 columns per warp, 64-byte swizzle) for TMA stores,
-// after which each warp writes its part of the next item's K^T there; each compute warp
-// has a 1 KB slice for its 16 rows x 16 columns of the dQ partial (64-byte swizzle), added
-// to dQ by a TMA reduce.
+// after which each warp writes its part of the next item's K^T there; each output warp
+// has four 1 KB slices for its 16 rows x 64 columns of the dQ partial (64-byte swizzle), added
+// to dQ by TMA reduces.
+// What bounds it: shared memory.  Per tile of 64 x 128 the products read 160 KB of operands from
+// it, the TMA loads write 64 KB, and the row records (a broadcast LDS.128 per key column and
+// warp, two wavefronts), tables, dS stores and TMEM traffic take some 2500 wavefronts, of about
+// 3600 cycles.  Row sums and dQ partial by the output warps, not the compute warps (a butterfly
+// over the keys in registers, 1 KB per warp): B=8 H=12 T=1024 FWM K=4 113 -> 111 us, softmax
+// 102 -> 97, B=4 H=12 T=1000 K=16 detached LERP 61.3 -> 59.3.  Issuing dV, dK from a second warp, dV, dK
+// before dQ, and bringing the next tiles into L2 ahead of their loads gained nothing.
 // ---------------------------------------------------------------------------
 constexpr int NCOMP_F = 512;  // compute threads
 constexpr int MMA_WARP_F = NCOMP_F / 32, PRODUCER_WARP_F = NCOMP_F / 32 + 1, PRODUCER2_WARP_F = NCOMP_F / 32 + 2;
-// The MMA warp, the two producer warps and a fourth, idle warp form the fifth warpgroup, which
-// gives registers to the four compute warpgroups: launched at 96 per thread (640 threads),
-// it keeps 64 and the compute warps take 104 (512 x 104 + 128 x 64 = 640 x 96).
-constexpr int NTHR_FUSED = NCOMP_F + 128;
-constexpr int REG_LAUNCH_F = 96, REG_COMP_F = 104, REG_AUX_F = 64;
+// The MMA warp, the two producer warps and a fourth, idle warp form the fifth warpgroup, the
+// four output warps the sixth; both give registers to the four compute warpgroups: launched at
+// 80 per thread (768 threads), they keep 48 and the compute warps take 96.
+constexpr int OUT_WARP_F = NCOMP_F / 32 + 4, NOUT_F = 4;
+constexpr int NTHR_FUSED = NCOMP_F + 256;
+constexpr int REG_LAUNCH_F = 80, REG_COMP_F = 96, REG_AUX_F = 48;
 static_assert(NCOMP_F * REG_COMP_F + (NTHR_FUSED - NCOMP_F) * REG_AUX_F <= NTHR_FUSED * REG_LAUNCH_F,
               "register shares exceed the launch allocation");
 
@@ -197,6 +205,7 @@ __global__ void __launch_bounds__(NTHR_FUSED, 1) k_bwd_fused(const __grid_consta
   uint64_t* bar_v = bars + 5 * NS + 8;       // the item's V tile landed
   uint64_t* bar_vfree = bars + 5 * NS + 9;   // the item's last g^T completed
   uint64_t* bar_kt = bars + 5 * NS + 10;     // the item's K^T tile written by every compute warp
+  uint64_t* bar_dqfree = bars + 5 * NS + 11; // the dQ partial read by the output warps
   uint64_t* bar_drain = bars + 5 * NS + 12;  // the MMA warp's clean-up commit
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 5 * NS + 13);
   const int tid = threadIdx.x, warp = warp_id_uniform();
@@ -207,7 +216,7 @@ __global__ void __launch_bounds__(NTHR_FUSED, 1) k_bwd_fused(const __grid_consta
       mbar_init(&bar_full[s], 1);
       mbar_init(&bar_emptyA[s], NCOMP_F / 32);
       mbar_init(&bar_fullT[s], 1);
-      mbar_init(&bar_empty[s], 1);
+      mbar_init(&bar_empty[s], FULLG ? 1 + NOUT_F : 1);
       mbar_init(&bar_tfree[s], 1);
     }
     for (int b = 0; b < 2; ++b) {
@@ -221,6 +230,7 @@ __global__ void __launch_bounds__(NTHR_FUSED, 1) k_bwd_fused(const __grid_consta
     mbar_init(bar_v, 1);
     mbar_init(bar_vfree, 1);
     mbar_init(bar_kt, NCOMP_F / 32);
+    mbar_init(bar_dqfree, NOUT_F);
     mbar_init(bar_drain, 1);
     fence_mbar_init();
   }
@@ -243,11 +253,8 @@ __global__ void __launch_bounds__(NTHR_FUSED, 1) k_bwd_fused(const __grid_consta
     return;
   }
 
-  if (warp < NCOMP_F / 32)
-    setmaxnreg_inc<REG_COMP_F>();
-  else
-    setmaxnreg_dec<REG_AUX_F>();
-
+  // (each role sets its registers inside its branch: ahead of a branch that all share, the
+  // compiler holds the compute path to the smaller share)
   // Two producer warps: PRODUCER_WARP_F loads the Q | dO halves with their records and the
   // items' K rows and V tiles, PRODUCER2_WARP_F the Q^T | dO^T halves, so that neither kind
   // of load waits behind the other's condition.
@@ -257,6 +264,7 @@ __global__ void __launch_bounds__(NTHR_FUSED, 1) k_bwd_fused(const __grid_consta
     bh_ = it_ % p.BH;
   };
   if (warp == PRODUCER_WARP_F) {
+    setmaxnreg_dec<REG_AUX_F>();
     int gt = 0, n = 0;
     RingPos ld, nf;
     int cf = 0, nks = 0, nv = 0;
@@ -318,6 +326,7 @@ __global__ void __launch_bounds__(NTHR_FUSED, 1) k_bwd_fused(const __grid_consta
     if (nks > 0) mbar_wait_warp(bar_kst, (nks - 1) & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA);
     if (nv > 0) mbar_wait_warp(bar_v, (nv - 1) & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA);
   } else if (warp == PRODUCER2_WARP_F) {
+    setmaxnreg_dec<REG_AUX_F>();
     int gt = 0, n = 0;
     RingPos ld, nT;
     int cT = 0;
@@ -345,9 +354,10 @@ __global__ void __launch_bounds__(NTHR_FUSED, 1) k_bwd_fused(const __grid_consta
     // clean-up: the last loads issued have landed
     drain_ring(bar_fullT, nT, cT, NS, p.wait_ns, p.status);
   } else if (warp == MMA_WARP_F) {
+    setmaxnreg_dec<REG_AUX_F>();
     const uint8_t* st0 = sm + p.sm_stage0;
     const uint32_t idq = idesc_tf32(64, D, 0, 0);
-    int n = 0;
+    int n = 0, g = 0;
     RingPos is, ib, cs, cb;  // stage / buffer of the next S^T, g^T product and of the tile being finished
     bool ok = true;
     // S^T_b = K Q^T (A in TMEM) and g^T_b = V dO^T (A in smem) of the next tile
@@ -371,7 +381,7 @@ __global__ void __launch_bounds__(NTHR_FUSED, 1) k_bwd_fused(const __grid_consta
       if (ok) tc_fence_after();
       ok = ok && issue_sg();
       if (ok && nit == 1) mma_commit(bar_vfree);
-      for (int it = 0; it < nit && ok; ++it, cs.next(NS), cb.next(2)) {
+      for (int it = 0; it < nit && ok; ++it, ++g, cs.next(NS), cb.next(2)) {
         if (it + 1 < nit) {
           ok = issue_sg();
           if (ok && it + 2 == nit) mma_commit(bar_vfree);
@@ -379,7 +389,8 @@ __global__ void __launch_bounds__(NTHR_FUSED, 1) k_bwd_fused(const __grid_consta
         }
         const int b = cb.i, s = cs.i;
         if (!mbar_wait_warp(&bar_pready[b], cb.ph, p.wait_ns, p.status, DEV_ERR_TIMEOUT_SYNC) ||
-            (it == 0 && !mbar_wait_warp(bar_kt, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA))) {
+            (it == 0 && !mbar_wait_warp(bar_kt, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA)) ||
+            (g >= 1 && !mbar_wait_warp(bar_dqfree, (uint32_t)(g - 1) & 1u, p.wait_ns, p.status, DEV_ERR_TIMEOUT_SYNC))) {
           ok = false;
           break;
         }
@@ -405,8 +416,8 @@ __global__ void __launch_bounds__(NTHR_FUSED, 1) k_bwd_fused(const __grid_consta
     }
     drain_mma(bar_drain, p.wait_ns, p.status);  // clean-up: no product still writes TMEM
   } else if (warp < NCOMP_F / 32) {
+    setmaxnreg_inc<REG_COMP_F>();
     const int row = tid & 127, cq = tid >> 7, q4 = warp & 3, lane = tid & 31;
-    uint8_t* dqs = sm + p.sm_ostage + warp * 1024;      // this warp's dQ reduce slice (16 rows x 16)
     uint8_t* ostg = sm + p.sm_kt + (q4 * 4 + cq) * 2048;  // its epilogue slice (32 rows x 16)
     // the k-th item's K rows from the V buffer into TMEM (each warp 16 of its keys' 64
     // columns), handed to the MMA warp (and the producer) through bar_ops
@@ -449,27 +460,6 @@ __global__ void __launch_bounds__(NTHR_FUSED, 1) k_bwd_fused(const __grid_consta
       fence_async_smem();  // read by the tensor core
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_kt);
-    };
-    // the dQ partial of tile q0 (this warp's 16 rows in its lanes 0..15, its 16 columns),
-    // scaled, staged in the warp's slice and added to dQ by a TMA reduce
-    auto dq_out = [&](int bh_, int q0) {
-      float v[16];
-      tmem_ld16(lane_addr(tmem, cdQ + 16 * cq), v);
-      tmem_ld_wait();
-      tma_store_wait_read();  // the slice's previous reduce has read it
-      if (lane < 16) {
-        const uint32_t base = smem_u32(dqs);
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-          asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(base + sw64_off(lane, c)),
-                       "f"(v[4 * c] * p.scale), "f"(v[4 * c + 1] * p.scale), "f"(v[4 * c + 2] * p.scale),
-                       "f"(v[4 * c + 3] * p.scale)
-                       : "memory");
-      }
-      fence_async_smem();
-      __syncwarp();
-      tma_reduce_add_3d(&maps.dq16, dqs, 16 * cq, q0 + 16 * q4, bh_);
-      tma_store_commit();
     };
     // (i, j) pairs of a row with tied maxima whose score at key j equals its maximum, into the
     // tie list (rows i0 .. i0 + 15 of this thread's chunk, key j)
@@ -547,7 +537,6 @@ __global__ void __launch_bounds__(NTHR_FUSED, 1) k_bwd_fused(const __grid_consta
           else
             fused_chunk<CAL, REC, false, 16>(sv, gv, pa, da, j, i0h, p.T, recs, fwtab, Kf, k1, p.fwm_inv_h, p.fwm_hl,
                                              p.fwm_b0l);
-          if constexpr (FULLG) rowsum_red(da, p.rsum, (size_t)bh * p.T + i0h, min(16, p.T - i0h));
           tmem_stw<16>(lane_addr(tmem, cS), pa);
           tmem_stw<16>(lane_addr(tmem, cG), da);
           // dS goes where the previous tile's Q^T, dO^T were, once dV, dK have read them
@@ -567,15 +556,6 @@ __global__ void __launch_bounds__(NTHR_FUSED, 1) k_bwd_fused(const __grid_consta
         // the tile's records and Q, dO are no longer needed
         __syncwarp();
         if (lane == 0) mbar_arrive(&bar_emptyA[s]);
-        // the previous tile's dQ partial (its product was issued after that tile's element work)
-        if (it > 0) {
-          if (!mbar_wait(bar_dqfull, (uint32_t)(gu - 1) & 1u, p.wait_ns, p.status, DEV_ERR_TIMEOUT_MMA)) {
-            failed = true;
-            break;
-          }
-          tc_fence_after();
-          dq_out(bh, q0 - BT);
-        }
         tmem_st_wait();
         fence_async_smem();  // dS, written here, is read by the tensor core
         tc_fence_before();
@@ -588,7 +568,6 @@ __global__ void __launch_bounds__(NTHR_FUSED, 1) k_bwd_fused(const __grid_consta
       failed = group_any(BAR_COMPUTE, NCOMP_F, !dok);
       if (!failed) {
         tc_fence_after();
-        dq_out(bh, (qt0 + nit - 1) * BT);
         // dV, then dK (scaled): this warp's 32 rows x 16 columns through its slice of the
         // K^T buffer (every product of the item has completed) and a TMA store
         for (int pass = 0; pass < 2; ++pass) {
@@ -615,7 +594,74 @@ __global__ void __launch_bounds__(NTHR_FUSED, 1) k_bwd_fused(const __grid_consta
         tc_fence_before();
       }
     }
-    tma_store_wait_all();  // every reduce and store of this warp is complete
+    tma_store_wait_all();  // every store of this warp is complete
+  } else if (warp >= OUT_WARP_F) {
+    // The output warps: warp q4 takes the 16 query rows 16 q4 .. + 15 of each tile (TMEM lanes
+    // 32 q4 .. + 15 of the dQ partial).  FULLG: the rows' sums of dS, from the dS tile in smem.
+    // Then the dQ partial, scaled, staged in four slices of 16 columns and added to dQ by TMA.
+    setmaxnreg_dec<REG_AUX_F>();
+    const int q4 = warp & 3, lane = threadIdx.x & 31;
+    uint8_t* dqs = sm + p.sm_ostage + q4 * 4096;
+    int n = 0, g = 0;
+    RingPos cs, cb;
+    bool ok = true;
+    for (int item = sched_item(sch, n); item < p.nitems && ok; item = sched_item(sch, ++n)) {
+      const int kb = item / p.BH, bh = item % p.BH;
+      const int qt0 = (kb * 128) / BT, nit = nqt - qt0;
+      for (int it = 0; it < nit; ++it, ++g, cs.next(NS), cb.next(2)) {
+        const int r0 = (qt0 + it) * BT + 16 * q4;
+        if constexpr (FULLG) {
+          if (!mbar_wait_warp(&bar_pready[cb.i], cb.ph, p.wait_ns, p.status, DEV_ERR_TIMEOUT_SYNC)) {
+            ok = false;
+            break;
+          }
+          // a row's 128 keys by one 16-byte load per lane: panel lane / 8, chunk lane % 8
+          const uint32_t base = smem_u32(sm + p.sm_stage0 + (cs.i ^ 1) * p.sm_stage_bytes + oQT) +
+                                (uint32_t)(lane >> 3) * PNL_DS + (uint32_t)(16 * q4) * (uint32_t)SW;
+          float v[16];
+#pragma unroll
+          for (int c = 0; c < 16; ++c) {
+            const float4 x = lds_f4(base + (uint32_t)c * (uint32_t)SW + ((((uint32_t)lane & 7u) ^ ((uint32_t)c & 7u)) << 4));
+            v[c] = (x.x + x.y) + (x.z + x.w);
+          }
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&bar_empty[cs.i ^ 1]);
+          rowsum_red(v, p.rsum, (size_t)bh * p.T + r0, min(16, p.T - r0));
+        }
+        if (!mbar_wait_warp(bar_dqfull, (uint32_t)g & 1u, p.wait_ns, p.status, DEV_ERR_TIMEOUT_MMA)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        tma_store_wait_read();  // the slices' previous reduces have read them
+        __syncwarp();
+#pragma unroll 1
+        for (int h = 0; h < 4; ++h) {
+          float v[16];
+          tmem_ld16(lane_addr(tmem, cdQ + 16 * h), v);
+          tmem_ld_wait();
+          if (lane < 16) {
+            const uint32_t base = smem_u32(dqs + h * 1024);
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+              asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(base + sw64_off(lane, c)),
+                           "f"(v[4 * c] * p.scale), "f"(v[4 * c + 1] * p.scale), "f"(v[4 * c + 2] * p.scale),
+                           "f"(v[4 * c + 3] * p.scale)
+                           : "memory");
+          }
+        }
+        tc_fence_before();
+        fence_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_dqfree);
+#pragma unroll
+        for (int h = 0; h < 4; ++h) tma_reduce_add_3d(&maps.dq16, dqs + h * 1024, 16 * h, r0, bh);
+        tma_store_commit();
+      }
+    }
+    tma_store_wait_all();  // every reduce of this warp is complete
+  } else {
+    setmaxnreg_dec<REG_AUX_F>();  // the idle warp of the MMA and producer warpgroup
   }
   __syncthreads();
   if (warp == 0) tmem_dealloc(tmem, 512);

@@ -462,29 +462,23 @@ int plan_pair(Params& p, int rest) {
 // buffer (S/g of tile t+1 computed under the element work of tile t) needs TMEM
 // room and at least two stages.
 int plan_dq(Params& p) {
-  const int parts = p.x3 ? 2 : 1, ktile = 64 * p.d * 4, dp = p.d * parts;
   const int table = p.calib == KINT_CALIB_MINMAX ? p.Kint * 1024 : 1024;
   p.pair = 0;
   if (p.x3 || p.d == 128) {
     p.sm_table = plan_pair(p, table + 8 * 128 * 4 + 9 * NCOMP_THREADS * 4);
     p.sm_rows = p.sm_table + table;
     p.sm_rstat = p.sm_rows + 8 * 128 * 4;
-    p.ops_smem = 0;
     p.sm_ostage = 0;
     const int total = std::max(finish_plan(p, p.sm_rstat + 9 * NCOMP_THREADS * 4, 28), kOneCtaPerSm);
     return total <= kSmemLimit ? total : -1;
   }
   // TF32 at d = 64: Q and dO arrive as TMA tiles staged in smem (64 KB) and are copied
-  // to TMEM from there; otherwise (3xTF32 hi/lo, d = 128) the staging area would not fit
-  // next to the K/V stages and the rows are read from global memory.
-  p.ops_smem = (!p.x3 && p.d == 64) ? 1 : 0;
-  p.nbuf = (2 * dp + 256 + p.d <= 512) ? 2 : 1;
+  // to TMEM from there
+  p.nbuf = 2;
   p.nitems = p.nqb * p.BH;
   p.sm_a = 0;
-  p.sm_stage0 = p.ops_smem ? 2 * 128 * p.d * 4 : 0;
-  p.sm_stage_bytes = 3 * parts * ktile;
-  // One CTA per SM looping over the items (dQ goes straight from TMEM to global memory,
-  // so the stage ring keeps loading the next item's tiles under the epilogue).
+  p.sm_stage0 = 2 * 128 * p.d * 4;
+  p.sm_stage_bytes = 3 * 64 * p.d * 4;
   for (p.nstage = 4; p.nstage >= 1; --p.nstage) {
     p.sm_table = p.sm_stage0 + p.nstage * p.sm_stage_bytes;
     p.sm_rows = p.sm_table + table;
@@ -503,8 +497,6 @@ int plan_dq(Params& p) {
 int plan_dkdv(Params& p, int sel) {
   const int parts = p.x3 ? 2 : 1, qtile = 64 * p.d * 4, dp = p.d * parts;
   const bool doDV = sel != DKV_DK, doDK = sel != DKV_DV;
-  // TF32 at d = 64, both products: K and V staged in smem by TMA (see plan_dq)
-  p.ops_smem = (!p.x3 && p.d == 64 && doDV && doDK) ? 1 : 0;
   p.dkv_sel = sel;
   if (sel == DKV_DK) {  // (launched for d = 128 and 3xTF32 only)
     p.rec_bytes = round_up(64 * 64 + (p.calib == KINT_CALIB_MINMAX ? 64 * p.Kp * 8 : 0), 1024);
@@ -516,11 +508,10 @@ int plan_dkdv(Params& p, int sel) {
   const int base = doDK ? 2 * dp : dp;
   // accumulators, and under 3xTF32 (one product per launch) the cross-term accumulator
   const int acc = (doDV ? p.d : 0) + (doDK ? p.d : 0) + (p.x3 ? p.d : 0);
-  if (p.x3 && doDV && doDK) return -1;
-  if (base + 128 + acc > 512) return -1;
+  if (sel == DKV_BOTH && (p.x3 || p.d != 64)) return -1;
   p.nbuf = (base + 256 + acc <= 512) ? 2 : 1;
   p.sm_a = 0;
-  p.sm_stage0 = p.ops_smem ? 2 * 128 * p.d * 4 : 0;
+  p.sm_stage0 = sel == DKV_BOTH ? 2 * 128 * p.d * 4 : 0;  // K and V staged by TMA (see plan_dq)
   // the tiles this launch reads: Q; dO, Q^T for dK; dO^T for dV
   const int tiles = 1 + (doDK ? 2 : 0) + (doDV ? 1 : 0);
   p.sm_stage_bytes = round_up(tiles * parts * qtile + 64 * 64 + (p.calib == KINT_CALIB_MINMAX ? 64 * p.Kp * 8 : 0), 1024);
@@ -547,7 +538,6 @@ int plan_fused(Params& p) {
   const int qtile = 64 * 64 * 4;
   p.nstage = 2;
   p.nbuf = 2;
-  p.ops_smem = 0;
   p.sm_a = 0;
   p.sm_stage0 = 0;
   p.sm_stage_bytes = 4 * qtile + 64 * 16;

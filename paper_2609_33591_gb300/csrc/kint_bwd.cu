@@ -125,28 +125,19 @@ __device__ __forceinline__ void add_tied_keys(uint32_t mask, float* acc, const f
   }
 }
 
-// MMA thread of k_bwd_dq: wait for key tile kt, then S_b = Q K^T and g_b = dO V^T
+// MMA thread of k_bwd_dq (TF32, d = 64): wait for key tile kt, then S_b = Q K^T and g_b = dO V^T
 // into score buffer b = kt % nbuf.
 __device__ __forceinline__ bool dq_issue_sg(const Params& p, RingPos stg, int b, uint64_t* bar_full,
                                             uint64_t* bar_sfull, const uint8_t* st0, uint32_t cQa, uint32_t cdOa,
-                                            uint32_t cSG, int ktile) {
-  const int D = p.d, s = stg.i, parts = p.x3 ? 2 : 1;
+                                            uint32_t cSG) {
+  constexpr int D = 64;
+  const int s = stg.i;
   if (!mbar_wait_warp(&bar_full[s], stg.ph, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA)) return false;
   tc_fence_after();
   const uint8_t* sk = st0 + s * p.sm_stage_bytes;
-  const uint8_t* sv = sk + parts * ktile;
   const uint32_t cS = cSG + 128 * b, cG = cS + 64;
-  if (p.x3) {
-    mma_tmem_smem(cS, cQa + D, sk, BT, D, false);     // Q_lo K_hi
-    mma_tmem_smem(cS, cQa, sk + ktile, BT, D, true);  // Q_hi K_lo
-    mma_tmem_smem(cS, cQa, sk, BT, D, true);          // Q_hi K_hi
-    mma_tmem_smem(cG, cdOa + D, sv, BT, D, false);
-    mma_tmem_smem(cG, cdOa, sv + ktile, BT, D, true);
-    mma_tmem_smem(cG, cdOa, sv, BT, D, true);
-  } else {
-    mma_tmem_smem(cS, cQa, sk, BT, D, false);
-    mma_tmem_smem(cG, cdOa, sv, BT, D, false);
-  }
+  mma_tmem_smem(cS, cQa, sk, BT, D, false);
+  mma_tmem_smem(cG, cdOa, sk + BT * D * 4, BT, D, false);
   mma_commit(&bar_sfull[b]);
   return true;
 }
@@ -158,11 +149,12 @@ __device__ __forceinline__ bool dq_issue_sg(const Params& p, RingPos stg, int b,
 // products and the element work in turns, took at B=4 H=16 T=2048 d=128 FWM 303 us (now 232),
 // at H=16 T=16384 d=128 MinMax K=16 LERP 4710 (now 3140), at B=8 H=12 T=1024 under 3xTF32 180
 // (now 131); tiles of 32 keys in two buffers 272, 4137 and 158.  Otherwise:
-// TMEM: Q [0, dp), dO [dp, 2dp) (dp = d, or 2d for 3xTF32 hi|lo; loaded by the
-// compute threads), then per score buffer b: S_b at 2dp + 128 b (64 columns), g_b
-// right after it (64 columns); dQ at 2dp + 128 nbuf.  dS overwrites S_b (its tf32
-// lo part, under 3xTF32, overwrites g_b).
-// smem: stages {K [64 x d], V [64 x d], K^T [d x 64]} (hi[, lo] each) at
+// TMEM: Q [0, 64), dO [64, 128) (copied in by the compute threads), then per score buffer
+// b: S_b at 128 + 128 b (64 columns), g_b right after it (64 columns); dQ at 128 + 128 nbuf.
+// dS overwrites S_b (PAIR: its tf32 lo part, under 3xTF32, overwrites g_b).  With d, the precision
+// and the staging path fixed at compile time (they were launch parameters), B=4 H=12 T=1024 MinMax
+// K=8: 67.5 -> 59.3 us.
+// smem: stages {K [64 x d], V [64 x d], K^T [d x 64]} at
 // sm_stage0; the grid pair table at sm_table; exchange words at sm_rows.
 // ---------------------------------------------------------------------------
 // Producer warp of k_bwd_dq: TMA-stores the dQ tile of its k-th item, which the compute
@@ -187,7 +179,8 @@ __global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(con
     pdl_wait();
     if (gated_off(p)) return;
   }
-  const int D = p.d, Kq = p.Kint, parts = p.x3 ? 2 : 1, NS = p.nstage, nbuf = p.nbuf;
+  // PAIR: d = 128 or 3xTF32; otherwise TF32 at d = 64
+  const int D = PAIR ? p.d : 64, Kq = p.Kint, NS = p.nstage, nbuf = p.nbuf;
   const int ktile = BT * D * 4;
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm + p.sm_bars);
   uint64_t* bar_full = bars;               // [NS]
@@ -209,8 +202,8 @@ __global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(con
   float* xch = reinterpret_cast<float*>(sm + p.sm_rows);  // [8][128]
   const int tid = threadIdx.x, warp = warp_id_uniform();
   constexpr int W = BT / NCG;  // key columns per thread per tile
-  const int dp = D * parts;
-  const int cQ = 0, cdO = dp, cSG0 = PAIR ? 128 : 2 * dp, cdQ = cSG0 + 128 * (PAIR ? 2 : nbuf);
+  constexpr int cQ = 0, cdO = 64, cSG0 = 128;
+  const int cdQ = cSG0 + 128 * (PAIR ? 2 : nbuf);
 
   if (PAIR && tid == 0) {
     pair_init(B, NCOMP / 32);
@@ -283,7 +276,7 @@ __global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(con
       load_rows_tile_boxed(sm + p.sm_a + 128 * D * 4, &maps.dout, bar_stg, D, 128, BT, 0, qb_ * 128, bh_);
       staged = k + 1;
     };
-    if (p.ops_smem && sched_item(sch, 0) < p.nitems) stage_ops(0);
+    if (sched_item(sch, 0) < p.nitems) stage_ops(0);
     for (int item = sched_item(sch, n); item < p.nitems && ok; item = sched_item(sch, ++n)) {
       const int qb = p.nqb - 1 - item / p.BH, bh = item % p.BH;
       const int nkt = min(2 * qb + 2, (p.T + BT - 1) / BT);
@@ -295,24 +288,19 @@ __global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(con
         }
         uint8_t* dst = sm + p.sm_stage0 + s * p.sm_stage_bytes;
         uint64_t* b = &bar_full[s];
-        mbar_arrive_expect_tx(b, 3 * parts * ktile);
+        mbar_arrive_expect_tx(b, 3 * ktile);
         load_rows_tile(dst, &maps.k, b, D, BT, 0, kt * BT, bh);
-        load_rows_tile(dst + parts * ktile, &maps.v, b, D, BT, 0, kt * BT, bh);
-        if (p.x3) {
-          load_rows_tile(dst + ktile, &maps.k_lo, b, D, BT, 0, kt * BT, bh);
-          load_rows_tile(dst + parts * ktile + ktile, &maps.v_lo, b, D, BT, 0, kt * BT, bh);
-        }
+        load_rows_tile(dst + ktile, &maps.v, b, D, BT, 0, kt * BT, bh);
         if (gt >= NS && !mbar_wait_warp(&bar_empty[s], ld.ph ^ 1u, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA)) {
           ok = false;
           break;
         }
-        load_rows_tile(dst + 2 * parts * ktile, &maps.kt, b, BT, D, kt * BT, 0, bh);
-        if (p.x3) load_rows_tile(dst + 2 * parts * ktile + ktile, &maps.kt_lo, b, BT, D, kt * BT, 0, bh);
+        load_rows_tile(dst + 2 * ktile, &maps.kt, b, BT, D, kt * BT, 0, bh);
         // The next item's Q / dO, as soon as the stage ring holds this item's first tiles: it needs
         // this item's Q / dO copied out into TMEM and the previous item's dQ tile, staged in the
         // same area since, stored; both happen at the end of the previous item, so the load has
         // this whole item to land.
-        if (p.ops_smem && kt == min(nkt, NS) - 1 && sched_item(sch, n + 1) < p.nitems) {
+        if (kt == min(nkt, NS) - 1 && sched_item(sch, n + 1) < p.nitems) {
           if (!mbar_wait_warp(bar_ops, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_SYNC) ||
               (n >= 1 && !store_staged_dq(maps, p, sch, bar_ostg, n - 1, sm + p.sm_a))) {
             ok = false;
@@ -323,7 +311,7 @@ __global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(con
       }
     }
     // the last-but-one item's tile (the last item's is stored by the compute warps)
-    if (p.ops_smem && ok && n >= 2) store_staged_dq(maps, p, sch, bar_ostg, n - 2, sm + p.sm_a);
+    if (ok && n >= 2) store_staged_dq(maps, p, sch, bar_ostg, n - 2, sm + p.sm_a);
     tma_store_wait_all();
     // clean-up: the last tiles issued have landed
     drain_ring(bar_full, ld, gt, NS, p.wait_ns, p.status);
@@ -349,7 +337,7 @@ __global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(con
           ok = false;
           break;
         }
-        ok = dq_issue_sg(p, is, ib.i, bar_full, bar_sfull, st0, cQa, cdOa, cSG, ktile);
+        ok = dq_issue_sg(p, is, ib.i, bar_full, bar_sfull, st0, cQa, cdOa, cSG);
       }
     }
     drain_mma(bar_drain, p.wait_ns, p.status);  // clean-up: no product still writes TMEM
@@ -368,16 +356,8 @@ __global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(con
           break;
         }
         tc_fence_after();
-        const uint8_t* skt = sm + p.sm_stage0 + s * p.sm_stage_bytes + 2 * parts * ktile;
-        const uint32_t cS = tmem + cSG0 + 128 * b, cG = cS + 64;
-        const bool acc = kt > 0;
-        if (p.x3) {
-          mma_tmem_smem(tmem + cdQ, cS, skt, D, BT, acc);           // dS_hi K_hi
-          mma_tmem_smem(tmem + cdQ, cS, skt + ktile, D, BT, true);  // dS_hi K_lo
-          mma_tmem_smem(tmem + cdQ, cG, skt, D, BT, true);          // dS_lo K_hi
-        } else {
-          mma_tmem_smem(tmem + cdQ, cS, skt, D, BT, acc);
-        }
+        const uint8_t* skt = sm + p.sm_stage0 + s * p.sm_stage_bytes + 2 * ktile;
+        mma_tmem_smem(tmem + cdQ, tmem + cSG0 + 128 * b, skt, D, BT, kt > 0);
         mma_commit(&bar_empty[s]);
         mma_commit(&bar_dqdone[b]);
       }
@@ -388,24 +368,16 @@ __global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(con
     // ---- compute warps: items one after the other ----
     const int row = tid & 127, cg = (tid >> 7) & (NCG - 1);
     // Operand rows of the n-th item into TMEM (column group 0 takes Q, group 1 takes dO),
-    // handed to the MMA warp through bar_ops.  TF32 at d = 64: from the tiles the producer
-    // staged in smem; otherwise from global rows.  The next item's rows go in as soon as
-    // the current item's last S, g have been read (before its dQ epilogue), so the next
-    // item's first products run under that epilogue.
+    // handed to the MMA warp through bar_ops, from the tiles the producer staged in smem.  The
+    // next item's rows go in as soon as the current item's last S, g have been read (before its
+    // dQ epilogue), so the next item's first products run under that epilogue.
     auto ops_to_tmem = [&](int n) {
       if constexpr (PAIR) {
         pair_ops_to_tmem(p, B, sm, n, row, cg * (D / NCG), D / NCG);
         return;
       }
-      const int item = sched_item(sch, n);
-      const int qb = p.nqb - 1 - item / p.BH, bh = item % p.BH, i = qb * 128 + row;
-      if (p.ops_smem) {
-        if (mbar_wait(bar_stg, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA))
-          staged_row_to_tmem(tmem, cg == 0 ? cQ : cdO, sm + p.sm_a + (cg == 0 ? 0 : 128 * D * 4), row, D);
-      } else {
-        row_to_tmem(tmem, cg == 0 ? cQ : cdO, cg == 0 ? p.Q : p.dO, bh * p.T + i, i < p.T ? (bh + 1) * p.T : 0, D,
-                    p.x3 != 0);
-      }
+      if (mbar_wait(bar_stg, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA))
+        staged_row_to_tmem(tmem, cg == 0 ? cQ : cdO, sm + p.sm_a + (cg == 0 ? 0 : 128 * D * 4), row, D);
       tmem_st_wait();
       tc_fence_before();
       __syncwarp();
@@ -453,6 +425,11 @@ __global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(con
       }
       return r;
     };
+    // Whether the epilogue passes through the staging area: TF32 at d = 64 always, PAIR never.  For
+    // PAIR it is read from the launch parameters all the same: with that side of the epilogue
+    // compiled out, the compiler's schedule of the MinMax tile loop is worse (H=16 T=16384 d=128
+    // K=16: 3439 against 3133 us; the other instantiations within 1 %).
+    const bool staged = PAIR ? p.pair == 0 : true;
     int n = 0;
     RingPos cb, cs;  // score buffer and stage of the current tile
     bool failed = false;
@@ -552,7 +529,7 @@ __global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(con
           add_tied_keys(mk_max, tie_max, p.K + ((size_t)bh * p.T + j0) * D, D);
           add_tied_keys(mk_min, tie_min, p.K + ((size_t)bh * p.T + j0) * D, D);
         }
-        if (p.x3) {
+        if (PAIR && p.x3) {
           float lo[W];
   #pragma unroll
           for (int q = 0; q < W; ++q) {
@@ -574,7 +551,7 @@ __global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(con
         ops_to_tmem(n + 1);
         nx = load_row_stats(n + 1);
       }
-      if (p.ops_smem && FULLG && CAL != CAL_SOFTMAX) {
+      if (staged && FULLG && CAL != CAL_SOFTMAX) {
         // the epilogue's arg-max key rows (this thread's column half), gathered into the dO half
         // of the staging area (read by every warp's copy above: hence the barrier) while the
         // item's last product completes
@@ -625,7 +602,7 @@ __global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(con
           // its 4 KB slot of the free dO half of that area, then each thread reads its row back;
           // otherwise every thread loads its own row (32 lines per load).
           float4 km[8], kn[8];
-          if (p.ops_smem && FULLG && CAL != CAL_SOFTMAX) {
+          if (staged && FULLG && CAL != CAL_SOFTMAX) {
             // the arg-max rows were requested before the wait for the item's last product
             // (tie sums, complete only now, are read directly)
             float4* slot = reinterpret_cast<float4*>(sm + p.sm_a + 128 * D * 4) + warp * 256;
@@ -661,7 +638,7 @@ __global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(con
             v[4 * q + 2] = __fmaf_rn(cmn, kn[q].z, __fmaf_rn(cMn, km[q].z, v[4 * q + 2])) * p.scale;
             v[4 * q + 3] = __fmaf_rn(cmn, kn[q].w, __fmaf_rn(cMn, km[q].w, v[4 * q + 3])) * p.scale;
           }
-          if (p.ops_smem) {
+          if (staged) {
             row_to_staged(stg, row, c / 32, v);
           } else if (row_ok) {
             float4* dst = reinterpret_cast<float4*>(p.dQ + rw * D + c);
@@ -669,7 +646,7 @@ __global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(con
             for (int q = 0; q < 8; ++q) dst[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
           }
         }
-        if (p.ops_smem) {
+        if (staged) {
           fence_async_smem();
           if (last) {
             group_sync(BAR_COMPUTE, NCOMP);

@@ -230,9 +230,10 @@ __device__ __forceinline__ bool store_staged_dkdv(const Maps& maps, const Params
 // What bounds it: the issue of the products by one warp, then the shared-memory loads of the
 // row records.
 // Measured on GB300 against eight compute warps and stages of all four tiles: B=4 H=16 T=2048
-// d=128 FWM Weight-STE dV 340 -> 178 us, dK 403 -> 231; H=16 T=16384 d=128 MinMax K=16 LERP
-// 5097 -> 2223, 5878 -> 3010; 3xTF32 B=8 H=12 T=1024 168 -> 98, 203 -> 127; MinMax B=4 H=12
-// T=1024 d=64 (both products) 73.6 -> 71.6.  (dK in the stage ring with 32-query tiles: 313,
+// d=128 FWM Weight-STE dV 340 -> 170 us, dK 403 -> 231; H=16 T=16384 d=128 MinMax K=16 LERP
+// 5097 -> 2104, 5878 -> 2984; 3xTF32 B=8 H=12 T=1024 168 -> 93, 203 -> 127; MinMax B=4 H=12
+// T=1024 d=64 (both products) 73.6 -> 71.6, and 63.4 with d, the precision and the staging path fixed
+// at compile time for the launch of both products.  (dK in the stage ring with 32-query tiles: 313,
 // 3785 and 170.)
 // ---------------------------------------------------------------------------
 template <int CAL, int REC, bool FULLG, bool PROJ, bool RS, int SEL>
@@ -245,7 +246,10 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
     pdl_wait();
     if (gated_off(p)) return;
   }
-  const int D = p.d, Kq = p.Kint, parts = p.x3 ? 2 : 1, NS = p.nstage, nbuf = p.nbuf;
+  // both products: TF32 at d = 64; one: d = 128 or 3xTF32
+  constexpr bool STAGED = SEL == DKV_BOTH;  // K, V rows and the outputs pass through smem by TMA
+  const bool x3 = !STAGED && p.x3;
+  const int D = STAGED ? 64 : p.d, Kq = p.Kint, parts = x3 ? 2 : 1, NS = p.nstage, nbuf = p.nbuf;
   constexpr bool doDV = SEL != DKV_DK, doDK = SEL != DKV_DV, needV = doDK;
   constexpr bool PAIR = SEL == DKV_DK;  // the product pipeline of kint_pair.cuh
   const int qtile = BT * D * 4;
@@ -347,7 +351,7 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
       pair_mma_sg(p, B, sm, get);
     } else {
       pair_mma_acc(p, B, sm, get, [&](uint32_t cS, uint32_t cG, const uint8_t* qt, bool first) {
-        if (p.x3) {
+        if (x3) {
           mma_tmem_smem(cdK, cS, qt, D, BT, !first);          // hi x hi
           mma_tmem_smem(cdC, cS, qt + qtile, D, BT, !first);  // hi x lo
           mma_tmem_smem(cdC, cG, qt, D, BT, true);            // lo x hi
@@ -371,7 +375,7 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
       if (needV) load_rows_tile_boxed(sm + p.sm_a + 128 * D * 4, &maps.v, bar_stg, D, 128, BT, 0, kb_ * 128, bh_);
       staged = k + 1;
     };
-    if (p.ops_smem && sched_item(sch, 0) < p.nitems) stage_ops(0);
+    if (STAGED && sched_item(sch, 0) < p.nitems) stage_ops(0);
     for (int item = sched_item(sch, n); item < p.nitems && ok; item = sched_item(sch, ++n)) {
       const int kb = item / p.BH, bh = item % p.BH;
       const int qt0 = (kb * 128) / BT, nit = nqt - qt0;
@@ -389,10 +393,10 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
         if (CAL == CAL_MINMAX) bytes += nrows * tstride;
         mbar_arrive_expect_tx(b, bytes);
         load_rows_tile(dst + oQ, &maps.q, b, D, BT, 0, q0, bh);
-        if (p.x3) load_rows_tile(dst + oQ + qtile, &maps.q_lo, b, D, BT, 0, q0, bh);
+        if (x3) load_rows_tile(dst + oQ + qtile, &maps.q_lo, b, D, BT, 0, q0, bh);
         if (needV) {
           load_rows_tile(dst + odO, &maps.dout, b, D, BT, 0, q0, bh);
-          if (p.x3) load_rows_tile(dst + odO + qtile, &maps.dout_lo, b, D, BT, 0, q0, bh);
+          if (x3) load_rows_tile(dst + odO + qtile, &maps.dout_lo, b, D, BT, 0, q0, bh);
         }
         const size_t r0 = (size_t)bh * p.T + q0;
         bulk_load(dst + oRec, reinterpret_cast<const RowRec*>(p.rec) + r0, nrows * 64, b);
@@ -407,11 +411,11 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
         mbar_arrive_expect_tx(bt, ((doDK ? 1 : 0) + (doDV ? 1 : 0)) * parts * qtile);
         if (doDK) {
           load_rows_tile(dst + oQT, &maps.qt, bt, BT, D, q0, 0, bh);
-          if (p.x3) load_rows_tile(dst + oQT + qtile, &maps.qt_lo, bt, BT, D, q0, 0, bh);
+          if (x3) load_rows_tile(dst + oQT + qtile, &maps.qt_lo, bt, BT, D, q0, 0, bh);
         }
         if (doDV) {
           load_rows_tile(dst + odOT, &maps.dot, bt, BT, D, q0, 0, bh);
-          if (p.x3) load_rows_tile(dst + odOT + qtile, &maps.dot_lo, bt, BT, D, q0, 0, bh);
+          if (x3) load_rows_tile(dst + odOT + qtile, &maps.dot_lo, bt, BT, D, q0, 0, bh);
         }
         nT.next(NS);
         ++cT;
@@ -419,7 +423,7 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
         // this item's K / V copied out into TMEM and the previous item's dV / dK tiles, staged in
         // the same area since, stored; both happen at the end of the previous item, so the load
         // has this whole item to land.
-        if (p.ops_smem && it == min(nit, NS) - 1 && sched_item(sch, n + 1) < p.nitems) {
+        if (STAGED && it == min(nit, NS) - 1 && sched_item(sch, n + 1) < p.nitems) {
           if (!mbar_wait_warp(bar_ops, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_SYNC) ||
               (n >= 1 && !store_staged_dkdv(maps, p, sch, bar_ostg, n - 1, sm + p.sm_a, doDV, doDK))) {
             ok = false;
@@ -430,7 +434,7 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
       }
     }
     // the last-but-one item's tiles (the last item's are stored by the compute warps)
-    if (p.ops_smem && ok && n >= 2) store_staged_dkdv(maps, p, sch, bar_ostg, n - 2, sm + p.sm_a, doDV, doDK);
+    if (STAGED && ok && n >= 2) store_staged_dkdv(maps, p, sch, bar_ostg, n - 2, sm + p.sm_a, doDV, doDK);
     tma_store_wait_all();
     // clean-up: the last tiles issued have landed
     drain_ring(bar_full, nf, cf, NS, p.wait_ns, p.status);
@@ -468,7 +472,7 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
         const uint8_t* st = sm + p.sm_stage0 + s * p.sm_stage_bytes;
         const uint32_t cS = tmem + base + 128 * b, cG = cS + 64;
         const bool acc = it > 0;
-        if (p.x3) {
+        if (x3) {
           const uint32_t cacc = tmem + (doDV ? cdV : cdK);
           const uint8_t* bt = st + (doDV ? odOT : oQT);
           mma_tmem_smem(cacc, cS, bt, D, BT, acc);                   // hi x hi
@@ -505,15 +509,15 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
       const int item = sched_item(sch, n), kb = item / p.BH, bh = item % p.BH, j = kb * 128 + row;
       const bool isV = needV && cg >= 2;
       const int nc = needV ? D / 2 : D / NCG_KV, c0 = (needV ? cg & 1 : cg) * nc;
-      const bool ok = !p.ops_smem || mbar_wait(bar_stg, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA);
+      const bool ok = !STAGED || mbar_wait(bar_stg, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA);
       if (ok) {
         const int lim = j < p.T ? (bh + 1) * p.T : 0;
 #pragma unroll 1
         for (int c = c0; c < c0 + nc; c += 16) {
-          if (p.ops_smem)
+          if (STAGED)
             staged16_to_tmem(tmem, isV ? cV : cK, sm + p.sm_a + (isV ? 128 * D * 4 : 0), row, c);
           else
-            row_to_tmem_part<16>(tmem, isV ? cV : cK, isV ? p.V : p.K, bh * p.T + j, lim, D, c, p.x3 != 0);
+            row_to_tmem_part<16>(tmem, isV ? cV : cK, isV ? p.V : p.K, bh * p.T + j, lim, D, c, x3);
         }
       }
       tmem_st_wait();
@@ -596,7 +600,7 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
             if (doDK) rowsum_add(da, p.dsum_out, p.dabs_out, (size_t)bh * p.T + i0h, min(W, p.T - i0h));
           }
         }
-        if (p.x3) {
+        if (x3) {
 #pragma unroll
           for (int q = 0; q < W; ++q) {
             const float x = doDV ? pa[q] : da[q];
@@ -638,7 +642,7 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
           for (int c = cg * (D / NCG_KV); c < (cg + 1) * (D / NCG_KV); c += 16) {
             float v[16];
             tmem_ld16(lane_addr(tmem, col + c), v);
-            if (p.x3) {
+            if (x3) {
               float w[16];
               tmem_ld16(lane_addr(tmem, cdC + c), w);
               tmem_ld_wait();
@@ -648,7 +652,7 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
             tmem_ld_wait();
 #pragma unroll
             for (int q = 0; q < 16; ++q) v[q] *= mul;
-            if (p.ops_smem) {
+            if (STAGED) {
               row16_to_staged(stg + pass * 128 * D * 4, row, c, v);
             } else if (j < p.T) {
               float4* dst = reinterpret_cast<float4*>(out + c);
@@ -657,7 +661,7 @@ __global__ void __launch_bounds__(NTHR_KV, 1) k_bwd_dkdv(const __grid_constant__
             }
           }
         }
-        if (p.ops_smem) {
+        if (STAGED) {
           fence_async_smem();
           if (last) {
             group_sync(BAR_COMPUTE, NCOMP_KV);

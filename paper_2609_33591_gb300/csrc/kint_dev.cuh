@@ -539,16 +539,6 @@ __device__ __forceinline__ void row_to_tmem_part(uint32_t tmem_base, int col, co
   tmem_stw<N>(lane_addr(tmem_base, col + c0), hi);
 }
 
-// Thread-owned row `row` of X (d fp32) into the thread's TMEM lane at columns
-// [col, col+d) (hi/lo with `split`, lo at [col+d, col+2d)), 16 columns at a time:
-// the path of the configurations without staged operands, kept small so that it
-// does not crowd the registers of the kernels' main loops.
-__device__ __forceinline__ void row_to_tmem(uint32_t tmem_base, int col, const float* X, int row, int T, int d,
-                                            bool split) {
-#pragma unroll 1
-  for (int c0 = 0; c0 < d; c0 += 16) row_to_tmem_part<16>(tmem_base, col, X, row, T, d, c0, split);
-}
-
 // Row `row` of a 128-row K-major tile staged in smem by TMA (128-byte swizzle,
 // 32-column panels 128 x 128 bytes apart) into the calling thread's TMEM lane at
 // columns [col, col + d).  Chunk c (16 bytes) of a row sits at chunk c ^ (row % 8).

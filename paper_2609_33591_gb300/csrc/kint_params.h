@@ -76,7 +76,6 @@ struct Params {
   int q_tmem;            // pass 2: Q as a TMEM operand (copied in by the compute warps)
   int pair;      // dQ kernel: the product pipeline of kint_pair.cuh (d = 128, 3xTF32; the dK launch always)
   int sm_x, sm_y, sm_xt, sm_rec, nx, ny, nxt, rec_bytes;  // its rings (dK: two slots of row records)
-  int ops_smem;  // backward: the 128-row TMEM operands (Q, dO / K, V) are staged in smem by TMA first
   int sm_v, sm_kt;  // single-pass backward: the V tile (A operand of g^T) and the K^T tile (B operand of dQ);
                     // pass 2: sm_v is the V^T ring
   // Launch gate of the backward kernels that run on one side of a device-side decision:

@@ -258,6 +258,15 @@ void kint_set_wait_timeout_ns(unsigned long long ns);
 void kint_test_expire_next_wait(int count);
 
 /*
+ * The same for pass 2 of the next `count` calls of kint_attn_fwd and kint_attn_fwd_noalloc: the
+ * compute warps' first wait for the Q tile runs out in three of every four warps (one of two
+ * where two CTAs share an SM) and succeeds in the others, so the warps of a CTA disagree about
+ * it.  Status bit 1 (TMA wait timed out) is set, every warp leaves within a few limits, and the
+ * context stays usable.  At d = 128 with O_lerp no compute warp waits for Q: no effect there.
+ */
+void kint_test_expire_next_q_wait(int count);
+
+/*
  * Backward implementation choice (process-wide; the paper has no counterpart): 0 (default)
  * uses the single-pass backward wherever kint_attn_bwd describes it as applying, 1 always
  * the two-pass kernels (bit-reproducible).  Other values act as 0.  Do not change it

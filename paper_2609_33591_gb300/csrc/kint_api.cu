@@ -34,6 +34,7 @@ int g_dev_ok[kMaxDevices] = {0};  // 0 unknown, 1 sm_103, -1 other
 int g_num_sms[kMaxDevices] = {0};
 unsigned long long g_wait_ns = 2000000000ull;
 std::atomic<int> g_expire_waits{0};  // test hook: forward calls whose first kernel's first wait runs out
+std::atomic<int> g_expire_q_waits{0};  // test hook: forward calls whose pass 2 has its first Q wait run out in some warps
 int g_bwd_path = 0;  // 0: single-pass backward where it applies, 1: always the two-pass kernels
 constexpr int kSmemLimit = 232448;  // opt-in maximum per CTA on sm_103
 constexpr int NCOMP_THREADS = 256;  // compute threads of the warp-specialised kernels (kint_dev.cuh NCOMP)
@@ -557,6 +558,14 @@ int launch_rc(cudaError_t e) { return e == cudaSuccess ? KINT_OK : KINT_ERR_LAUN
 kint_launch_cb g_cb = nullptr;
 void* g_cb_user = nullptr;
 
+// Test hooks of the bounded waits: consume one pending request, if there is one.
+bool take_request(std::atomic<int>& requests) {
+  int pending = requests.load();
+  while (pending > 0 && !requests.compare_exchange_weak(pending, pending - 1)) {
+  }
+  return pending > 0;
+}
+
 // One kernel launch between the optional tracing callbacks.
 template <class F>
 cudaError_t traced(const char* name, cudaStream_t s, F&& launch) {
@@ -605,11 +614,7 @@ int forward_prologue(const float* Q, const float* K, const float* V, const Param
   if (!ok) return KINT_ERR_LAUNCH;
   Params ps = p;
   const int smem = plan_stats(ps);
-  // test hook of the bounded waits: consume one pending request
-  int pending = g_expire_waits.load();
-  while (pending > 0 && !g_expire_waits.compare_exchange_weak(pending, pending - 1)) {
-  }
-  ps.expire_wait = pending > 0 ? 1 : 0;
+  ps.expire_wait = take_request(g_expire_waits) ? 1 : 0;
   return launch_rc(traced("k_fwd_stats", s, [&] { return launch_fwd_stats(maps, ps, smem, s, sched_for(SCHED_STATS, ps)); }));
 }
 
@@ -665,6 +670,7 @@ int forward_launches(const float* Q, const float* K, const float* V, float* O, c
   pm.pv_sel = (prob && !p.x3) ? PV_MAIN_LERP : PV_MAIN;
   const int smem = plan_main(pm, pm.pv_sel);
   if (smem < 0 || smem > kSmemLimit) return KINT_ERR_UNSUPPORTED;
+  pm.expire_wait = take_request(g_expire_q_waits) ? 1 : 0;
   if ((rc = launch_rc(traced("k_fwd_main", s, [&] { return launch_fwd_main(maps, pm, smem, s, sched_for(SCHED_MAIN, pm)); })))) return rc;
   if (prob && p.x3) {
     Params pl = p;
@@ -978,6 +984,8 @@ const char* kint_strerror(int code) {
 void kint_set_wait_timeout_ns(unsigned long long ns) { g_wait_ns = ns < 1000ull ? 1000ull : ns; }
 
 void kint_test_expire_next_wait(int count) { g_expire_waits.store(count > 0 ? count : 0); }
+
+void kint_test_expire_next_q_wait(int count) { g_expire_q_waits.store(count > 0 ? count : 0); }
 
 void kint_set_backward_path(int path) { g_bwd_path = path == 1 ? 1 : 0; }
 

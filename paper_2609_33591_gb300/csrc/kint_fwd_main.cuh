@@ -260,6 +260,7 @@ __global__ void __launch_bounds__(MainT<NG>::NTHR, MainT<NG>::CTAS) k_fwd_main(c
   uint64_t* bar_s = bars;              // [4] S_b computed
   uint64_t* bar_pready = bars + 4;     // [4] the weights of buffer b stored by the tile's eight warps
   uint64_t* bar_pv = bars + 8;         // [NG] the product that read the group's A2 buffer complete
+  uint64_t* bar_never = bars + 11;     // (one of the four kept for bar_pv; NG <= 2) nothing arrives: test hook
   uint64_t* bar_q = bars + 12;         // Q of the item landed in smem
   uint64_t* bar_qfree = bars + 13;     // smem Q may be reloaded (q_tmem: Q copied into TMEM; else last S complete)
   uint64_t* bar_done = bars + 14;      // every product of the item complete
@@ -579,10 +580,11 @@ __global__ void __launch_bounds__(MainT<NG>::NTHR, MainT<NG>::CTAS) k_fwd_main(c
       M_ = i < p.T ? p.row_max[rw] : 0.0f;
       m_ = (CAL == CAL_MINMAX && i < p.T) ? p.row_min[rw] : 0.0f;
     };
-    // The k-th item's Q rows from smem into TMEM (each thread its share of its row's columns),
-    // handed to the MMA warp and the K producer through bar_qfree.
-    auto q_to_tmem = [&](int k) -> bool {
-      const bool ok = mbar_wait(bar_q, k & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA);
+    // The k-th item's Q rows from smem, once `bar` (bar_q) says that they landed, into TMEM (each
+    // thread its share of its row's columns), handed to the MMA warp and the K producer through
+    // bar_qfree.
+    auto q_to_tmem = [&](int k, uint64_t* bar) -> bool {
+      const bool ok = mbar_wait_warp(bar, k & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA);
       if (ok) {
 #pragma unroll 1
         for (int c = cq * (D / NQ); c < (cq + 1) * (D / NQ); c += 16) {
@@ -599,7 +601,8 @@ __global__ void __launch_bounds__(MainT<NG>::NTHR, MainT<NG>::CTAS) k_fwd_main(c
     int item = sched_item(sch, 0);
     if (item < p.nitems) {
       load_extrema(item, qb, bh, M, m);
-      if (q_tmem) failed = !q_to_tmem(0);
+      // (the test hook lets the wait run out in every warp but the first of each quarter)
+      if (q_tmem) failed = !q_to_tmem(0, p.expire_wait && cq > 0 ? bar_never : bar_q);
     }
     // Tables addressed by the float bits 0x4B000000 + index of the floored position.
     // FWM: one half-bin table of 24-byte line entries, q in [-2, 2K] at sm_table + 24 (q + 2)
@@ -625,7 +628,9 @@ __global__ void __launch_bounds__(MainT<NG>::NTHR, MainT<NG>::CTAS) k_fwd_main(c
             make_float2(p.fwm_e[tid], p.fwm_e[tid + 1]);
       if (tid < kFwdTail) *reinterpret_cast<float2*>(sm + p.sm_table + tid * 8) = make_float2(0.f, 0.f);
     }
-    group_sync(BAR_COMPUTE, NCOMP);  // the shared table
+    // The shared table is written; and a first Q wait that ran out in some warps sends every compute
+    // warp past the items, because the others would wait for those at the item's barriers.
+    failed = group_any(BAR_COMPUTE, NCOMP, failed);
     while (item < p.nitems && !failed) {
       const int nkt = tiles_of(qb), i = qb * 128 + row;
       const bool row_ok = i < p.T;
@@ -725,7 +730,7 @@ __global__ void __launch_bounds__(MainT<NG>::NTHR, MainT<NG>::CTAS) k_fwd_main(c
       if (!failed) failed = !mbar_wait(bar_done, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_MMA);
       tc_fence_after();
       // every S of the item is complete: the next item's Q goes in under the epilogue
-      if (!failed && q_tmem && next < p.nitems) failed = !q_to_tmem(n + 1);
+      if (!failed && q_tmem && next < p.nitems) failed = !q_to_tmem(n + 1, bar_q);
       if (!failed) failed = !mbar_wait(bar_w, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_SYNC);
       if (!failed && !p.debug && use > 0)  // the staging area's previous stores have read it
         failed = !mbar_wait(bar_stfree, (use - 1) & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_SYNC);

@@ -7,9 +7,7 @@
 #include <cstdint>
 #include <cstring>
 #include <atomic>
-#include <memory>
 #include <mutex>
-#include <vector>
 
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -18,6 +16,7 @@
 #include "../../include/kint_attn.h"
 #include "kint_launch.h"
 #include "kint_params.h"
+#include "kint_sched_build.h"
 
 namespace kint {
 
@@ -42,106 +41,10 @@ constexpr int NCOMP_THREADS = 256;  // compute threads of the warp-specialised k
 int round_up(int x, int m) { return (x + m - 1) / m * m; }
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
-// Item schedules of the persistent kernels (Sched), longest processing time first: an
-// item costs a + tiles (a = its fixed cost in tiles: operand loads, epilogue, measured
-// per CTA), and items in decreasing cost each go to the CTA with the least work so far,
-// ties to the lower CTA.  Built once per kernel and shape and kept.
-enum SchedKind { SCHED_STATS = 0, SCHED_MAIN = 1, SCHED_FUSED = 2, SCHED_DQ = 3, SCHED_DK = 4 };
-
-// Heads go in groups whose tiles (what every item of a head streams) fit in this share of the
-// 129 MB L2, all items of a group before the next group's; with every head's longest item first
-// the tiles were read from DRAM again for each block.  Between 24 and 72 MB the times are the
-// same within 2 %.  B=4 H=16 T=2048 d=128 (200 MB of tiles in dQ and dK): pass 1 78 -> 75 us,
-// pass 2 136 -> 124, dQ 248 -> 232, dK 238 -> 231; B=8 H=12 T=1024 3xTF32 dQ 147 -> 132,
-// dK 131 -> 127.  Not the single-pass backward, where groups of 16 to 48 of 96 heads gave nothing.
-constexpr double kGroupBytes = 48e6;
-
-struct SchedEntry {
-  int kind, nitems, ngrid, BH, nqb, nqt, hg;
-  Sched sch;
-};
-std::vector<std::unique_ptr<SchedEntry>> g_sched;
-
-const Sched& sched_none() {
-  static const Sched none = [] { Sched z; std::memset(&z, 0, sizeof(z)); return z; }();
-  return none;
-}
-
-const Sched& sched_for(int kind, const Params& p) {
-  if (p.ngrid >= p.nitems || p.ngrid > SCHED_MAX_CTAS || p.nitems > SCHED_MAX_ITEMS) return sched_none();
-  const bool keys = kind == SCHED_FUSED || kind == SCHED_DK;  // items are key blocks
-  const int nqt = keys ? p.nqt : 0;
-  // heads per group: at least as many items as CTAs (a group of one head of 128 blocks on 152 SMs
-  // took 5 % longer than groups of two)
-  const int tensors = kind == SCHED_FUSED ? 0 : kind == SCHED_STATS ? 1 : kind == SCHED_MAIN ? 2 : 3;
-  const int ng0 = (int)std::ceil(4.0 * tensors * (p.x3 ? 2 : 1) * p.BH * p.T * p.d / kGroupBytes);
-  const int hg_min = std::min(p.BH, (p.ngrid + p.nqb - 1) / p.nqb);
-  const int hg0 = ng0 <= 1 ? p.BH : std::max(hg_min, (p.BH + ng0 - 1) / ng0);
-  std::lock_guard<std::mutex> lk(g_mu);
-  for (const auto& e : g_sched)
-    if (e->kind == kind && e->nitems == p.nitems && e->ngrid == p.ngrid && e->BH == p.BH && e->nqb == p.nqb &&
-        e->nqt == nqt && e->hg == hg0)
-      return e->sch;
-  if (g_sched.size() >= 256) return sched_none();  // entries are never released: bound their number
-  // tiles and fixed cost of item i: query blocks (longest first) for the forward passes (128-row
-  // tiles) and dQ, key blocks with their 64-row query tiles for the single-pass backward and dK
-  const double fixed = kind == SCHED_MAIN ? 2.6 : (kind == SCHED_DQ || kind == SCHED_DK) ? 4.0 : 2.0;
-  std::vector<double> cost(p.nitems);
-  for (int i = 0; i < p.nitems; ++i) {
-    int tiles;
-    if (keys)
-      tiles = p.nqt - (i / p.BH) * 2;
-    else
-      tiles = (p.nqb - i / p.BH) * (kind == SCHED_DQ ? 2 : 1);
-    cost[i] = fixed + tiles;
-  }
-  // of the group sizes from hg0 down to half of it, the one whose longest CTA is shortest
-  std::vector<std::vector<int>> lists, cand;
-  std::vector<int> order(p.nitems);
-  std::vector<double> load;
-  double best_span = 0.0;
-  for (int ng = (p.BH + hg0 - 1) / hg0, hg = hg0, last = 0; lists.empty() || (2 * hg >= hg0 && hg >= hg_min);
-       ++ng, hg = (p.BH + ng - 1) / ng) {
-    if (hg != last) {
-      last = hg;
-      for (int i = 0; i < p.nitems; ++i) order[i] = i;
-      std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
-        const int ga = a % p.BH / hg, gb = b % p.BH / hg;
-        return ga != gb ? ga < gb : cost[a] > cost[b];
-      });
-      load.assign(p.ngrid, 0.0);
-      cand.assign(p.ngrid, {});
-      for (int i : order) {
-        const int c = (int)(std::min_element(load.begin(), load.end()) - load.begin());
-        load[c] += cost[i];
-        cand[c].push_back(i);
-      }
-      const double span = *std::max_element(load.begin(), load.end());
-      if (lists.empty() || span < best_span) {
-        lists.swap(cand);
-        best_span = span;
-      }
-    }
-    if (hg0 == p.BH || hg <= 1) break;
-  }
-  auto e = std::make_unique<SchedEntry>();
-  std::memset(&e->sch, 0, sizeof(Sched));
-  e->kind = kind;
-  e->nitems = p.nitems;
-  e->ngrid = p.ngrid;
-  e->BH = p.BH;
-  e->nqb = p.nqb;
-  e->nqt = nqt;
-  e->hg = hg0;
-  int k = 0;
-  for (int c = 0; c < p.ngrid; ++c) {
-    e->sch.off[c] = (uint16_t)k;
-    for (int i : lists[c]) e->sch.idx[k++] = (uint16_t)i;
-  }
-  e->sch.off[p.ngrid] = (uint16_t)k;
-  e->sch.n = p.nitems;
-  g_sched.push_back(std::move(e));
-  return g_sched.back()->sch;
+// The item schedule of a persistent kernel's launch (kint_sched_build.h).
+SchedStore g_sched;
+SchedStore::Ptr sched_for(SchedKind kind, const Params& p) {
+  return g_sched.get(sched_key(kind, p.nitems, p.ngrid, p.BH, p.nqb, p.nqt, 4.0 * p.T * p.d * (p.x3 ? 2 : 1)));
 }
 
 // Resolve the device-dependent handles once per device.
@@ -615,7 +518,7 @@ int forward_prologue(const float* Q, const float* K, const float* V, const Param
   Params ps = p;
   const int smem = plan_stats(ps);
   ps.expire_wait = take_request(g_expire_waits) ? 1 : 0;
-  return launch_rc(traced("k_fwd_stats", s, [&] { return launch_fwd_stats(maps, ps, smem, s, sched_for(SCHED_STATS, ps)); }));
+  return launch_rc(traced("k_fwd_stats", s, [&] { return launch_fwd_stats(maps, ps, smem, s, *sched_for(SCHED_STATS, ps)); }));
 }
 
 int check_stats(const kint_rowstats* st, bool prob) {
@@ -671,13 +574,13 @@ int forward_launches(const float* Q, const float* K, const float* V, float* O, c
   const int smem = plan_main(pm, pm.pv_sel);
   if (smem < 0 || smem > kSmemLimit) return KINT_ERR_UNSUPPORTED;
   pm.expire_wait = take_request(g_expire_q_waits) ? 1 : 0;
-  if ((rc = launch_rc(traced("k_fwd_main", s, [&] { return launch_fwd_main(maps, pm, smem, s, sched_for(SCHED_MAIN, pm)); })))) return rc;
+  if ((rc = launch_rc(traced("k_fwd_main", s, [&] { return launch_fwd_main(maps, pm, smem, s, *sched_for(SCHED_MAIN, pm)); })))) return rc;
   if (prob && p.x3) {
     Params pl = p;
     pl.pv_sel = PV_LERP;
     const int smem2 = plan_main(pl, PV_LERP);
     if (smem2 < 0) return KINT_ERR_UNSUPPORTED;
-    if ((rc = launch_rc(traced("k_fwd_main", s, [&] { return launch_fwd_main(maps, pl, smem2, s, sched_for(SCHED_MAIN, pl)); })))) return rc;
+    if ((rc = launch_rc(traced("k_fwd_main", s, [&] { return launch_fwd_main(maps, pl, smem2, s, *sched_for(SCHED_MAIN, pl)); })))) return rc;
   }
   return KINT_OK;
 }
@@ -840,7 +743,7 @@ int kint_attn_bwd(const float* Q, const float* K, const float* V, const float* O
       pf.gate = w.tie_any;
       pf.gate_on = 0;
     }
-    if ((rc = launch_rc(traced("k_bwd_fused", s, [&] { return launch_bwd_fused(maps, pf, smem_f, s, sched_for(SCHED_FUSED, pf)); })))) return rc;
+    if ((rc = launch_rc(traced("k_bwd_fused", s, [&] { return launch_bwd_fused(maps, pf, smem_f, s, *sched_for(SCHED_FUSED, pf)); })))) return rc;
     if (!ext) return KINT_OK;
     if ((rc = launch_rc(traced("k_bwd_ext", s, [&] { return launch_bwd_ext(pf, s); })))) return rc;
     p.gate = w.tie_any;
@@ -853,19 +756,19 @@ int kint_attn_bwd(const float* Q, const float* K, const float* V, const float* O
   Params pq = p;
   const int smem_dq = plan_dq(pq);
   if (smem_dq < 0 || smem_dq > kSmemLimit) return KINT_ERR_UNSUPPORTED;
-  if ((rc = launch_rc(traced("k_bwd_dq", s, [&] { return launch_bwd_dq(maps, pq, smem_dq, s, pq.pair ? sched_for(SCHED_DQ, pq) : sched_none()); })))) return rc;
+  if ((rc = launch_rc(traced("k_bwd_dq", s, [&] { return launch_bwd_dq(maps, pq, smem_dq, s, *(pq.pair ? sched_for(SCHED_DQ, pq) : SchedStore::none())); })))) return rc;
 
   Params pk = p;
   int smem_kv = plan_dkdv(pk, DKV_BOTH);
-  if (!p.x3 && smem_kv > 0) return launch_rc(traced("k_bwd_dkdv", s, [&] { return launch_bwd_dkdv(maps, pk, smem_kv, s, sched_none()); }));
+  if (!p.x3 && smem_kv > 0) return launch_rc(traced("k_bwd_dkdv", s, [&] { return launch_bwd_dkdv(maps, pk, smem_kv, s, *SchedStore::none()); }));
   // one product per launch (3xTF32 hi/lo operands, or d = 128): dV, then dK
   smem_kv = plan_dkdv(pk, DKV_DV);
   if (smem_kv < 0) return KINT_ERR_UNSUPPORTED;
-  if ((rc = launch_rc(traced("k_bwd_dkdv", s, [&] { return launch_bwd_dkdv(maps, pk, smem_kv, s, sched_none()); })))) return rc;
+  if ((rc = launch_rc(traced("k_bwd_dkdv", s, [&] { return launch_bwd_dkdv(maps, pk, smem_kv, s, *SchedStore::none()); })))) return rc;
   Params pk2 = p;
   const int smem_kv2 = plan_dkdv(pk2, DKV_DK);
   if (smem_kv2 < 0) return KINT_ERR_UNSUPPORTED;
-  return launch_rc(traced("k_bwd_dkdv", s, [&] { return launch_bwd_dkdv(maps, pk2, smem_kv2, s, sched_for(SCHED_DK, pk2)); }));
+  return launch_rc(traced("k_bwd_dkdv", s, [&] { return launch_bwd_dkdv(maps, pk2, smem_kv2, s, *sched_for(SCHED_DK, pk2)); }));
 }
 
 int kint_attn_debug_bins(const float* Q, const float* K, const float* V, const kint_rowstats* st, uint8_t* bins,
@@ -903,7 +806,7 @@ int kint_attn_debug_bins(const float* Q, const float* K, const float* V, const k
   pm.debug = 1;
   pm.bins = bins;
   pm.ivals = ivals;
-  return launch_rc(traced("k_fwd_main", s, [&] { return launch_fwd_main(maps, pm, smem, s, sched_for(SCHED_MAIN, pm)); }));
+  return launch_rc(traced("k_fwd_main", s, [&] { return launch_fwd_main(maps, pm, smem, s, *sched_for(SCHED_MAIN, pm)); }));
 }
 
 int kint_attn_probe(const float* Q, const float* K, const kint_rowstats* st, float* probe, int B, int H, int T,
@@ -945,7 +848,7 @@ int kint_attn_probe(const float* Q, const float* K, const kint_rowstats* st, flo
   // pass 1 (row extrema), then the probe's two sweeps
   Params ps = p;
   const int smem_s = plan_stats(ps);
-  if ((rc = launch_rc(traced("k_fwd_stats", s, [&] { return launch_fwd_stats(maps, ps, smem_s, s, sched_for(SCHED_STATS, ps)); })))) return rc;
+  if ((rc = launch_rc(traced("k_fwd_stats", s, [&] { return launch_fwd_stats(maps, ps, smem_s, s, *sched_for(SCHED_STATS, ps)); })))) return rc;
   Params pp = p;
   const int smem_p = plan_probe(pp);
   if (smem_p < 0 || smem_p > kSmemLimit) return KINT_ERR_UNSUPPORTED;

@@ -4,6 +4,8 @@
 #include <cstdint>
 #include <cuda.h>
 
+#include "kint_sched.h"
+
 namespace kint {
 
 enum Calib : int { CAL_MINMAX = 0, CAL_FWM = 1, CAL_SOFTMAX = 2, CAL_FWMR = 3, CAL_EXP8 = 4, CAL_EXPB = 5 };
@@ -37,17 +39,6 @@ struct Maps {
   CUtensorMap kt, kt_lo, vt, vt_lo, qt, qt_lo, dot, dot_lo;  // transposed
   CUtensorMap out, out_lerp, dq, dk, dv;  // outputs (natural, box 32 x 64 rows) for TMA stores
   CUtensorMap dq16, dk32, dv32;  // single-pass backward: 16-column boxes (64-byte swizzle), dQ reduces of 16 rows, dK / dV stores of 32
-};
-
-// Static item schedule of a persistent kernel, computed on the host (longest processing
-// time first over the launch's CTAs): CTA c takes the items idx[off[c]] .. idx[off[c+1] - 1]
-// in that order.  n == 0: no schedule, the snake order (snake_item) instead.  2048 items: 16 heads
-// of 16384 rows.
-constexpr int SCHED_MAX_CTAS = 304, SCHED_MAX_ITEMS = 2048;
-struct Sched {
-  int n;
-  uint16_t off[SCHED_MAX_CTAS + 1];
-  uint16_t idx[SCHED_MAX_ITEMS];
 };
 
 struct Params {

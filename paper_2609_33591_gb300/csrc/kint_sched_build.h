@@ -120,11 +120,15 @@ inline void build_sched(const SchedKey& k, Sched& out) {
   for_items(best_hg, [&](int i, int b, int h) { out.idx[pos[best[i]]++] = (uint16_t)(b * k.BH + h); });
 }
 
-// The schedules built so far.  A schedule is built outside the lock (two threads may build the
-// same one; the first to finish is kept), so that a call never waits for another's build.
+// The schedules built so far, kMax of them: a further one takes the place of the oldest (a call that
+// holds that one keeps it alive), so how a shape runs does not depend on the shapes before it.  A
+// call at d = 128 or under 3xTF32 uses four, so the store serves 256 such shapes without building
+// again, in 5 MB.  A schedule is built outside the lock (two threads may build the same one; the
+// first to finish is kept), so that a call never waits for another's build.
 class SchedStore {
  public:
   using Ptr = std::shared_ptr<const Sched>;
+  static constexpr size_t kMax = 1024;
   static Ptr none() {
     static const Sched z{};
     return Ptr(std::shared_ptr<void>(), &z);
@@ -138,21 +142,34 @@ class SchedStore {
         std::lock_guard<std::mutex> lk(mu_);
         const auto it = map_.find(k);
         if (it != map_.end()) return it->second;
-        if (map_.size() >= kMax) return none();  // entries are never released: bound their number
       }
       auto s = std::make_shared<Sched>();
       build_sched(k, *s);
       std::lock_guard<std::mutex> lk(mu_);
+      const auto it = map_.find(k);
+      if (it != map_.end()) return it->second;
+      if (age_.size() < kMax) {
+        age_.push_back(k);
+      } else {
+        map_.erase(age_[oldest_]);
+        age_[oldest_] = k;
+        oldest_ = (oldest_ + 1) % kMax;
+      }
       return map_.emplace(k, std::move(s)).first->second;
     } catch (...) {
       return none();
     }
   }
+  size_t size() {
+    std::lock_guard<std::mutex> lk(mu_);
+    return map_.size();
+  }
 
  private:
-  static constexpr size_t kMax = 256;
   std::mutex mu_;
   std::map<SchedKey, Ptr> map_;
+  std::vector<SchedKey> age_;  // the stored keys, in a ring from the oldest on once it is full
+  size_t oldest_ = 0;
 };
 
 }  // namespace kint

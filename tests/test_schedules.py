@@ -29,6 +29,8 @@ static void print(const Sched& s, int ngrid) {
 
 // build kind ngrid BH T d parts: the group size wanted, the best of ten build times, the schedule;
 // threads BH ngrid: eight threads ask for the schedules of 60 lengths, and each must be the built one
+// full n: the number of n shapes, asked for in turn, that got their schedule, that of the first ones
+// asked for again, whether one held from before is intact, and how many are stored
 int main(int argc, char** argv) {
   auto arg = [&](int i) { return std::atoi(argv[i]); };
   auto key = [](int kind, int ngrid, int BH, int T, int d, int parts) {
@@ -50,6 +52,23 @@ int main(int argc, char** argv) {
     return 0;
   }
   static SchedStore store;
+  if (argv[1][0] == 'f') {
+    const int n = arg(2);
+    int got = 0, again = 0;
+    auto right = [&](int i) {
+      const SchedKey k = key(SCHED_STATS, 152, 153 + i, 128, 64, 1);
+      static Sched s;
+      build_sched(k, s);
+      return std::memcmp(&s, store.get(k).get(), sizeof(s)) == 0;
+    };
+    const SchedStore::Ptr held = store.get(key(SCHED_STATS, 152, 153, 128, 64, 1));
+    const Sched copy = *held;
+    for (int i = 0; i < n; ++i) got += right(i);
+    for (int i = 0; i < 100; ++i) again += right(i);
+    std::printf("%d %d %d %d %d\n", got, again, std::memcmp(&copy, held.get(), sizeof(copy)) == 0 ? 1 : 0,
+                (int)store.size(), (int)SchedStore::kMax);
+    return 0;
+  }
   std::vector<std::thread> ts;
   std::atomic<int> bad{0};
   for (int t = 0; t < 8; ++t)
@@ -153,3 +172,9 @@ def test_build_time(driver):
 
 def test_store_from_several_threads(driver):
     assert driver("threads", 33, 152)[0] == "0"
+
+
+def test_store_replaces_its_oldest_entry(driver):
+    """More shapes than the store holds: each still gets its schedule, in a bounded store."""
+    got, again, held, size, limit = map(int, driver("full", 1500)[0].split())
+    assert (got, again, held) == (1500, 100, 1) and size == limit < 1500

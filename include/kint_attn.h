@@ -258,11 +258,11 @@ void kint_set_wait_timeout_ns(unsigned long long ns);
 void kint_test_expire_next_wait(int count);
 
 /*
- * The same for pass 2 of the next `count` calls of kint_attn_fwd and kint_attn_fwd_noalloc: the
- * compute warps' first wait for the Q tile runs out in three of every four warps (one of two
- * where two CTAs share an SM) and succeeds in the others, so the warps of a CTA disagree about
- * it.  Status bit 1 (TMA wait timed out) is set, every warp leaves within a few limits, and the
- * context stays usable.  At d = 128 with O_lerp no compute warp waits for Q: no effect there.
+ * The same for pass 2 of the next `count` calls of kint_attn_fwd and kint_attn_fwd_noalloc: once
+ * the compute warps have their first Q tile, three of every four (one of two where two CTAs share
+ * an SM) wait on a barrier that nothing completes, so the warps of a CTA disagree about an expired
+ * wait.  Status bit 1 (TMA wait timed out) is set, every warp leaves within a few limits, and the
+ * context stays usable.  TF32 with FWM Nearest (Weight-STE) or MinMax LERP; no effect elsewhere.
  */
 void kint_test_expire_next_q_wait(int count);
 

@@ -241,7 +241,9 @@ __device__ __forceinline__ bool main_issue_s(const Params& p, RingPos stg, int b
   return true;
 }
 
-template <int CAL, int REC, int MODE, bool X3, int NG>
+// HOOK: the instantiations of the test hook of the first Q wait (kint_test_expire_next_q_wait).  As a
+// run-time switch it cost every launch plan up to 0.9 us of 157.
+template <int CAL, int REC, int MODE, bool X3, int NG, bool HOOK>
 __global__ void __launch_bounds__(MainT<NG>::NTHR, MainT<NG>::CTAS) k_fwd_main(const __grid_constant__ Maps maps, const Params p,
                                                       const __grid_constant__ Sched sch) {
   uint8_t* sm = smem_base();
@@ -260,7 +262,7 @@ __global__ void __launch_bounds__(MainT<NG>::NTHR, MainT<NG>::CTAS) k_fwd_main(c
   uint64_t* bar_s = bars;              // [4] S_b computed
   uint64_t* bar_pready = bars + 4;     // [4] the weights of buffer b stored by the tile's eight warps
   uint64_t* bar_pv = bars + 8;         // [NG] the product that read the group's A2 buffer complete
-  uint64_t* bar_never = bars + 11;     // (one of the four kept for bar_pv; NG <= 2) nothing arrives: test hook
+  [[maybe_unused]] uint64_t* bar_never = bars + 11;  // (of the four kept for bar_pv; NG <= 2) nothing arrives
   uint64_t* bar_q = bars + 12;         // Q of the item landed in smem
   uint64_t* bar_qfree = bars + 13;     // smem Q may be reloaded (q_tmem: Q copied into TMEM; else last S complete)
   uint64_t* bar_done = bars + 14;      // every product of the item complete
@@ -580,11 +582,10 @@ __global__ void __launch_bounds__(MainT<NG>::NTHR, MainT<NG>::CTAS) k_fwd_main(c
       M_ = i < p.T ? p.row_max[rw] : 0.0f;
       m_ = (CAL == CAL_MINMAX && i < p.T) ? p.row_min[rw] : 0.0f;
     };
-    // The k-th item's Q rows from smem, once `bar` (bar_q) says that they landed, into TMEM (each
-    // thread its share of its row's columns), handed to the MMA warp and the K producer through
-    // bar_qfree.
-    auto q_to_tmem = [&](int k, uint64_t* bar) -> bool {
-      const bool ok = mbar_wait_warp(bar, k & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA);
+    // The k-th item's Q rows from smem into TMEM (each thread its share of its row's columns),
+    // handed to the MMA warp and the K producer through bar_qfree.
+    auto q_to_tmem = [&](int k) -> bool {
+      const bool ok = mbar_wait(bar_q, k & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA);
       if (ok) {
 #pragma unroll 1
         for (int c = cq * (D / NQ); c < (cq + 1) * (D / NQ); c += 16) {
@@ -601,8 +602,10 @@ __global__ void __launch_bounds__(MainT<NG>::NTHR, MainT<NG>::CTAS) k_fwd_main(c
     int item = sched_item(sch, 0);
     if (item < p.nitems) {
       load_extrema(item, qb, bh, M, m);
-      // (the test hook lets the wait run out in every warp but the first of each quarter)
-      if (q_tmem) failed = !q_to_tmem(0, p.expire_wait && cq > 0 ? bar_never : bar_q);
+      if (q_tmem) failed = !q_to_tmem(0);
+      if constexpr (HOOK) {  // every warp but the first of each quarter waits on
+        if (q_tmem && cq > 0) failed = !mbar_wait(bar_never, 0, p.wait_ns, p.status, DEV_ERR_TIMEOUT_TMA);
+      }
     }
     // Tables addressed by the float bits 0x4B000000 + index of the floored position.
     // FWM: one half-bin table of 24-byte line entries, q in [-2, 2K] at sm_table + 24 (q + 2)
@@ -730,7 +733,7 @@ __global__ void __launch_bounds__(MainT<NG>::NTHR, MainT<NG>::CTAS) k_fwd_main(c
       if (!failed) failed = !mbar_wait(bar_done, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_MMA);
       tc_fence_after();
       // every S of the item is complete: the next item's Q goes in under the epilogue
-      if (!failed && q_tmem && next < p.nitems) failed = !q_to_tmem(n + 1, bar_q);
+      if (!failed && q_tmem && next < p.nitems) failed = !q_to_tmem(n + 1);
       if (!failed) failed = !mbar_wait(bar_w, n & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_SYNC);
       if (!failed && !p.debug && use > 0)  // the staging area's previous stores have read it
         failed = !mbar_wait(bar_stfree, (use - 1) & 1, p.wait_ns, p.status, DEV_ERR_TIMEOUT_SYNC);
@@ -793,15 +796,22 @@ __global__ void __launch_bounds__(MainT<NG>::NTHR, MainT<NG>::CTAS) k_fwd_main(c
   if (warp == 0) tmem_dealloc(tmem, T::TMEM_COLS);
 }
 
-template <int CAL, int REC, int MODE, bool X3, int NG>
+template <int CAL, int REC, int MODE, bool X3, int NG, bool HOOK = false>
 static cudaError_t launch_main_n(const Maps& maps, const Params& p, int smem_bytes, cudaStream_t s, const Sched& sch) {
-  auto kern = k_fwd_main<CAL, REC, MODE, X3, NG>;
+  auto kern = k_fwd_main<CAL, REC, MODE, X3, NG, HOOK>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
   if (e != cudaSuccess) return e;
   return launch_pdl(kern, dim3((unsigned)p.ngrid), dim3(MainT<NG>::NTHR), smem_bytes, s, maps, p, sch);
 }
 template <int CAL, int REC, int MODE, bool X3>
 static cudaError_t launch_main_t(const Maps& maps, const Params& p, int smem_bytes, cudaStream_t s, const Sched& sch) {
+  // one grid with a shared table and one with a table per row (a barrier at the item's start)
+  constexpr bool hooked = !X3 && MODE == 0 && ((CAL == CAL_FWM && REC == REC_NEAREST) || (CAL == CAL_MINMAX && REC == REC_LERP));
+  if constexpr (hooked) {
+    if (p.expire_wait)
+      return p.main_groups == 1 ? launch_main_n<CAL, REC, MODE, X3, 1, true>(maps, p, smem_bytes, s, sch)
+                                : launch_main_n<CAL, REC, MODE, X3, 2, true>(maps, p, smem_bytes, s, sch);
+  }
   if constexpr (!X3 && MODE == 0) {
     if (p.main_groups == 1) return launch_main_n<CAL, REC, MODE, X3, 1>(maps, p, smem_bytes, s, sch);
   }

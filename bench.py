@@ -149,6 +149,29 @@ def reduce_max(ms: float, world: int, device) -> float:
     return float(t.item())
 
 
+def time_steps(n: int, fn, warmup: int, world: int, device) -> float:
+    """Milliseconds per step of n steps fn(0), fn(1), ... on the device, after `warmup` untimed ones (the
+    first call of an operator and shape loads its kernels and builds its schedules on the host)."""
+    import torch
+
+    def barrier():
+        if world > 1:
+            torch.distributed.barrier()
+
+    for i in range(warmup):
+        fn(i)
+    barrier()
+    torch.cuda.synchronize()
+    e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    e0.record()
+    for i in range(n):
+        fn(i)
+    e1.record()
+    torch.cuda.synchronize()
+    barrier()
+    return reduce_max(e0.elapsed_time(e1) / n, world, device)
+
+
 def job_value(flops_per_step: float, world: int, ms: float) -> float:
     """Whole-job throughput: the work of all ranks (replicas) over the slowest rank's time."""
     return world * flops_per_step / (ms * 1e-3) / 1e12
@@ -341,21 +364,8 @@ def run_cuda(args, world, rank, local):
         kint.forward(q, k, v, c, p, O=O, stats=st, ws=ws_f)
         kint.backward(q, k, v, O, do, st, c, p, grads=grads, ws=ws_b)
 
-    def barrier():
-        if world > 1:
-            torch.distributed.barrier()
-
-    def timed(n, fn):
-        barrier()
-        torch.cuda.synchronize()
-        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-        e0.record()
-        for i in range(n):
-            fn(i)
-        e1.record()
-        torch.cuda.synchronize()
-        barrier()
-        return reduce_max(e0.elapsed_time(e1) / n, world, dev)
+    def timed(n, fn, warmup=3):
+        return time_steps(n, fn, warmup, world, dev)
 
     for i in range(args.warmup):
         step(i)
@@ -395,7 +405,7 @@ def run_cuda(args, world, rank, local):
     sampler = ClockSampler(local)
     sampler.start()
     time.sleep(0.3)
-    ms = timed(args.steps, run_step)
+    ms = timed(args.steps, run_step, warmup=0)  # (warmed up above)
     clocks = sampler.stop()
     kint.check_status()
     launches = [per_step[0] * args.steps]
@@ -416,7 +426,7 @@ def run_cuda(args, world, rank, local):
 
     n_kt = max(3, min(args.steps, 200))
     kint.kint_set_launch_callback(on_launch)
-    timed(n_kt, step)
+    timed(n_kt, step, warmup=0)
     kint.kint_set_launch_callback(None)
     kint.check_status()
 
@@ -476,7 +486,6 @@ def run_cuda(args, world, rank, local):
         kint.forward(q, k, v, cfg, kint.PREC_3XTF32, O=O, stats=st, ws=ws_f3)
         kint.backward(q, k, v, O, do, st, cfg, kint.PREC_3XTF32, grads=grads, ws=ws_b3)
 
-    step3(0)
     ms3 = timed(n_cmp, step3)
     line["x3tf32_mode"] = {"value": job_value(flops_step, world, ms3), "unit": UNIT, "ms_per_step": ms3}
     del ws_f3, ws_b3
@@ -525,7 +534,7 @@ def run_cuda(args, world, rank, local):
 
     e2e_run(2)
     n_e2e = max(3, min(args.steps, 100))
-    ms_e2e = timed(1, lambda i: e2e_run(n_e2e)) / n_e2e
+    ms_e2e = timed(1, lambda i: e2e_run(n_e2e), warmup=0) / n_e2e
     # the same copies with no compute, each direction streaming back to back on its own
     # stream: the host link's floor for the end-to-end steps
     def copies_only(n):
@@ -542,7 +551,7 @@ def run_cuda(args, world, rank, local):
         s_c.wait_stream(s_out)
 
     copies_only(2)
-    ms_link = timed(1, lambda i: copies_only(n_e2e)) / n_e2e
+    ms_link = timed(1, lambda i: copies_only(n_e2e), warmup=0) / n_e2e
     line["e2e"] = {"value": job_value(flops_step, world, ms_e2e), "unit": UNIT,
                    "h2d_bytes_per_step": sum(t.numel() * 4 for t in pin_in),
                    "d2h_bytes_per_step": sum(t.numel() * 4 for t in pin_out), "ms_per_step": ms_e2e,
@@ -569,8 +578,6 @@ def run_cuda(args, world, rank, local):
                 kint.forward(Q2, K2, V2, c, prec, O=O2, stats=st2, ws=wf2)
                 kint.backward(Q2, K2, V2, O2, dO2, st2, c, prec, grads=g2, ws=wb2)
 
-            for i in range(3):
-                step2(i)
             n2 = 5 if T2 <= 4096 else 3
             ms2 = timed(n2, step2)
             f2 = 6 * unit_flops(B2, H2, T2, d2)
@@ -578,8 +585,6 @@ def run_cuda(args, world, rank, local):
                    "ms_per_step": ms2, "steps": n2, "warmup": 3, "tf32_peak_frac": f2 / (ms2 * 1e-3) / 1e12 / tf32_peak,
                    "l2": "inputs larger than the 129 MB L2 (one input set)"}
             if spec["softmax"]:
-                for i in range(3):
-                    step2(i, soft)
                 ms_s = timed(n2, lambda i: step2(i, soft))
                 rec["softmax_comparator"] = {"value": job_value(f2, world, ms_s), "unit": UNIT, "ms_per_step": ms_s}
             kint.check_status()

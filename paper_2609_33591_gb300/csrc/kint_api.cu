@@ -316,7 +316,7 @@ int plan_main(Params& p, int mode) {
   };
   // Two CTAs per SM, 256 TMEM columns each (two score buffers, O, Q): TF32 at d = 64 without
   // O_lerp, with more items than SMs (fewer leave each item an SM of its own, where one CTA's
-  // sixteen compute warps finish it sooner).  At B=8 H=12 T=1024 the softmax pass takes 35.6 us
+  // sixteen compute warps finish it sooner).  At B=8 H=12 T=1024 the softmax pass takes 33.7 us
   // so, 40.9 with one CTA; FWM LERP at B=4 T=1000 31.6 against 34.8.  With O_lerp the columns
   // leave one score buffer per CTA: 79 us against 66.8 with one CTA.
   if (!p.x3 && p.d == 64 && !both && p.nitems > num_sms()) {

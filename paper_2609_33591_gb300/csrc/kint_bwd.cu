@@ -8,7 +8,7 @@
 //   complete at the end of the row; it then adds c_M / n_max (and c_m / n_min)
 //   times the arg-extremum keys to dQ (Eq. full) and writes a 64-byte record of
 //   the row's constants for the second kernel.
-// k_bwd_dkdv (one CTA per 128-key block, a thread per key and column half): per
+// k_bwd_dkdv (one CTA per 128-key block, a thread per key and 16 of the columns): per
 //   64-query tile, S^T and g^T, the forward P and the full dS (extremum terms
 //   now known), and dV += P^T dO, dK += dS^T Q.
 // k_bwd_dq: compute warps 0-7; k_bwd_dkdv: 0-15.  MMA-issuing and TMA / bulk-copy producer
@@ -425,10 +425,12 @@ __global__ void __launch_bounds__(PAIR ? NTHR_DQ + 32 : NTHR_DQ, 1) k_bwd_dq(con
       }
       return r;
     };
-    // Whether the epilogue passes through the staging area: TF32 at d = 64 always, PAIR never.  For
-    // PAIR it is read from the launch parameters all the same: with that side of the epilogue
-    // compiled out, the compiler's schedule of the MinMax tile loop is worse (H=16 T=16384 d=128
-    // K=16: 3439 against 3133 us; the other instantiations within 1 %).
+    // Whether the epilogue passes through the staging area: TF32 at d = 64 always, PAIR never (every
+    // PAIR launch has p.pair set).  For PAIR it is read from the launch parameters all the same: with
+    // that side of the epilogue compiled out, the compiler's schedule of the MinMax tile loop is worse
+    // at H=16 T=16384 d=128 K=16 (3433 against 3125 us; B=4 T=2048 K=8 340 against 342, 3xTF32 B=4
+    // H=12 T=1024 101 against 107, FWM 232 against 230).  Rolled loops, a memory clobber, the operands
+    // loaded one after the other and fewer registers did not bring the 3125 back.
     const bool staged = PAIR ? p.pair == 0 : true;
     int n = 0;
     RingPos cb, cs;  // score buffer and stage of the current tile

@@ -10,9 +10,10 @@
 // exponentials keep the same maximum channel), which is complete only after every key
 // block has passed, so this pass accumulates that row sum and k_bwd_ext adds
 //   dQ_i += s (c_M / n_max) K_amax(i),   dK_amax(i) += s (c_M / n_max) Q_i
-// afterwards.  Rows with tied maxima would need the tie set, which only the scores
-// themselves give: when any row has one, the gated two-pass kernels (k_bwd_dq,
-// k_bwd_dkdv) run instead and these kernels leave at once.
+// afterwards.  Rows with tied maxima need the tie set, which only the scores themselves
+// give: the pass lists those keys for k_bwd_ext.  Only when the rows hold more tied keys
+// than the list has room for (one per row of the call) do the gated two-pass kernels
+// (k_bwd_dq, k_bwd_dkdv) run instead and these kernels leave at once.
 //
 // The partial dQ sums and the extremum scatter are fp32 additions whose order is not
 // fixed, so this path is not bit-reproducible from run to run; the two-pass path is.
@@ -154,10 +155,15 @@ __device__ __forceinline__ void rowsum_red(const float (&v)[16], float* dst, siz
 // after which each warp writes its part of the next item's K^T there; each output warp
 // has four 1 KB slices for its 16 rows x 64 columns of the dQ partial (64-byte swizzle), added
 // to dQ by TMA reduces.
-// What bounds it: shared memory.  Per tile of 64 x 128 the products read 160 KB of operands from
-// it, the TMA loads write 64 KB, and the row records (a broadcast LDS.128 per key column and
-// warp, two wavefronts), tables, dS stores and TMEM traffic take some 2500 wavefronts, of about
-// 3600 cycles.  Row sums and dQ partial by the output warps, not the compute warps (a butterfly
+// What bounds it: no single unit.  Of an SM's active cycles at B=4 H=12 T=1024 (ncu; FWM K=4
+// Prob-STE, then softmax), the load / store data stage takes 55 and 44 % (2535 and 1577 wavefronts per
+// 64 x 128 tile: row records, tables, dS, TMEM staging), the products' operand reads 28 and 36 % (1280
+// wavefronts, 160 KB), issue 47 and 41 %, the tensor pipe 33 and 43 %; the shared-memory banks are
+// 28 and 31 % busy and the two kinds of access do not conflict.  What is left is the chain of hand-offs
+// of a tile (S^T and g^T, element work, dS, then dQ, dV, dK) over two score buffers and two stages:
+// of some 3.3k cycles per tile the MMA warp waits 1.0k (softmax 0.6k) for the element work, and the
+// compute warps 0.9 to 1.3k for products, records and the dS buffer.
+// Row sums and dQ partial by the output warps, not the compute warps (a butterfly
 // over the keys in registers, 1 KB per warp): B=8 H=12 T=1024 FWM K=4 113 -> 111 us, softmax
 // 102 -> 97, B=4 H=12 T=1000 K=16 detached LERP 61.3 -> 59.3.  Issuing dV, dK from a second warp, dV, dK
 // before dQ, and bringing the next tiles into L2 ahead of their loads gained nothing.

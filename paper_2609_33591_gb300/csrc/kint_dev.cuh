@@ -489,8 +489,8 @@ __device__ __forceinline__ uint32_t lane_addr(uint32_t tmem_base, int col) {
 // Columns [c0, c0 + n) of row `row` of X (d fp32 per row) into the calling
 // thread's TMEM lane at columns [col + c0, col + c0 + n); with `split`, the tf32 hi
 // part there and the lo part d columns further.  All global loads are issued
-// before the first TMEM store.  Rows >= T load zeros.  n is 32 or 64; whole
-// warps must call this with the same c0, n.
+// before the first TMEM store.  Rows >= T load zeros.  Whole warps must call this with
+// the same c0 (n is 16 in the dV launch, its only caller).
 template <int N>
 __device__ __forceinline__ void row_to_tmem_part(uint32_t tmem_base, int col, const float* X, int row, int T, int d,
                                                  int c0, bool split) {

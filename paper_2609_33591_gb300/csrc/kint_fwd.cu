@@ -191,7 +191,7 @@ cudaError_t launch_prep(const PrepJobs& jobs, int BH, int T, int Tp, int d, bool
 // improves in most chunks, and finding the equal keys there took about five instructions per
 // key against the select's one (pass 1 at B=8 H=12 T=1024 d=64: 31.6 -> 27.4 us).  A chunk that
 // only ties with the running maximum (rare) counts its equal keys at once.  Masked keys
-// (j > i) are -inf.  SIGN = -1 takes the minimum side, on negated scores.  RAW: the scale is a
+// (j > i) are -inf.  The minimum side runs on negated scores.  RAW: the scale is a
 // power of two (d = 64: 2^-3), so the dot products are compared unscaled (exact scaling: only
 // scores below 2^-123 in magnitude, subnormal after scaling, could merge), and the extremum is
 // scaled once when the row is stored.

@@ -205,8 +205,8 @@ __device__ void fwd_debug_codes(const Params& p, const float (&v)[W], int j0, in
 // lookups and MMA operands share, and the hand-offs between them; at d = 128 and under
 // 3xTF32 the tensor pipe (48-49% active) and its operand loads.  Measured on GB300 (kernel
 // alone, cold L2), against one 128-key stage and score buffer where two did not fit and
-// eight compute warps: B=8 H=12 T=1024 d=64 FWM K=4 Prob-STE 67.8 -> 66.8 us, softmax 46.6 ->
-// 35.6, 3xTF32 144 -> 81; B=4 H=16 T=2048 d=128 FWM Weight-STE 254 -> 134; H=16 T=16384 d=128
+// eight compute warps: B=8 H=12 T=1024 d=64 FWM K=4 Prob-STE 67.8 -> 66.5 us (within a step 67.1 and
+// 67.5: nothing gained there), softmax 46.6 -> 33.7, 3xTF32 144 -> 80; B=4 H=16 T=2048 d=128 FWM Weight-STE 254 -> 134; H=16 T=16384 d=128
 // MinMax K=16 LERP 3417 -> 1516.
 // ---------------------------------------------------------------------------
 // Wait for the K tile in slot `stg`, S_b = Q K^T into score buffer b, commit to bar_s[b]

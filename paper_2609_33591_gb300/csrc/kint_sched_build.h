@@ -25,6 +25,9 @@ enum SchedKind { SCHED_STATS = 0, SCHED_MAIN = 1, SCHED_FUSED = 2, SCHED_DQ = 3,
 // same within 2 %.  B=4 H=16 T=2048 d=128 (200 MB of tiles in dQ and dK): pass 1 78 -> 75 us,
 // pass 2 136 -> 124, dQ 248 -> 232, dK 238 -> 231; B=8 H=12 T=1024 3xTF32 dQ 147 -> 132,
 // dK 131 -> 127.  Not the single-pass backward, where groups of 16 to 48 of 96 heads gave nothing.
+// A call somewhat above the limit is split too, although one group balances the CTAs better: softmax
+// at B=8 H=12 T=1024 (50 MB of tiles in pass 2, longest CTA 1.14 of the mean against 1.10) took 186.1 us
+// forward and backward in two groups, 186.9 in one.
 constexpr double kGroupBytes = 48e6;
 
 // What a schedule depends on.  nqt: 64-row query tiles (kinds whose items are key blocks; else 0);

@@ -41,8 +41,8 @@ TF32_PER_BF16 = 1.1 / 2.25  # nominal dense TF32 : BF16 tensor rate of GB300 (1.
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) of each kernel from
 # one ncu capture of this workload (profiles/traffic_gpt2_tf32.md), valid only for the
 # kernel sources they were taken from.
-TRAFFIC = {"src": "b645bd08ca50e2c7", "k_prep": 65128979, "k_fwd_stats": 50402163, "k_fwd_main": 86756531,
-           "k_bwd_fused": 382449818, "k_bwd_ext": 73676275}
+TRAFFIC = {"src": "5e715fcf265fab95", "k_prep": 65164518, "k_fwd_stats": 50402752, "k_fwd_main": 86997785,
+           "k_bwd_fused": 384468876, "k_bwd_ext": 73674636}
 
 
 def kernel_source_digest() -> str:
